@@ -177,7 +177,11 @@ size_t stage_scratch_bytes(rsv_operator op, int kg) {
   return 0;
 }
 
-int march_tile_kernels(rsv_operator op, int steps, int kg) {
+int march_tile_kernels(rsv_operator op, int steps, int kg, bool step_form) {
+  if (step_form) {   // 2-D FP32: one launch per step; 3-D: two; FP64: one per stage
+    if (op->kind == RSV_OP_ADR2D) return (op->prec == RSV_PREC_FP32 ? steps : 4 * steps) + 1;
+    return 2 * steps + 1;
+  }
   switch (op->kind) {
     case RSV_OP_GL1D:
       return 1;
@@ -207,9 +211,64 @@ rsv_status on_frequencies(rsv_operator op) {
   return RSV_OK;
 }
 
+// ---------------------------------------------------------------------------
+// Step form (step2d.cu): forcing transformed once per march, one synthesis time per step
+// ---------------------------------------------------------------------------
+bool step_form_taken(rsv_operator op, int k) {
+  if (op->scheme != RSV_SCHEME_RK4 || k > 65535) return false;
+  if (op->kind == RSV_OP_ADR2D) {
+    const char* e = getenv("RSV_STENCIL_FUSED");
+    if (e != nullptr && e[0] == '1') return false;
+    if (op->prec == RSV_PREC_FP32 && !adr2d_pairs_enabled()) return false;
+    return op->ny <= (1 << 17) && step_points(op) < ((int64_t)1 << 31);
+  }
+  if (op->kind == RSV_OP_ADV3D)
+    return op->prec == RSV_PREC_FP32 && !op->bf16_state && adv3d_pairs_enabled() &&
+           step_points(op) < ((int64_t)1 << 31);
+  return false;
+}
+
+int64_t step_points(rsv_operator op) {
+  if (op->kind == RSV_OP_ADR2D || op->kind == RSV_OP_ADV3D) return op->n / op->nx * ((op->nx + 3) / 4 * 4);
+  return op->n;
+}
+
+// A second state buffer and one stage buffer.
+size_t step_scratch_bytes(rsv_operator op, int kg) {
+  return 2 * (size_t)kg * step_points(op) * (op->prec == RSV_PREC_FP64 ? 8 : 4);
+}
+
+// The temporary of the coefficient transform holds as many frequencies as 64 MB take (at least one),
+// so that it stays in L2 between the transform's passes.
+size_t step_coef_bytes(rsv_operator op, int kg, size_t* tmp) {
+  const size_t row = (size_t)kg * step_points(op) * 2 * (op->prec == RSV_PREC_FP64 ? 8 : 4);
+  const size_t nf = std::min<size_t>((size_t)op->n_omega, std::max<size_t>(1, ((size_t)64 << 20) / row));
+  if (tmp) *tmp = nf * row;
+  return (size_t)op->n_omega * row;
+}
+
 template <typename R>
-rsv_status prepare_coefficients(rsv_operator op, const void* fhat, int64_t f_stride, int kg, bool adjoint,
+rsv_status step_coefficients(rsv_operator op, const void* fhat, int64_t f_stride, int kg, bool adjoint) {
+  size_t tmp = 0;
+  const size_t bytes = step_coef_bytes(op, kg, &tmp);
+  rsv_status s = ensure(op->ws_coef, bytes);
+  if (s == RSV_OK) s = ensure(op->ws_coef2, tmp);
+  if (s != RSV_OK) return s;
+  const cudaError_t e = step_coefs_grid<R>(op, fhat, f_stride, kg, adjoint, op->ws_coef.ptr, op->ws_coef2.ptr,
+                                           (int64_t)(tmp / (bytes / op->n_omega)));
+  return e == cudaSuccess ? RSV_OK : cuda_fail(e, "forcing transform");
+}
+
+template <typename R>
+rsv_status prepare_coefficients(rsv_operator op, const void* fhat, int64_t f_stride, int kg, bool adjoint, bool step_form,
                                 const void** coef, int64_t* coef_stride, int* synth_stride) {
+  if (step_form) {
+    rsv_status s = step_coefficients<R>(op, fhat, f_stride, kg, adjoint);
+    *coef = op->ws_coef.ptr;
+    *coef_stride = (int64_t)kg * step_points(op);
+    *synth_stride = 2;
+    return s;
+  }
   if (op->kind != RSV_OP_DENSE) {
     *coef = fhat;
     *coef_stride = f_stride;
@@ -340,11 +399,11 @@ cudaError_t probe_initial_state(rsv_operator op, uint64_t seed) {
   return cudaGetLastError();
 }
 
-// Squared 2-norm of each of the kg vectors of the march state after step n_end
+// Squared 2-norm of each of the kg vectors (of `points` points each) of the march state after step n_end
 // (the dense path keeps two step-parity copies of the state).
-cudaError_t state_sq_norms(rsv_operator op, int kg, int64_t n_end, double* d_out) {
+cudaError_t state_sq_norms(rsv_operator op, int kg, int64_t n_end, int64_t points, double* d_out) {
   const size_t elem = op->prec == RSV_PREC_FP64 ? 8 : 4;
-  const int64_t vals = (op->real_state ? 1 : 2) * op->n;
+  const int64_t vals = (op->real_state ? 1 : 2) * points;
   const char* st = static_cast<const char*>(op->ws_state.ptr);
   if (op->kind == RSV_OP_DENSE) st += (size_t)(n_end & 1) * (size_t)kg * vals * elem;
   cudaError_t e = cudaMemsetAsync(d_out, 0, sizeof(double) * kg, op->stream);
@@ -517,6 +576,12 @@ static cudaError_t gl1d_build_packs(rsv_operator op, int kg) {
 template <typename R>
 static cudaError_t march_tile_direct(rsv_operator op, const MarchTile& t, void* state, const void* F, void* Y,
                                      double* norms) {
+  if (t.step_form) {
+    if (op->kind == RSV_OP_ADR2D) return step_march_2d<R>(op, t, state, F, Y);
+    if constexpr (sizeof(R) == 4)
+      if (op->kind == RSV_OP_ADV3D) return step_march_3d(op, t, state, F, Y);
+    return cudaErrorNotSupported;
+  }
   switch (op->kind) {
     case RSV_OP_GL1D: {
       Gl1dTile g = gl1d_geom(op, t.adjoint, t.kg);
@@ -592,7 +657,7 @@ cudaError_t march_tile(rsv_operator op, const MarchTile& t, void* state, const v
   rel.n_forced = F != nullptr ? std::max<int64_t>(0, std::min<int64_t>(t.steps, t.n_forced - t.n0)) : 0;
   const void* Fk = rel.n_forced > 0 ? F : nullptr;
   TileGraphKey key{sizeof(R), rel.steps, (int)rel.n_forced, Y != nullptr ? rel.y_first : -1, rel.kg,
-                   rel.adjoint, state, Fk, Y, norms};
+                   rel.adjoint, rel.step_form, state, Fk, Y, norms};
   TileGraph* hit = nullptr;
   for (TileGraph& g : op->tile_graphs)
     if (g.key == key) hit = &g;
@@ -652,9 +717,9 @@ cudaError_t apply_op(rsv_operator op, const void* x, int k, bool adjoint, void* 
 
 template cudaError_t march_tile<double>(rsv_operator, const MarchTile&, void*, const void*, void*, double*);
 template cudaError_t march_tile<float>(rsv_operator, const MarchTile&, void*, const void*, void*, double*);
-template rsv_status prepare_coefficients<double>(rsv_operator, const void*, int64_t, int, bool, const void**,
+template rsv_status prepare_coefficients<double>(rsv_operator, const void*, int64_t, int, bool, bool, const void**,
                                                  int64_t*, int*);
-template rsv_status prepare_coefficients<float>(rsv_operator, const void*, int64_t, int, bool, const void**,
+template rsv_status prepare_coefficients<float>(rsv_operator, const void*, int64_t, int, bool, bool, const void**,
                                                 int64_t*, int*);
 template cudaError_t apply_op<double>(rsv_operator, const void*, int, bool, void*);
 template cudaError_t apply_op<float>(rsv_operator, const void*, int, bool, void*);

@@ -259,14 +259,23 @@ extern "C" rsv_status rsv_describe(rsv_operator op, char* buf, int32_t buflen) {
     const char* e = getenv("RSV_STENCIL3D_STAGED");
     const bool pairs = !(e != nullptr && e[0] == '1') && !op->bf16_state && op->nx % 4 == 0 &&
                        op->n < ((int64_t)1 << 31);
-    path = pairs ? "cuda-core 3-D stage-pair kernels" : (op->bf16_state ? "cuda-core stages, bf16 state" : "cuda-core stages");
+    path = step_form_taken(op, 1) ? (pairs ? "cuda-core 3-D half-step kernels (sampled forcing: 3-D stage-pair kernels)"
+                                           : "cuda-core 3-D half-step kernels (sampled forcing: stages)")
+           : pairs              ? "cuda-core 3-D stage-pair kernels"
+           : op->bf16_state     ? "cuda-core stages, bf16 state"
+                                : "cuda-core stages";
   }
   if (op->kind == RSV_OP_ADR2D) {
     const char* e = getenv("RSV_STENCIL_FUSED");
     if (e != nullptr && e[0] == '1')
       path = "cuda-core whole-step kernel";
-    else if (op->prec == RSV_PREC_FP32 && adr2d_pairs_enabled() && op->nx % 4 == 0 && op->n < ((int64_t)1 << 31))
-      path = "cuda-core 2-D stage-pair kernels";
+    else if (op->prec == RSV_PREC_FP64)
+      path = step_form_taken(op, 1) ? "cuda-core step-form stages" : "cuda-core stages";
+    else if (adr2d_pairs_enabled() && op->nx % 4 == 0 && op->n < ((int64_t)1 << 31))
+      path = step_form_taken(op, 1) ? "cuda-core 2-D step kernel (sampled forcing: 2-D stage-pair kernels)"
+                                    : "cuda-core 2-D stage-pair kernels";
+    else if (step_form_taken(op, 1))
+      path = "cuda-core 2-D step kernel (sampled forcing: stages)";
   }
   if (op->kind == RSV_OP_DENSE) {
     if (op->prec == RSV_PREC_FP32 && op->tc_tiles[0] && !op->tc_disabled)
@@ -574,6 +583,10 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
   if (st != RSV_OK) return st;
   const int64_t n = op->n;
   const size_t se = state_elem_bytes(op);
+  const bool sf = step_form_taken(op, k);
+  const int64_t np = sf ? step_points(op) : n;     // points per vector of the march's tiles
+  auto scratch_bytes = [&](int kg_) { return sf ? step_scratch_bytes(op, kg_) : stage_scratch_bytes(op, kg_); };
+  const bool acc_in_out = op->prec == RSV_PREC_FP64 && trial == nullptr && np == n;
   // Tile length S and vector-group size kg: the requested / default tile and all k vectors, shrunk
   // (kg halved, then S down to 16) until the march workspace fits in 90% of the device memory not
   // held by others.
@@ -595,9 +608,14 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
                         op->ws_coef.bytes + op->ws_coef2.bytes;
     const double budget = 0.9 * (double)(free_b + held);
     auto need = [&](int s_, int kg_) {
-      const double rows_ = (double)kg_ * n;
-      double b = rows_ * se + (double)stage_scratch_bytes(op, kg_) + (2.0 * s_ + 1) * rows_ * se + s_ * rows_ * se;
-      if (op->prec != RSV_PREC_FP64) b += (double)op->n_omega * rows_ * sizeof(cpx<double>);
+      const double rows_ = (double)kg_ * np;
+      double b = rows_ * se + (double)scratch_bytes(kg_) + (sf ? s_ : 2.0 * s_ + 1) * rows_ * se + s_ * rows_ * se;
+      if (!acc_in_out) b += (double)op->n_omega * rows_ * sizeof(cpx<double>);
+      if (sf) {
+        size_t tmp = 0;
+        b += (double)step_coef_bytes(op, kg_, &tmp);
+        b += (double)tmp;
+      }
       if (s_in) b += (double)op->n_omega * rows_ * coef_bytes(op);
       if (op->kind == RSV_OP_DENSE) b += 2.0 * op->n_omega * rows_ * 2 * sizeof(R);
       if (host_in) b += 2.0 * op->n_omega * rows_ * coef_bytes(op);   // staging buffers
@@ -617,12 +635,11 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
   cudaError_t e;
   op->last_tile = S;
   op->last_group = kg;
-  const int64_t rows_max = (int64_t)kg * n;
-  if ((st = ensure(op->ws_state, rows_max * se + stage_scratch_bytes(op, kg))) != RSV_OK) return st;
-  if ((st = ensure(op->ws_ftile, (size_t)(2 * S + 1) * rows_max * se)) != RSV_OK) return st;
+  const int64_t rows_max = (int64_t)kg * np;
+  if ((st = ensure(op->ws_state, rows_max * se + scratch_bytes(kg))) != RSV_OK) return st;
+  if ((st = ensure(op->ws_ftile, (size_t)(sf ? S : 2 * S + 1) * rows_max * se)) != RSV_OK) return st;
   if ((st = ensure(op->ws_ysnap, (size_t)S * rows_max * se)) != RSV_OK) return st;
   if ((st = ensure(op->ws_norm, (size_t)kg * op->n_inst * sizeof(double))) != RSV_OK) return st;
-  const bool acc_in_out = (op->prec == RSV_PREC_FP64) && trial == nullptr;
   if (!acc_in_out && (st = ensure(op->ws_acc, (size_t)op->n_omega * rows_max * sizeof(cpx<double>))) != RSV_OK)
     return st;
   if ((e = cudaMemsetAsync(op->d_flag, 0, sizeof(int), stream)) != cudaSuccess) return cuda_fail(e, "flag reset");
@@ -679,7 +696,7 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
   if (host_in && (e = stage_copy(0)) != cudaSuccess) return cuda_fail(e, "staging copy");
   for (int v0 = 0; v0 < (trial ? std::min(kg, k) : k); v0 += kg) {
     const int kv = std::min(kg, k - v0);
-    const int64_t rows = (int64_t)kv * n;
+    const int64_t rows = (int64_t)kv * np;
     cpx<double>* acc;
     int64_t acc_stride;
     if (acc_in_out) {
@@ -692,7 +709,7 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
       acc_stride = rows;
       e = cudaMemsetAsync(acc, 0, (size_t)op->n_omega * rows * sizeof(cpx<double>), stream);
     }
-    if (e == cudaSuccess) e = cudaMemsetAsync(op->ws_state.ptr, 0, rows * se + stage_scratch_bytes(op, kv), stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(op->ws_state.ptr, 0, rows * se + scratch_bytes(kv), stream);
     if (e != cudaSuccess) return cuda_fail(e, "march reset");
     TileGeom g;
     g.rows = rows;
@@ -709,19 +726,20 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
       if (v0 + kg < k && (e = stage_copy(gi + 1)) != cudaSuccess) return cuda_fail(e, "staging copy");
       if ((e = cudaStreamWaitEvent(stream, op->ev_copied[gi & 1], 0)) != cudaSuccess) return cuda_fail(e, "staging wait");
       gin = op->ws_stage[gi & 1].ptr;
-      gin_stride = rows;
+      gin_stride = (int64_t)kv * n;
     }
     if (s_in) {   // the group's coefficients times the input scaling (B, or C W_y for the adjoint)
-      if ((st = ensure(op->ws_scaled, (size_t)op->n_omega * rows * ce)) != RSV_OK) return st;
+      const int64_t urows = (int64_t)kv * n;
+      if ((st = ensure(op->ws_scaled, (size_t)op->n_omega * urows * ce)) != RSV_OK) return st;
       ProfScope ps(op, PROF_GLUE);
-      e = launch_scale_block<R>(gin, gin_stride, op->ws_scaled.ptr, rows, op->n_omega, rows, n, s_in, stream);
+      e = launch_scale_block<R>(gin, gin_stride, op->ws_scaled.ptr, urows, op->n_omega, urows, n, s_in, stream);
       if (e != cudaSuccess) return cuda_fail(e, "input scaling");
       gin = op->ws_scaled.ptr;
-      gin_stride = rows;
+      gin_stride = urows;
     }
     {
-      ProfScope ps(op, PROF_GLUE, op->kind == RSV_OP_DENSE ? (kv == k ? 3 : 2 * op->n_omega + 1) : 0);
-      st = prepare_coefficients<R>(op, gin, gin_stride, kv, adjoint, &fh, &g.coef_stride, &synth_stride);
+      ProfScope ps(op, PROF_GLUE, op->kind == RSV_OP_DENSE ? (kv == k ? 3 : 2 * op->n_omega + 1) : sf ? 3 : 0);
+      st = prepare_coefficients<R>(op, gin, gin_stride, kv, adjoint, sf, &fh, &g.coef_stride, &synth_stride);
     }
     if (st != RSV_OK) return st;
     g.tau_stride = synth_stride;
@@ -755,8 +773,9 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
       mt.y_first = y_first;
       mt.kg = kv;
       mt.adjoint = adjoint;
+      mt.step_form = sf;
       {
-        ProfScope ps(op, PROF_MARCH, march_tile_kernels(op, g.steps, kv));
+        ProfScope ps(op, PROF_MARCH, march_tile_kernels(op, g.steps, kv, sf));
         e = march_tile<R>(op, mt, op->ws_state.ptr, forced ? op->ws_ftile.ptr : nullptr,
                           analysed ? op->ws_ysnap.ptr : nullptr, (double*)op->ws_norm.ptr);
       }
@@ -774,7 +793,7 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
       }
       if (truncate) {
         const int64_t n_end = n0 + g.steps;
-        e = state_sq_norms(op, kv, n_end, (double*)op->ws_norm.ptr);
+        e = state_sq_norms(op, kv, n_end, np, (double*)op->ws_norm.ptr);
         if (e == cudaSuccess)
           e = cudaMemcpyAsync(nrm.data(), op->ws_norm.ptr, sizeof(double) * kv, cudaMemcpyDeviceToHost, stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
@@ -803,8 +822,8 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
     }
     if (!truncate) op->last_steps = sc.total;
     void* o = static_cast<char*>(out) + (size_t)v0 * n * ce;
-    e = launch_finish<R>(acc, acc_stride, op->n_omega, rows, 1.0 / (double)op->n_t, o, (int64_t)k * n, stream,
-                         s_out, n);
+    e = launch_finish<R>(acc, acc_stride, op->n_omega, (int64_t)kv * n, 1.0 / (double)op->n_t, o, (int64_t)k * n, stream,
+                         s_out, n, np == n ? 0 : op->nx, np == n ? 0 : (op->nx + 3) / 4 * 4);
     if (e != cudaSuccess) return cuda_fail(e, "finish");
   }
   int flag = 0;

@@ -94,11 +94,11 @@ namespace rsv {
 struct TileGraphKey {
   size_t elem;
   int steps, forced, y_first, kg;
-  bool adjoint;
+  bool adjoint, step_form;
   const void *state, *F, *Y, *norms;
   bool operator==(const TileGraphKey& o) const {
     return elem == o.elem && steps == o.steps && forced == o.forced && y_first == o.y_first && kg == o.kg &&
-           adjoint == o.adjoint && state == o.state && F == o.F && Y == o.Y && norms == o.norms;
+           adjoint == o.adjoint && step_form == o.step_form && state == o.state && F == o.F && Y == o.Y && norms == o.norms;
   }
 };
 struct TileGraph {
@@ -169,6 +169,7 @@ struct rsv_operator_s {
   void* tc_acc = nullptr;       // its FP32 partial-sum accumulators
   // stencil kinds: base-flow fields
   void* fld[8] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+  void* fldp[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};   // ADV3D, FP32: rows padded to 4 cells
   double c_dx = 0, c_dy = 0, c_dz = 0;
   int nx = 0, ny = 0, nz = 0;
   double visc = 0;
@@ -260,11 +261,12 @@ template <typename R>
 cudaError_t launch_analysis(const TileGeom& g, const void* Y, int s0, int s1, const void* tw,
                             const int64_t* pj, bool real_state, cpx<double>* acc, int64_t acc_stride,
                             cudaStream_t st);
-// out[j][r] = acc[j][r] * scale (* pscale[r mod n] when given), converted to the element type R
+// out[j][r] = acc[j][r] * scale (* pscale[r mod n] when given), converted to the element type R; with
+// nx > 0 the accumulator's rows of nx cells are padded to nxp (r counts the unpadded ones)
 template <typename R>
 cudaError_t launch_finish(const cpx<double>* acc, int64_t acc_stride, int n_omega, int64_t rows,
                           double scale, void* out, int64_t out_stride, cudaStream_t st,
-                          const double* pscale = nullptr, int64_t n = 0);
+                          const double* pscale = nullptr, int64_t n = 0, int nx = 0, int nxp = 0);
 // out[j][r] = in[j][r] * s[r mod n] for j < n_omega, r < rows (in and out may alias)
 template <typename R>
 cudaError_t launch_scale_block(const void* in, int64_t in_stride, void* out, int64_t out_stride, int n_omega,

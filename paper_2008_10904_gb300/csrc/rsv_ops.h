@@ -12,6 +12,7 @@ struct MarchTile {
   int y_first;       // tile steps s >= y_first store their starting state in Y
   int kg;            // vectors in the current group
   bool adjoint;      // march with A^H
+  bool step_form = false;   // F holds g_n at the tile's steps (step2d.cu), not the stage times' forcing
 };
 
 rsv_status build_gl1d(rsv_operator op, const rsv_operator_desc* d);
@@ -24,7 +25,24 @@ int default_tile_steps(rsv_operator op);
 size_t stage_scratch_bytes(rsv_operator op, int kg);
 
 // Number of kernels one march_tile call launches (for the launch accounting).
-int march_tile_kernels(rsv_operator op, int steps, int kg);
+int march_tile_kernels(rsv_operator op, int steps, int kg, bool step_form = false);
+
+// Step form of the march (step2d.cu): whether a march of k vectors takes it, the padded points per
+// vector of its tiles, and its scratch behind the state.
+bool step_form_taken(rsv_operator op, int k);
+int64_t step_points(rsv_operator op);
+size_t step_scratch_bytes(rsv_operator op, int kg);
+// Bytes of transformed coefficients (and their temporary) of one vector group.
+size_t step_coef_bytes(rsv_operator op, int kg, size_t* tmp);
+template <typename R>
+rsv_status step_coefficients(rsv_operator op, const void* fhat, int64_t f_stride, int kg, bool adjoint);
+// grid kinds (step2d.cu, step3d.cu)
+template <typename R>
+cudaError_t step_coefs_grid(rsv_operator op, const void* fhat, int64_t f_stride, int kg, bool adjoint, void* out,
+                            void* tmp, int64_t tmp_freqs);
+template <typename R>
+cudaError_t step_march_2d(rsv_operator op, const MarchTile& t, void* state, const void* G, void* Y);
+cudaError_t step_march_3d(rsv_operator op, const MarchTile& t, void* state, const void* G, void* Y);
 
 // S RK4 steps of the operator's stage kernel(s) on the state block (kg vectors).
 template <typename R>
@@ -32,9 +50,9 @@ cudaError_t march_tile(rsv_operator op, const MarchTile& t, void* state, const v
 
 // Coefficients the synthesis reads for one vector group: the input block itself
 // (stage-based kinds) or a per-march transform of it (dense kind).  Sets
-// *coef / *coef_stride / *n_tau_per_step.
+// *coef / *coef_stride / *synth_stride.  step_form: the step form's coefficients.
 template <typename R>
-rsv_status prepare_coefficients(rsv_operator op, const void* fhat, int64_t f_stride, int kg, bool adjoint,
+rsv_status prepare_coefficients(rsv_operator op, const void* fhat, int64_t f_stride, int kg, bool adjoint, bool step_form,
                                 const void** coef, int64_t* coef_stride, int* synth_stride);
 
 // Kind-specific work when the frequency grid (and so the step h) changes.
@@ -42,7 +60,7 @@ rsv_status on_frequencies(rsv_operator op);
 
 // Sets the flag if the state block holds a NaN / Inf (kinds without an in-kernel norm monitor).
 cudaError_t check_finite(rsv_operator op, const void* state, int64_t count, bool real_state);
-cudaError_t state_sq_norms(rsv_operator op, int kg, int64_t n_end, double* d_out);
+cudaError_t state_sq_norms(rsv_operator op, int kg, int64_t n_end, int64_t points, double* d_out);
 // Per-instance squared norms of vector 0 of the state after step n_end; the decay probe's initial state.
 cudaError_t instance_sq_norms(rsv_operator op, int64_t n_end, double* d_out);
 cudaError_t probe_initial_state(rsv_operator op, uint64_t seed);

@@ -1322,7 +1322,27 @@ rsv_status build_adv3d(rsv_operator op, const rsv_operator_desc* d) {
     il[4 * q + 2] = (float)Uy[q];
     il[4 * q + 3] = (float)Uz[q];
   }
-  return upload(op, il.data(), il.size() * sizeof(float), &op->fld[4]);
+  st = upload(op, il.data(), il.size() * sizeof(float), &op->fld[4]);
+  const int nxp = (d->nx + 3) / 4 * 4;
+  for (int a = 0; a < 5; ++a) op->fldp[a] = op->fld[a];
+  if (st != RSV_OK || nxp == d->nx) return st;
+  // the step form's rows are padded to four cells (zeros)
+  const size_t rows = (size_t)d->ny * d->nz;
+  for (int a = 0; a < 5; ++a) {
+    const size_t w = (a < 4 ? 1 : 4) * sizeof(float);
+    void* p = nullptr;
+    cudaError_t e = cudaMalloc(&p, rows * nxp * w);
+    if (e != cudaSuccess) return cuda_fail(e, "operator allocation");
+    op->dev.push_back(p);
+    e = cudaMemset(p, 0, rows * nxp * w);
+    if (e == cudaSuccess)
+      e = cudaMemcpy2D(p, nxp * w, op->fld[a], d->nx * w, d->nx * w, rows, cudaMemcpyDeviceToDevice);
+    if (e != cudaSuccess) return cuda_fail(e, "operator upload");
+    op->fldp[a] = p;
+  }
+  const cudaError_t e = cudaStreamSynchronize(nullptr);
+  if (e != cudaSuccess) return cuda_fail(e, "operator upload");
+  return st;
 }
 
 // Workspace behind the state in the march: two stage-input buffers and the accumulator.

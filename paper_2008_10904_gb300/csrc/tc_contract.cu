@@ -257,8 +257,9 @@ __global__ void __launch_bounds__(256, 1) tc_contract_kernel(ContractArgs a) {
 //
 // One CTA per SM walks the 128-row tiles blockIdx.x, blockIdx.x + gridDim.x, ...
 // with warp roles connected by mbarrier rings:
-//   warp 12 (one thread) producer: bulk-copies each K chunk of the long operand
-//                        in its storage precision into a 4-deep raw ring;
+//   warp 12              producer: bulk-copies each K chunk of the long operand
+//                        in its storage precision into an 8-deep raw ring, one
+//                        row slice per lane;
 //   warp 14 (one thread) producer: bulk-copies the chunk's pre-split twiddles
 //                        into a 2-deep B ring;
 //   warps 0-3            converters: one row each, raw value -> TF32 hi / lo in
@@ -317,9 +318,10 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 
 // Raw layout of one chunk in shared memory: complex modes [8][128] float2
 // (pair index jj = frequency or step within the chunk), real analysis
-// [16][128] float.  Only the valid pair indices and rows are copied.
-__device__ __forceinline__ uint32_t issue_raw(const ContractArgs& a, int64_t r0, int nr, int kc, unsigned char* raw,
-                                              uint64_t* bar) {
+// [16][128] float.  Only the valid pair indices and rows are copied.  Called by the whole warp: lane l
+// issues the copy of pair index l (one thread issuing all 8 or 16 bounded the kernel's chunk rate).
+__device__ __forceinline__ void issue_raw(const ContractArgs& a, int64_t r0, int nr, int kc, unsigned char* raw,
+                                          uint64_t* bar, int lane) {
   const bool real = a.mode == ANAL_R;
   const int npair = real ? kKc : kKc / 2;
   const uint32_t esz = real ? 4 : 8;
@@ -332,13 +334,14 @@ __device__ __forceinline__ uint32_t issue_raw(const ContractArgs& a, int64_t r0,
   }
   const uint32_t bytes_row = (uint32_t)nr * esz;
   const uint32_t total = hi > lo ? (uint32_t)(hi - lo) * bytes_row : 0u;
-  tc::mbar_arrive_expect_tx(bar, total);
+  if (lane == 0) tc::mbar_arrive_expect_tx(bar, total);
+  __syncwarp();
   const int64_t stride = (a.mode == ANAL_C || a.mode == ANAL_R) ? a.rows : a.src_stride;
-  for (int idx = lo; idx < hi; ++idx) {
+  const int idx = lo + lane;
+  if (idx < hi) {
     const unsigned char* src = reinterpret_cast<const unsigned char*>(a.src) + ((int64_t)idx * stride + r0) * esz;
     tc::bulk_g2s(raw + (uint32_t)(idx - kc * npair) * kRowsCta * esz, src, bytes_row, bar);
   }
-  return total;
 }
 
 __device__ __forceinline__ void convert_row(const ContractArgs& a, int64_t r0, int kc, int rr, const unsigned char* raw,
@@ -471,7 +474,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(Contr
   const int nsub = a.N > 256 ? 2 : 1;
 
   if (warp == 12) {
-    if (lane == 0) {  // producer of the long operand
+    {  // producer of the long operand (the whole warp)
       uint32_t g = 0;
       bool ok = true;
       for (int64_t t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
@@ -480,8 +483,11 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(Contr
         for (int h = 0; h < nsub && ok; ++h) {   // the second sub-tile re-reads the rows from L2
           for (int kc = 0; kc < chunks; ++kc, ++g) {
             const uint32_t rs = g % kRawRing, ru = g / kRawRing;
-            if (ru > 0 && !pwait(&pb->raw_empty[rs], (ru - 1) & 1, abort_flag)) { ok = false; break; }
-            issue_raw(a, r0, nr, kc, raw + rs * kRawBytes, &pb->raw_full[rs]);
+            if (ru > 0 && !__all_sync(0xffffffffu, pwait(&pb->raw_empty[rs], (ru - 1) & 1, abort_flag))) {
+              ok = false;
+              break;
+            }
+            issue_raw(a, r0, nr, kc, raw + rs * kRawBytes, &pb->raw_full[rs], lane);
           }
         }
       }
