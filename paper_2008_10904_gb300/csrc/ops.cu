@@ -79,6 +79,9 @@ rsv_status build_gl1d(rsv_operator op, const rsv_operator_desc* d) {
   }
   const std::vector<std::complex<double>>* arrs[6] = {&lo, &di, &up, &alo, &adi, &aup};
   op->tri_host.assign((size_t)12 * tot, 0.0);
+  op->tri_real = true;
+  for (const auto* a : arrs)
+    for (const std::complex<double>& x : *a) op->tri_real = op->tri_real && x.imag() == 0.0;
   for (int a = 0; a < 6; ++a) {
     rsv_status s = upload_cvec(op, *arrs[a], &op->tri[a]);
     if (s != RSV_OK) return s;
@@ -179,7 +182,7 @@ size_t stage_scratch_bytes(rsv_operator op, int kg) {
 
 int march_tile_kernels(rsv_operator op, int steps, int kg, bool step_form) {
   if (step_form) {   // 2-D FP32: one launch per step; 3-D: two; FP64: one per stage
-    if (op->kind == RSV_OP_ADR2D) return (op->prec == RSV_PREC_FP32 ? steps : 4 * steps) + 1;
+    if (op->kind == RSV_OP_ADR2D) return op->prec == RSV_PREC_FP32 ? steps + 1 : 4 * steps + 2;
     return 2 * steps + 1;
   }
   switch (op->kind) {
@@ -206,6 +209,7 @@ int march_tile_kernels(rsv_operator op, int steps, int kg, bool step_form) {
 }
 
 rsv_status on_frequencies(rsv_operator op) {
+  for (JumpPlan& p : op->jump) p = JumpPlan();
   if (op->kind == RSV_OP_DENSE) return dense_on_frequencies(op);
   if (op->kind == RSV_OP_GL1D && op->scheme == RSV_SCHEME_CN) return gl1d_cn_factors(op);
   return RSV_OK;
@@ -233,9 +237,11 @@ int64_t step_points(rsv_operator op) {
   return op->n;
 }
 
-// A second state buffer and one stage buffer.
+// A second state buffer and one stage buffer, then (2-D FP64) the stages' row and sponge tables.
 size_t step_scratch_bytes(rsv_operator op, int kg) {
-  return 2 * (size_t)kg * step_points(op) * (op->prec == RSV_PREC_FP64 ? 8 : 4);
+  const size_t el = op->prec == RSV_PREC_FP64 ? 8 : 4;
+  const size_t tab = op->kind == RSV_OP_ADR2D && el == 8 ? (size_t)(17 * (size_t)op->ny + op->nx) * el : 0;
+  return 2 * (size_t)kg * step_points(op) * el + tab;
 }
 
 // The temporary of the coefficient transform holds as many frequencies as 64 MB take (at least one),

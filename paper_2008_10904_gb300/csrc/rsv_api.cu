@@ -138,6 +138,8 @@ rsv_operator_s::~rsv_operator_s() {
   }
   if (copy_stream) cudaStreamDestroy(copy_stream);
   if (ws_scaled.ptr) cudaFree(ws_scaled.ptr);
+  for (Workspace* w : {&ws_band[0], &ws_band[1], &ws_part})
+    if (w->ptr) cudaFree(w->ptr);
   for (cudaEvent_t e : prof.pool) cudaEventDestroy(e);
 }
 
@@ -253,8 +255,13 @@ extern "C" rsv_status rsv_describe(rsv_operator op, char* buf, int32_t buflen) {
   if (!op || !buf || buflen < 1) return fail(RSV_ERR_INVALID_ARG, "bad describe arguments");
   static const char* kinds[] = {"gl1d", "dense", "adr2d", "adv3d"};
   const char* path = "cuda-core stages";
-  if (op->kind == RSV_OP_GL1D)
-    path = op->scheme == RSV_SCHEME_CN ? "cuda-core crank-nicolson tile kernel" : "cuda-core tile kernel";
+  if (op->kind == RSV_OP_GL1D) {
+    if (jump_taken(op, 1))
+      path = op->scheme == RSV_SCHEME_CN ? "cuda-core crank-nicolson jump kernels (few pairs, else tile kernel)"
+                                         : "cuda-core jump kernels (few pairs, else tile kernel)";
+    else
+      path = op->scheme == RSV_SCHEME_CN ? "cuda-core crank-nicolson tile kernel" : "cuda-core tile kernel";
+  }
   if (op->kind == RSV_OP_ADV3D && op->prec == RSV_PREC_FP32) {
     const char* e = getenv("RSV_STENCIL3D_STAGED");
     const bool pairs = !(e != nullptr && e[0] == '1') && !op->bf16_state && op->nx % 4 == 0 &&
@@ -584,7 +591,11 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
   const int64_t n = op->n;
   const size_t se = state_elem_bytes(op);
   const bool sf = step_form_taken(op, k);
+  const bool jump = jump_taken(op, k);
+  const int jp = jump ? jump_plan(op, adjoint).p : 1;
   const int64_t np = sf ? step_points(op) : n;     // points per vector of the march's tiles
+  // TRM truncation by the state norm: per-vector peak over the tile ends so far
+  const bool truncate = opts != nullptr && opts->variant == RSV_TRM && opts->tail_tol > 0.0;
   auto scratch_bytes = [&](int kg_) { return sf ? step_scratch_bytes(op, kg_) : stage_scratch_bytes(op, kg_); };
   const bool acc_in_out = op->prec == RSV_PREC_FP64 && trial == nullptr && np == n;
   // Tile length S and vector-group size kg: the requested / default tile and all k vectors, shrunk
@@ -597,7 +608,12 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
   if (trial) {
     S = trial->S;
     kg = trial->kg;
+  } else if (jump && !truncate && !(opts && opts->tile_steps > 0) && op->tuned_k != k) {
+    // the jumps' launches are short: tiles as long as 128 MB of snapshots, a window at most
+    S = (int)std::max<int64_t>(S, std::min<int64_t>(op->n_t, ((int64_t)128 << 20) / ((int64_t)kg * n * 16)));
   }
+  // rows of the forcing tile: steps and stage times, whole steps only, or whole steps and jumps
+  auto f_rows = [&](int s_) -> int64_t { return jump ? s_ + s_ / jp + jp + 1 : sf ? s_ : 2 * (int64_t)s_ + 1; };
   {
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
@@ -609,13 +625,15 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
     const double budget = 0.9 * (double)(free_b + held);
     auto need = [&](int s_, int kg_) {
       const double rows_ = (double)kg_ * np;
-      double b = rows_ * se + (double)scratch_bytes(kg_) + (sf ? s_ : 2.0 * s_ + 1) * rows_ * se + s_ * rows_ * se;
+      double b = rows_ * se + (double)scratch_bytes(kg_) + (double)f_rows(s_) * rows_ * se + s_ * rows_ * se;
       if (!acc_in_out) b += (double)op->n_omega * rows_ * sizeof(cpx<double>);
       if (sf) {
         size_t tmp = 0;
         b += (double)step_coef_bytes(op, kg_, &tmp);
         b += (double)tmp;
       }
+      if (jump) b += 2.0 * op->n_omega * rows_ * sizeof(cpx<double>);
+      if (op->prec == RSV_PREC_FP64) b += (double)analysis64_part_bytes(op, (int64_t)rows_, s_);
       if (s_in) b += (double)op->n_omega * rows_ * coef_bytes(op);
       if (op->kind == RSV_OP_DENSE) b += 2.0 * op->n_omega * rows_ * 2 * sizeof(R);
       if (host_in) b += 2.0 * op->n_omega * rows_ * coef_bytes(op);   // staging buffers
@@ -637,9 +655,17 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
   op->last_group = kg;
   const int64_t rows_max = (int64_t)kg * np;
   if ((st = ensure(op->ws_state, rows_max * se + scratch_bytes(kg))) != RSV_OK) return st;
-  if ((st = ensure(op->ws_ftile, (size_t)(sf ? S : 2 * S + 1) * rows_max * se)) != RSV_OK) return st;
+  if ((st = ensure(op->ws_ftile, (size_t)f_rows(S) * rows_max * se)) != RSV_OK) return st;
   if ((st = ensure(op->ws_ysnap, (size_t)S * rows_max * se)) != RSV_OK) return st;
   if ((st = ensure(op->ws_norm, (size_t)kg * op->n_inst * sizeof(double))) != RSV_OK) return st;
+  if (jump) {
+    const size_t cb = (size_t)op->n_omega * rows_max * sizeof(cpx<double>);
+    if ((st = ensure(op->ws_coef, cb)) != RSV_OK || (st = ensure(op->ws_coef2, cb)) != RSV_OK) return st;
+  }
+  if (op->prec == RSV_PREC_FP64) {
+    const size_t pb = analysis64_part_bytes(op, rows_max, S);
+    if (pb > 0 && (st = ensure(op->ws_part, pb)) != RSV_OK) return st;
+  }
   if (!acc_in_out && (st = ensure(op->ws_acc, (size_t)op->n_omega * rows_max * sizeof(cpx<double>))) != RSV_OK)
     return st;
   if ((e = cudaMemsetAsync(op->d_flag, 0, sizeof(int), stream)) != cudaSuccess) return cuda_fail(e, "flag reset");
@@ -737,24 +763,40 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
       gin = op->ws_scaled.ptr;
       gin_stride = urows;
     }
-    {
+    if (jump) {
+      ProfScope ps(op, PROF_GLUE, 1);
+      st = jump_coefficients(op, gin, gin_stride, kv, adjoint, op->ws_coef.ptr, op->ws_coef2.ptr);
+      g.coef_stride = rows;
+    } else {
       ProfScope ps(op, PROF_GLUE, op->kind == RSV_OP_DENSE ? (kv == k ? 3 : 2 * op->n_omega + 1) : sf ? 3 : 0);
       st = prepare_coefficients<R>(op, gin, gin_stride, kv, adjoint, sf, &fh, &g.coef_stride, &synth_stride);
     }
     if (st != RSV_OK) return st;
     g.tau_stride = synth_stride;
-    // TRM truncation by the state norm: per-vector peak over the tile ends so far
-    const bool truncate = opts != nullptr && opts->variant == RSV_TRM && opts->tail_tol > 0.0;
     std::vector<double> peak(truncate ? kv : 0, 0.0), nrm(truncate ? kv : 0, 0.0);
     if (trial && (e = cudaEventRecord(ev0, stream)) != cudaSuccess) return cuda_fail(e, "trial event");
-    for (int64_t n0 = 0; n0 < (trial ? std::min<int64_t>(S, sc.total) : sc.total); n0 += S) {
+    for (int64_t n0 = 0; n0 < (trial ? std::min<int64_t>(S, sc.total) : sc.total); n0 += g.steps) {
       g.n0 = n0;
       g.steps = (int)std::min<int64_t>(S, sc.total - n0);
+      if (jump && !trial) {   // tiles forced or unforced, analysed or not, as a whole; long ones before the analysis
+        const int64_t end = n0 < sc.first && !truncate && !(opts && opts->tile_steps > 0)
+                                ? std::min<int64_t>(sc.first, n0 + (int64_t)S * jp)
+                                : std::min<int64_t>(sc.total, (n0 / S + 1) * S);
+        g.steps = (int)((n0 < sc.forced ? std::min(end, sc.forced) : end) - n0);
+      }
       g.n_tau = synth_stride == 2 ? g.steps : 0;
       const bool forced = trial ? true : n0 < sc.forced;
       const bool analysed = trial ? true : n0 + g.steps > sc.first;
-      if (forced) {
-        if (sizeof(R) == 4 && tc_contract_supported(op, true)) {
+      if (jump) {
+        const int yf = trial ? 0 : (analysed ? (int)std::max<int64_t>(0, sc.first - n0) : g.steps);
+        e = jump_march(op, g, adjoint, kv, g.steps, forced, yf, op->ws_coef.ptr, op->ws_coef2.ptr, op->ws_state.ptr,
+                       op->ws_ftile.ptr, analysed ? op->ws_ysnap.ptr : nullptr);
+        if (e != cudaSuccess) return cuda_fail(e, "march tile");
+      } else if (forced) {
+        if (sizeof(R) == 8 && synth_stride == 2) {
+          ProfScope ps(op, PROF_SYNTH);
+          e = synth64(op, g, fh, op->ws_ftile.ptr);
+        } else if (sizeof(R) == 4 && tc_contract_supported(op, true)) {
           const int nt = g.n_tau > 0 ? g.n_tau : 2 * g.steps + 1;
           const int calls = (nt + (op->real_state ? 511 : 255)) / (op->real_state ? 512 : 256);
           ProfScope ps(op, PROF_SYNTH, 2 * calls);
@@ -774,7 +816,7 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
       mt.kg = kv;
       mt.adjoint = adjoint;
       mt.step_form = sf;
-      {
+      if (!jump) {
         ProfScope ps(op, PROF_MARCH, march_tile_kernels(op, g.steps, kv, sf));
         e = march_tile<R>(op, mt, op->ws_state.ptr, forced ? op->ws_ftile.ptr : nullptr,
                           analysed ? op->ws_ysnap.ptr : nullptr, (double*)op->ws_norm.ptr);
@@ -785,13 +827,16 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
           ProfScope ps(op, PROF_ANALYSIS, 2);
           e = tc_analysis(op, g, op->ws_ysnap.ptr, y_first, g.steps, acc, acc_stride);
         } else {
-          ProfScope ps(op, PROF_ANALYSIS);
-          e = launch_analysis<R>(g, op->ws_ysnap.ptr, y_first, g.steps, op->d_tw, op->d_pj, op->real_state, acc,
-                                 acc_stride, stream);
+          ProfScope ps(op, PROF_ANALYSIS, sizeof(R) == 8 && analysis64_part_bytes(op, rows, g.steps - y_first) > 0 ? 2 : 1);
+          if (sizeof(R) == 8)
+            e = analysis64(op, g, op->ws_ysnap.ptr, y_first, g.steps, acc, acc_stride, op->ws_part.ptr);
+          else
+            e = launch_analysis<R>(g, op->ws_ysnap.ptr, y_first, g.steps, op->d_tw, op->d_pj, op->real_state, acc,
+                                   acc_stride, stream);
         }
         if (e != cudaSuccess) return cuda_fail(e, "analysis");
       }
-      if (truncate) {
+      if (truncate && ((n0 + g.steps) % S == 0 || n0 + g.steps == sc.total)) {   // check points: the tile ends
         const int64_t n_end = n0 + g.steps;
         e = state_sq_norms(op, kv, n_end, np, (double*)op->ws_norm.ptr);
         if (e == cudaSuccess)

@@ -101,6 +101,14 @@ struct TileGraphKey {
            adjoint == o.adjoint && step_form == o.step_form && state == o.state && F == o.F && Y == o.Y && norms == o.norms;
   }
 };
+// Jumps of FP64 1-D marches (step1d.cu), per direction: length p, diagonals -wl .. wr of the p-step and
+// -wl1 .. wr1 of the one-step matrix, and the matrices once built.
+struct JumpPlan {
+  int state = 0;            // 0 not planned, 1 taken, 2 not
+  int p = 1, wl = 0, wr = 0, wl1 = 0, wr1 = 0;
+  bool built = false;
+  void *Tp = nullptr, *T1 = nullptr;
+};
 struct TileGraph {
   TileGraphKey key;
   cudaGraphExec_t exec;
@@ -139,6 +147,9 @@ struct rsv_operator_s {
   // GL1D: tridiagonal coefficients, direct then adjoint: lo, di, up
   void* tri[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   int gl_max_n = 0;
+  bool tri_real = false;                // every coefficient is real
+  rsv::JumpPlan jump[2];                // direct, adjoint (reset with the frequencies)
+  rsv::Workspace ws_band[2], ws_part;   // step matrices; partial sums of the FP64 analysis
   // packed launch of uneven GL1D batches (built per vector-group size): slot map, CTA count, threads
   // and slots per thread of a CTA, CTAs per wave (SMs x CTAs resident per SM)
   void* pack_map = nullptr;

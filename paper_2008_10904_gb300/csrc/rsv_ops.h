@@ -44,6 +44,19 @@ template <typename R>
 cudaError_t step_march_2d(rsv_operator op, const MarchTile& t, void* state, const void* G, void* Y);
 cudaError_t step_march_3d(rsv_operator op, const MarchTile& t, void* state, const void* G, void* Y);
 
+// FP64 1-D marches of few pairs by jumps over several steps (step1d.cu)
+bool jump_taken(rsv_operator op, int k);
+const JumpPlan& jump_plan(rsv_operator op, bool adjoint);
+rsv_status jump_coefficients(rsv_operator op, const void* fhat, int64_t f_stride, int kg, bool adjoint, void* c1, void* cp);
+cudaError_t jump_march(rsv_operator op, TileGeom g, bool adjoint, int kg, int steps, bool forced, int y_first,
+                       const void* c1, const void* cp, void* state, void* G, void* Y);
+
+// FP64 contractions at whole steps (contract64.cu)
+cudaError_t synth64(rsv_operator op, const TileGeom& g, const void* coef, void* F);
+size_t analysis64_part_bytes(rsv_operator op, int64_t rows, int steps);
+cudaError_t analysis64(rsv_operator op, const TileGeom& g, const void* Y, int s0, int s1, cpx<double>* acc,
+                       int64_t acc_stride, void* part);
+
 // S RK4 steps of the operator's stage kernel(s) on the state block (kg vectors).
 template <typename R>
 cudaError_t march_tile(rsv_operator op, const MarchTile& t, void* state, const void* F, void* Y, double* norms);

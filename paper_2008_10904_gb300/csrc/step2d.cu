@@ -174,26 +174,35 @@ Grid3<R> grid3_of(rsv_operator op) {
 //
 // A warp owns a strip of 120 cells in x (lane l: four consecutive cells; lanes 0 and 31 are the halo
 // of four cells, one per stage) and a run of rows, and walks up the rows: with row r of u just
-// loaded it evaluates w1 on row r - 1, w2 on r - 2, w3 on r - 3 and u' on r - 4.  Rows live in
-// registers (x neighbours across lanes by shuffles), so there is no barrier and no shared-memory
-// traffic but the per-warp ring that stages u and g by 16-byte asynchronous copies.  A run starts
-// four rows early and ends four late; what it computes there is not stored.  Rows outside the grid
-// have zero coefficients, so they stay zero.  Issue slots bound it, not bytes: per row and warp 96
-// arithmetic instructions of about 150.
+// loaded it evaluates w1 on row r - 1, w2 on r - 2, w3 on r - 3 and u' on r - 4.  The rows of a
+// stencil live in registers (x neighbours across lanes by shuffles), so there is no barrier and no
+// shared-memory traffic but the per-warp ring that stages u and g by 16-byte asynchronous copies.  A
+// run starts four rows early and ends four late; what it computes there is not stored.  Rows and
+// columns outside the grid have zero factors, so they stay zero.  Issue slots bound it, not bytes: the
+// stage factors h / m are multiplied into the row coefficients, so that a cell costs one addition and
+// four multiply-adds per stage.
+//
+// The rows of all (vector, strip) columns are one list that is cut into equal chunks, one per warp
+// (block of one warp) and as many as the GPU holds at once; a chunk that crosses from one column to
+// the next runs as two runs.  1024 x 512 x 16 vectors: 28 us per step with 16 warps per SM (12: 33, 8: 43),
+// against 103 us for the two stage-pair kernels; 96 MB of DRAM traffic per step.
 // ---------------------------------------------------------------------------
-constexpr int kStripCells = 120, kStreamWarps = 2, kRing = 8, kAhead = 6, kMaxRun = 128;
+constexpr int kStripCells = 120, kGroups = 3, kMaxChunk = 256, kWarpsPerSm = 16;
 
 struct Stream2D {
   int nx, nxp, ny, kg;
-  int strips, runs, run_rows;
+  int strips, chunk;
+  int64_t total;             // rows of all columns
   int64_t vstride;
   const float *U, *r;
-  float i2dx, nx2, ny2, h, h2, h3, h4;   // h / m for the stages' factors
+  float i2dx, nx2, ny2;
+  float f[4];                // h / 4, h / 3, h / 2, h: the stages' factors
   int sponge_cells;
   float sponge_amp, sponge_inv;
   int adj;
 };
 
+// Copies 16 bytes, or writes zeros without reading.
 __device__ __forceinline__ void cp16_zfill(uint32_t dst, const float* src, bool ok) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
 }
@@ -201,214 +210,243 @@ __device__ __forceinline__ void cp16_zfill(uint32_t dst, const float* src, bool 
 struct F4 {
   float v[4];
 };
+__device__ __forceinline__ F4 lds4(uint32_t a) {
+  F4 o;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(o.v[0]), "=f"(o.v[1]), "=f"(o.v[2]), "=f"(o.v[3]) : "r"(a) : "memory");
+  return o;
+}
 
-// The rows of one warp.  WALL: the strip or the run reaches a wall or its sponge.
+constexpr uint32_t kSlotBytes = 2 * 32 * 16;                       // a row of u and a row of g
+constexpr uint32_t kRingBytes = kGroups * 3 * kSlotBytes;
+// per row of the run (with 8 rows before and after it): 4 stages x (west, east, diagonal, north / south) x h / m,
+// then the sponge depths
+constexpr uint32_t kRowBytes = 4 * 16;
+constexpr size_t stream2d_smem(int chunk) { return kRingBytes + (size_t)(chunk + 16) * (kRowBytes + 4); }
+
+// One run: rows [ya, yb) of a column.  WALL: the strip reaches a wall in x or its sponge (elsewhere the
+// row's sponge rate is part of the row's diagonal coefficient).
 template <bool WALL>
 __device__ __forceinline__ void stream2d_rows(const Stream2D& P, const float* __restrict__ u, const float* __restrict__ g,
-                                              float* __restrict__ out, float* __restrict__ ysnap, float4 (*ring)[2][32],
-                                              const float4* rowc, const float* rowt, int ya, int yb, int gx, int lane,
+                                              float* __restrict__ out, float* __restrict__ ysnap, uint32_t ring,
+                                              uint32_t rows, const float* rowt, int ya, int yb, int gx, int lane,
                                               int64_t base) {
   const bool in_x = gx >= 0 && gx < P.nxp;
   const bool owner = lane >= 1 && lane <= 30 && gx < P.nxp;
   const bool forced = g != nullptr;
-  bool cell[4];
-  float sx[4];   // sponge depth of the lane's columns (0: none)
+  float sx[4], sg[4];   // sponge depth and rate of the lane's columns (0: none)
+  float m[4];           // 1 inside the grid, 0 outside
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     const int i = gx + c;
-    cell[c] = i >= 0 && i < P.nx;
+    const bool in = i >= 0 && i < P.nx;
     const int d = min(i, P.nx - 1 - i);
-    sx[c] = cell[c] && d < P.sponge_cells ? (float)(P.sponge_cells - d) * P.sponge_inv : 0.f;
+    m[c] = in ? 1.f : 0.f;
+    sx[c] = in && d < P.sponge_cells ? (float)(P.sponge_cells - d) * P.sponge_inv : 0.f;
+    sg[c] = P.sponge_amp * sx[c] * sx[c];
   }
-  // row r of u (from ya - 4) and row r - 4 of g go to ring slot (r - ya + 4) mod kRing
+  const bool edge_x = WALL && __any_sync(0xffffffffu, m[0] * m[1] * m[2] * m[3] == 0.f);
+  // iteration i loads row ya - 4 + i of u and row ya - 8 + i of g; three groups of three ring slots:
+  // the current three iterations', the previous three's and the next three's
+  const int iters = yb - ya + 8;
+  const int u_lo = max(0, 4 - ya), u_n = min(iters, P.ny - ya + 4) - u_lo;   // iterations whose row is inside the grid
   const int64_t off = base + (in_x ? gx : 0);
   const float* pu = u + off + (int64_t)(ya - 4) * P.nxp;
   const float* pg = (forced ? g : u) + off + (int64_t)(ya - 8) * P.nxp;
-  const uint32_t slot0 = (uint32_t)__cvta_generic_to_shared(&ring[0][0][lane]);
-  const int iters = yb - ya + 8;
-  auto prefetch = [&](int i) {   // iteration i: row ya - 4 + i
-    if (i < iters) {
-      const uint32_t d = slot0 + (uint32_t)(i & (kRing - 1)) * (2 * 32 * 16);
-      const int r = ya - 4 + i;
-      const bool oku = in_x && r >= 0 && r < P.ny;
-      cp16_zfill(d, oku ? pu : u, oku);
-      if (forced && i >= 8) cp16_zfill(d + 32 * 16, in_x ? pg : u, in_x);
-    }
+  auto prefetch = [&](int i, uint32_t dst) {
+    cp16_zfill(dst, pu, in_x && (unsigned)(i - u_lo) < (unsigned)u_n);
+    if (forced) cp16_zfill(dst + 32 * 16, pg, in_x && i >= 8 && i < iters);
     pu += P.nxp;
     pg += P.nxp;
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
+  uint32_t cur = ring + 16 * lane, prev = cur + 3 * kSlotBytes, next = cur + 6 * kSlotBytes;
 #pragma unroll
-  for (int q = 0; q < kAhead; ++q) prefetch(q);
-  F4 ur[6], w1[3], w2[3], w3[3];
+  for (int q = 0; q < 3; ++q) prefetch(q, cur + q * kSlotBytes);
+  F4 ur[3], w1[3], w2[3], w3[3];
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
+  for (int q = 0; q < 3; ++q)
 #pragma unroll
-    for (int q = 0; q < 6; ++q) ur[q].v[c] = 0.f;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) w1[q].v[c] = w2[q].v[c] = w3[q].v[c] = 0.f;
-  }
-  // u0 + f A x on a row from the rows below, at and above it; e: the row's index in rowc
-  auto stage = [&](const F4& xb, const F4& xc, const F4& xt, const F4& u0, int e, float f) -> F4 {
-    const float4 rc = rowc[e];   // west, east, diagonal, north / south
+    for (int c = 0; c < 4; ++c) ur[q].v[c] = w1[q].v[c] = w2[q].v[c] = w3[q].v[c] = 0.f;
+  // u0 + h/m A x on a row from the rows below, at and above it; e: the row's index in the table
+  auto stage = [&](const F4& xb, const F4& xc, const F4& xt, const F4& u0, int e, int st) -> F4 {
+    const F4 rc = lds4(rows + (uint32_t)e * kRowBytes + 16 * st);   // west, east, diagonal, north / south
     const float left = __shfl_up_sync(0xffffffffu, xc.v[3], 1), right = __shfl_down_sync(0xffffffffu, xc.v[0], 1);
+    float cc[4] = {rc.v[2], rc.v[2], rc.v[2], rc.v[2]};
+    if (WALL) {
+      const float ty = rowt[e];   // the rate of the nearer wall: the larger depth
+#pragma unroll
+      for (int c = 0; c < 4; ++c) cc[c] = fmaf(-P.f[st], sx[c] > ty ? sg[c] : P.sponge_amp * ty * ty, rc.v[2]);
+    }
     F4 o;
-    const float ty = WALL ? rowt[e] : 0.f;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      float cc = rc.z;
-      if (WALL) {
-        const float t = fmaxf(sx[c], ty);
-        cc = rc.z - P.sponge_amp * t * t;
-      }
-      float a = rc.w * (xb.v[c] + xt.v[c]);
-      a = fmaf(rc.x, c == 0 ? left : xc.v[c - 1], a);
-      a = fmaf(rc.y, c == 3 ? right : xc.v[c + 1], a);
-      a = fmaf(cc, xc.v[c], a);
-      o.v[c] = fmaf(f, a, u0.v[c]);
-      if (WALL) o.v[c] = cell[c] ? o.v[c] : 0.f;
+      float a = fmaf(rc.v[3], xb.v[c] + xt.v[c], u0.v[c]);
+      a = fmaf(rc.v[0], c == 0 ? left : xc.v[c - 1], a);
+      a = fmaf(rc.v[1], c == 3 ? right : xc.v[c + 1], a);
+      o.v[c] = fmaf(cc[c], xc.v[c], a);
+    }
+    if (edge_x) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) o.v[c] = m[c] != 0.f ? o.v[c] : 0.f;
     }
     return o;
   };
-  float* po = out + base + (int64_t)ya * P.nxp + gx;
-  float* py = ysnap + base + (int64_t)ya * P.nxp + gx;   // used only when ysnap is given
-  for (int i0 = 0; i0 < iters; i0 += 6) {
+  float* po = out + base + (int64_t)(ya - 8) * P.nxp + gx;
+  float* py = ysnap + base + (int64_t)(ya - 8) * P.nxp + gx;   // used only when ysnap is given
+  for (int i0 = 0; i0 < iters; i0 += 3) {
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
+    for (int q = 0; q < 3; ++q) {
       const int i = i0 + q;
       if (i >= iters) break;
-      asm volatile("cp.async.wait_group %0;" ::"n"(kAhead - 1) : "memory");
-      const float4(&slot)[2][32] = ring[i & (kRing - 1)];
-      const float4 nu4 = slot[0][lane];
-      ur[q].v[0] = nu4.x;
-      ur[q].v[1] = nu4.y;
-      ur[q].v[2] = nu4.z;
-      ur[q].v[3] = nu4.w;
-      float4 gv = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (forced && i >= 8) gv = slot[1][lane];
-      prefetch(i + kAhead);
-      // rows: u[r - d] in ur[(q - d) mod 6], w_s[r - d] in w_s[(q - d) mod 3]; rowc[e] holds row ya - 8 + e
-      w1[(q + 2) % 3] = stage(ur[(q + 4) % 6], ur[(q + 5) % 6], ur[q], ur[(q + 5) % 6], i + 3, P.h4);
-      w2[(q + 1) % 3] = stage(w1[q % 3], w1[(q + 1) % 3], w1[(q + 2) % 3], ur[(q + 4) % 6], i + 2, P.h3);
-      w3[q % 3] = stage(w2[(q + 2) % 3], w2[q % 3], w2[(q + 1) % 3], ur[(q + 3) % 6], i + 1, P.h2);
-      if (i >= 8) {
-        const F4 o = stage(w3[(q + 1) % 3], w3[(q + 2) % 3], w3[q % 3], ur[(q + 2) % 6], i, P.h);
-        if (owner) {
-          *reinterpret_cast<float4*>(po) = make_float4(o.v[0] + gv.x, o.v[1] + gv.y, o.v[2] + gv.z, o.v[3] + gv.w);
-          if (ysnap) {
-            const F4& y = ur[(q + 2) % 6];
-            __stcs(reinterpret_cast<float4*>(py), make_float4(y.v[0], y.v[1], y.v[2], y.v[3]));
-          }
-        }
-        po += P.nxp;
-        py += P.nxp;
+      asm volatile("cp.async.wait_group 2;" ::: "memory");
+      ur[q] = lds4(cur + q * kSlotBytes);
+      // rows r - 3 and r - 4 of u are read again from the ring
+      const F4 u3 = lds4(prev + q * kSlotBytes);
+      const F4 u4 = lds4(q == 0 ? next + 2 * kSlotBytes : prev + (q - 1) * kSlotBytes);
+      const F4 gv = lds4(cur + q * kSlotBytes + 32 * 16);
+      prefetch(i + 3, next + q * kSlotBytes);
+      // rows: u[r - d], w_s[r - d] in slot (q - d) mod 3; the table's row e is row ya - 8 + e
+      w1[(q + 2) % 3] = stage(ur[(q + 1) % 3], ur[(q + 2) % 3], ur[q], ur[(q + 2) % 3], i + 3, 0);
+      w2[(q + 1) % 3] = stage(w1[q], w1[(q + 1) % 3], w1[(q + 2) % 3], ur[(q + 1) % 3], i + 2, 1);
+      w3[q] = stage(w2[(q + 2) % 3], w2[q], w2[(q + 1) % 3], u3, i + 1, 2);
+      const F4 o = stage(w3[(q + 1) % 3], w3[(q + 2) % 3], w3[q], u4, i, 3);
+      if (owner && i >= 8) {
+        float4 v = make_float4(o.v[0], o.v[1], o.v[2], o.v[3]);
+        if (forced) v = make_float4(v.x + gv.v[0], v.y + gv.v[1], v.z + gv.v[2], v.w + gv.v[3]);
+        *reinterpret_cast<float4*>(po) = v;
+        if (ysnap) __stcs(reinterpret_cast<float4*>(py), make_float4(u4.v[0], u4.v[1], u4.v[2], u4.v[3]));
       }
+      po += P.nxp;
+      py += P.nxp;
     }
+    const uint32_t t = prev;
+    prev = cur;
+    cur = next;
+    next = t;
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncwarp();
 }
 
-__global__ void __launch_bounds__(32 * kStreamWarps, 8) adr2d_stream_kernel(Stream2D P, const float* __restrict__ u,
-                                                                           const float* __restrict__ g,
-                                                                           float* __restrict__ out,
-                                                                           float* __restrict__ ysnap) {
-  __shared__ float4 ring[kStreamWarps][kRing][2][32];   // rows of u and g
-  __shared__ float4 rowc[kMaxRun + 16];                 // rows ya - 8 .. yb + 7: west, east, diagonal, north / south
-  __shared__ float rowt[kMaxRun + 16];                  // sponge depth of the row
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int run = blockIdx.y;
-  const int ya = run * P.run_rows, yb = min(P.ny, ya + P.run_rows);
-  // row coefficients of the run (constant over the march: read before the previous launch is waited for)
-  for (int e = threadIdx.x; e < yb - ya + 16; e += blockDim.x) {
-    const int j = ya - 8 + e;
-    float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
-    float t = 0.f;
-    if (j >= 0 && j < P.ny) {
-      const float ux = (P.adj ? -__ldg(P.U + j) : __ldg(P.U + j)) * P.i2dx;
-      c = make_float4(ux + P.nx2, P.nx2 - ux, -2.f * (P.nx2 + P.ny2) + __ldg(P.r + j), P.ny2);
-      const int d = min(j, P.ny - 1 - j);
-      t = d < P.sponge_cells ? (float)(P.sponge_cells - d) * P.sponge_inv : 0.f;
+__global__ void __launch_bounds__(32, kWarpsPerSm) adr2d_stream_kernel(Stream2D P, const float* __restrict__ u,
+                                                                      const float* __restrict__ g,
+                                                                      float* __restrict__ out,
+                                                                      float* __restrict__ ysnap) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x;
+  const uint32_t ring = (uint32_t)__cvta_generic_to_shared(smem_raw), rows = ring + kRingBytes;
+  float4* rowc = reinterpret_cast<float4*>(smem_raw + kRingBytes);
+  float* rowt = reinterpret_cast<float*>(rowc + 4 * (P.chunk + 16));
+  int64_t at = (int64_t)blockIdx.x * P.chunk;
+  const int64_t end = min(P.total, at + P.chunk);
+  bool waited = false;
+  while (at < end) {
+    const int col = (int)(at / P.ny);
+    const int ya = (int)(at - (int64_t)col * P.ny), yb = (int)min((int64_t)P.ny, ya + (end - at));
+    const int v = col % P.kg, strip = col / P.kg;
+    const int x0 = strip * kStripCells - 4, x1 = x0 + 128;   // the warp's cells
+    const int sc = max(P.sponge_cells, 0);
+    const bool wall = x0 < sc || x1 > P.nx - sc;
+    // row coefficients of the run (constant over the march: read before the previous launch is waited for)
+    for (int e = lane; e < yb - ya + 16; e += 32) {
+      const int j = ya - 8 + e;
+      float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
+      float t = 0.f;
+      if (j >= 0 && j < P.ny) {
+        const float ux = (P.adj ? -__ldg(P.U + j) : __ldg(P.U + j)) * P.i2dx;
+        const int d = min(j, P.ny - 1 - j);
+        t = d < P.sponge_cells ? (float)(P.sponge_cells - d) * P.sponge_inv : 0.f;
+        c = make_float4(ux + P.nx2, P.nx2 - ux, -2.f * (P.nx2 + P.ny2) + __ldg(P.r + j), P.ny2);
+        if (!wall) c.z -= P.sponge_amp * t * t;
+      }
+#pragma unroll
+      for (int st = 0; st < 4; ++st)
+        rowc[4 * e + st] = make_float4(P.f[st] * c.x, P.f[st] * c.y, P.f[st] * c.z, P.f[st] * c.w);
+      rowt[e] = t;
     }
-    rowc[e] = c;
-    rowt[e] = t;
-  }
-  __syncthreads();
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int item = blockIdx.x * kStreamWarps + warp;    // vector and strip
-  if (item >= P.strips * P.kg) return;
-  const int v = item % P.kg, strip = item / P.kg;
-  const int x0 = strip * kStripCells - 4, x1 = x0 + 128;   // the warp's cells
-  const int64_t base = (int64_t)v * P.vstride;
-  const int sc = max(P.sponge_cells, 0);
-  const bool wall = x0 < sc || x1 > P.nx - sc || ya - 4 < sc || yb + 4 > P.ny - sc;
-  if (wall)
-    stream2d_rows<true>(P, u, g, out, ysnap, ring[warp], rowc, rowt, ya, yb, x0 + 4 * lane, lane, base);
-  else
-    stream2d_rows<false>(P, u, g, out, ysnap, ring[warp], rowc, rowt, ya, yb, x0 + 4 * lane, lane, base);
-}
-
-// Rows per run: the run length with the least estimated time.  A row costs a warp about 450 cycles of
-// its own dependent chain, and the SM about 45 cycles of issue slots per resident warp (16 at most).
-int stream2d_run_rows(int items, int ny, int sms) {
-  int best = std::min(ny, kMaxRun);
-  double best_t = 1e300;
-  for (int runs = (ny + kMaxRun - 1) / kMaxRun; runs <= std::min(65535, std::max(1, ny / 4)); ++runs) {
-    const int rows = (ny + runs - 1) / runs;
-    const int nr = (ny + rows - 1) / rows;
-    const double warps = std::ceil((double)items * nr / std::max(1, sms));
-    const double t = (rows + 8) * std::max(450.0 * std::ceil(warps / 16.0), 45.0 * warps);
-    if (t < best_t) {
-      best_t = t;
-      best = rows;
+    __syncwarp();
+    if (!waited) {
+      asm volatile("griddepcontrol.wait;" ::: "memory");
+      asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+      waited = true;
     }
+    const int64_t base = (int64_t)v * P.vstride;
+    if (wall)
+      stream2d_rows<true>(P, u, g, out, ysnap, ring, rows, rowt, ya, yb, x0 + 4 * lane, lane, base);
+    else
+      stream2d_rows<false>(P, u, g, out, ysnap, ring, rows, rowt, ya, yb, x0 + 4 * lane, lane, base);
+    at += yb - ya;
   }
-  return best;
 }
 
 // ---------------------------------------------------------------------------
-// One stage per launch (FP64): out = u + f A x (+ g).  FP64 arithmetic bounds it: the constants come
-// ready from the host and a point costs six FP64 operations (seven in the sponge).
+// One stage per launch (FP64): out = u + f A x (+ g).  FP64 arithmetic bounds it (one warp instruction
+// per 19 cycles and SM), so the row coefficients times h / m come ready from a table built per march
+// tile: a point costs one addition and four multiply-adds, one more in the sponge and for the forcing.
 // ---------------------------------------------------------------------------
+template <typename R>
+struct RowTab {
+  R w, e, c, y;   // west, east, diagonal, north / south
+};
+
+// rows [4 stages][ny] of the table, then the sponge rates of the columns [nx] and of the rows [ny]
+template <typename R>
+__global__ void row_table_kernel(Grid3<R> g, bool adj, RowTab<R>* __restrict__ rows, R* __restrict__ sp) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  auto rate = [&](int d) {
+    if (d >= g.sponge_cells) return R(0);
+    const R t = R(g.sponge_cells - d) * g.sponge_inv;
+    return g.sponge_amp * t * t;
+  };
+  if (e < g.ny) {
+    const R ux = (adj ? -g.f0[e] : g.f0[e]) * g.i2dx;
+    for (int st = 0; st < 4; ++st) {
+      const R f = g.h / R(4 - st);
+      RowTab<R> t;
+      t.w = f * (ux + g.nx2);
+      t.e = f * (g.nx2 - ux);
+      t.c = f * (R(-2) * (g.nx2 + g.ny2) + g.f1[e]);
+      t.y = f * g.ny2;
+      rows[st * g.ny + e] = t;
+    }
+    sp[g.nx + e] = rate(min(e, g.ny - 1 - e));
+  }
+  if (e < g.nx) sp[e] = rate(min(e, g.nx - 1 - e));
+}
+
 template <typename R, bool LAST>
-__global__ void __launch_bounds__(128) adr2d_horner_kernel(Grid3<R> g, bool adj, const R* x, const R* u,
-                                                           const R* __restrict__ gf, R* out, R* __restrict__ ysnap,
-                                                           R f) {
+__global__ void __launch_bounds__(128) adr2d_horner_kernel(Grid3<R> g, const RowTab<R>* __restrict__ rows,
+                                                           const R* __restrict__ sp, R f, const R* x, const R* u,
+                                                           const R* __restrict__ gf, R* out, R* __restrict__ ysnap) {
   const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 4 + threadIdx.y;
-  const int64_t base = (int64_t)blockIdx.z * g.ncellp;
-  const bool in = i < g.nx && j < g.ny;
-  R cw = 0, ce = 0, cc = 0;
-  if (in) {   // constant over the march: read before the previous launch is waited for
-    const R ux = (adj ? -g.f0[j] : g.f0[j]) * g.i2dx;
-    cw = ux + g.nx2;
-    ce = g.nx2 - ux;
-    cc = R(-2) * (g.nx2 + g.ny2) + g.f1[j];
-    if (min(min(i, g.nx - 1 - i), min(j, g.ny - 1 - j)) < g.sponge_cells) cc -= sponge2d<R>(i, j, g);
-  }
+  const int64_t p = (int64_t)blockIdx.z * g.ncellp + (int64_t)j * g.nxp + i;
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (!in) return;
-  const int64_t p = base + (int64_t)j * g.nxp + i;
+  if (i >= g.nx || j >= g.ny) return;
+  const RowTab<R> t = rows[j];
   const R* q = x + p;
   const R c = q[0];
   const R w = i > 0 ? q[-1] : R(0), e = i < g.nx - 1 ? q[1] : R(0);
   const R s = j > 0 ? q[-g.nxp] : R(0), n = j < g.ny - 1 ? q[g.nxp] : R(0);
   const R u0 = u == x ? c : u[p];
-  R a = g.ny2 * (s + n);
-  a = fma(cw, w, a);
-  a = fma(ce, e, a);
-  a = fma(cc, c, a);
-  R o = fma(f, a, u0);
+  R cc = t.c;
+  const int dx = min(i, g.nx - 1 - i), dy = min(j, g.ny - 1 - j);
+  if (min(dx, dy) < g.sponge_cells) cc = fma(-f, sp[dx < dy ? i : g.nx + j], cc);   // the nearer wall's rate
+  R o = fma(t.y, s + n, u0);
+  o = fma(t.w, w, o);
+  o = fma(t.e, e, o);
+  o = fma(cc, c, o);
   if (LAST && gf != nullptr) o += gf[p];
   out[p] = o;
   if (ysnap != nullptr) ysnap[p] = u0;
 }
 
 template <typename F, typename... A>
-cudaError_t launch_pdl(F kernel, dim3 grid, dim3 block, cudaStream_t st, A... args) {
+cudaError_t launch_pdl(F kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -467,44 +505,50 @@ cudaError_t step_march_2d(rsv_operator op, const MarchTile& t, void* state, cons
     P.ny = g.ny;
     P.kg = t.kg;
     P.strips = (g.nx + kStripCells - 1) / kStripCells;
-    P.run_rows = stream2d_run_rows(P.strips * t.kg, g.ny, op->sm_count);
-    P.runs = (g.ny + P.run_rows - 1) / P.run_rows;
+    P.total = (int64_t)P.strips * t.kg * g.ny;
+    // one chunk per resident warp, of 4 rows at least (a run pays 8 rows for its start and end)
+    const int64_t warps = (int64_t)std::max(1, op->sm_count) * kWarpsPerSm;
+    P.chunk = (int)std::min<int64_t>(kMaxChunk, std::max<int64_t>(4, (P.total + warps - 1) / warps));
     P.vstride = g.ncellp;
     P.U = g.f0;
     P.r = g.f1;
     P.i2dx = g.i2dx;
     P.nx2 = g.nx2;
     P.ny2 = g.ny2;
-    P.h = g.h;
-    P.h2 = g.h / 2.f;
-    P.h3 = g.h / 3.f;
-    P.h4 = g.h / 4.f;
+    for (int m = 0; m < 4; ++m) P.f[m] = g.h / (float)(4 - m);
     P.sponge_cells = g.sponge_cells;
     P.sponge_amp = g.sponge_amp;
     P.sponge_inv = g.sponge_inv;
     P.adj = t.adjoint ? 1 : 0;
-    const dim3 grid((unsigned)((P.strips * t.kg + kStreamWarps - 1) / kStreamWarps), (unsigned)P.runs);
+    const unsigned blocks = (unsigned)((P.total + P.chunk - 1) / P.chunk);
     for (int s = 0; s < t.steps && e == cudaSuccess; ++s) {
       const float* gs = (G != nullptr && t.n0 + s < t.n_forced) ? static_cast<const float*>(G) + (size_t)s * rows : nullptr;
       float* ys = (Y != nullptr && s >= t.y_first) ? static_cast<float*>(Y) + (size_t)s * rows : nullptr;
-      e = launch_pdl(adr2d_stream_kernel, grid, dim3(32 * kStreamWarps), op->stream, P, (const float*)cur, gs, nxt, ys);
+      e = launch_pdl(adr2d_stream_kernel, dim3(blocks), dim3(32), stream2d_smem(P.chunk), op->stream, P, (const float*)cur, gs, nxt,
+                     ys);
       std::swap(cur, nxt);
     }
     if (e == cudaSuccess && cur != static_cast<R*>(state))
       e = cudaMemcpyAsync(state, cur, sizeof(R) * rows, cudaMemcpyDeviceToDevice, op->stream);
   } else {
     R* w = nxt + rows;
+    RowTab<R>* tab = reinterpret_cast<RowTab<R>*>(w + rows);
+    R* sp = reinterpret_cast<R*>(tab + 4 * (size_t)g.ny);
     const dim3 grid((unsigned)((g.nx + 31) / 32), (unsigned)((g.ny + 3) / 4), (unsigned)t.kg), block(32, 4);
+    row_table_kernel<R><<<(unsigned)((std::max(g.nx, g.ny) + 127) / 128), 128, 0, op->stream>>>(g, t.adjoint, tab, sp);
+    e = cudaGetLastError();
+    auto stage = [&](auto kernel, int st, const R* x, const R* u, const R* gs, R* o, R* ys) {
+      if (e == cudaSuccess)
+        e = launch_pdl(kernel, grid, block, 0, op->stream, g, (const RowTab<R>*)(tab + (size_t)st * g.ny), (const R*)sp,
+                       g.h / R(4 - st), x, u, gs, o, ys);
+    };
     for (int s = 0; s < t.steps && e == cudaSuccess; ++s) {
       const R* gs = (G != nullptr && t.n0 + s < t.n_forced) ? static_cast<const R*>(G) + (size_t)s * rows : nullptr;
       R* ys = (Y != nullptr && s >= t.y_first) ? static_cast<R*>(Y) + (size_t)s * rows : nullptr;
-      const R* none = nullptr;
-      R* nosnap = nullptr;
-      e = launch_pdl(adr2d_horner_kernel<R, false>, grid, block, op->stream, g, t.adjoint, (const R*)cur, (const R*)cur, none, nxt, ys, g.h / R(4));
-      if (e == cudaSuccess) e = launch_pdl(adr2d_horner_kernel<R, false>, grid, block, op->stream, g, t.adjoint, (const R*)nxt, (const R*)cur, none, w, nosnap, g.h / R(3));
-      if (e == cudaSuccess) e = launch_pdl(adr2d_horner_kernel<R, false>, grid, block, op->stream, g, t.adjoint, (const R*)w, (const R*)cur, none, nxt, nosnap, g.h / R(2));
-      // the last stage reads its own point of u only: in place
-      if (e == cudaSuccess) e = launch_pdl(adr2d_horner_kernel<R, true>, grid, block, op->stream, g, t.adjoint, (const R*)nxt, (const R*)cur, gs, cur, nosnap, g.h);
+      stage(adr2d_horner_kernel<R, false>, 0, cur, cur, nullptr, nxt, ys);
+      stage(adr2d_horner_kernel<R, false>, 1, nxt, cur, nullptr, w, nullptr);
+      stage(adr2d_horner_kernel<R, false>, 2, w, cur, nullptr, nxt, nullptr);
+      stage(adr2d_horner_kernel<R, true>, 3, nxt, cur, gs, cur, nullptr);   // reads its own point of u only: in place
     }
   }
   if (e == cudaSuccess) e = check_finite(op, state, rows, true);
