@@ -17,13 +17,13 @@ namespace {
 constexpr int kMaxK = 32;
 
 // One CTA per (frequency, instance, chunk of points).  The CTA stages the k vectors of 256 points at a
-// time in shared memory (each value read once from HBM).  The k x k Gram is Hermitian and cut into
+// time in shared memory (each value read once from HBM, the next slab in flight during the current one).  The k x k Gram is Hermitian and cut into
 // tiles of T x T pairs on and above the diagonal, one or a few per warp: a lane holds the T x T sums of
 // its points (every 32nd), so that 2 T loads feed T^2 complex multiply-adds.  The lanes' sums over a slab
 // (8 points each) are added up across the warp by a halving exchange that leaves one of the 2 T^2 values
 // per lane, which goes on in FP64 across the slabs.  One FP64 atomic per value and chunk.  k = 16, 4.2 M points, FP32: 0.22 ms (one pair per thread: 0.70).
 constexpr int kSlab = 256;
-constexpr int kSlabsPerCta = 16;
+constexpr int kSlabsPerCta = 8;
 constexpr int kGramWarps = 12;
 
 template <typename R>
@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(32 * kGramWarps) gram_kernel(const cpx<R>* __r
   constexpr int T = gram_tile<R>(), NV = 2 * T * T;
   constexpr int kMaxOwn = sizeof(R) == 4 ? 3 : 12;                 // tiles per warp at k = 32
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cpx<R>* xs = reinterpret_cast<cpx<R>*>(smem_raw);                // [kt T][kSlab], rows from k on zero
+  cpx<R>* slabs = reinterpret_cast<cpx<R>*>(smem_raw);             // [2][kt T][kSlab], rows from k on zero
   const int inst = blockIdx.y;
   const int j = blockIdx.z;
   const int64_t p0 = inst_off[inst], p1 = inst_off[inst + 1];
@@ -63,7 +63,26 @@ __global__ void __launch_bounds__(32 * kGramWarps) gram_kernel(const cpx<R>* __r
   const cpx<R>* Xj = X + (int64_t)j * k * n;
   const int kt = (k + T - 1) / T, tiles = kt * (kt + 1) / 2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int e = threadIdx.x; e < (kt * T - k) * kSlab; e += blockDim.x) xs[k * kSlab + e] = mk<R>(0, 0);
+  const int slab_len = kt * T * kSlab;
+  for (int e = threadIdx.x; e < (kt * T - k) * kSlab; e += blockDim.x)
+    slabs[k * kSlab + e] = slabs[slab_len + k * kSlab + e] = mk<R>(0, 0);
+  // asynchronous copies of slab sl into its buffer (zeros past the instance's end); nothing past the chunk
+  auto copy_slab = [&](int sl) {
+    const int64_t s0 = c0 + (int64_t)sl * kSlab;
+    if (sl < kSlabsPerCta && s0 < p1) {
+      const int cnt = (int)min((int64_t)kSlab, p1 - s0);
+      cpx<R>* dst = slabs + (sl & 1) * slab_len;
+      for (int e = threadIdx.x; e < k * kSlab; e += blockDim.x) {
+        const int a = e / kSlab, pp = e % kSlab;
+        const cpx<R>* src = Xj + (int64_t)a * n + s0 + (pp < cnt ? pp : 0);
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"((uint32_t)__cvta_generic_to_shared(dst + e)),
+                     "l"(src), "n"(sizeof(cpx<R>)), "r"(pp < cnt ? (int)sizeof(cpx<R>) : 0)
+                     : "memory");
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  copy_slab(0);
   // this warp's tiles warp, warp + nw, ...: rows ta, columns tb >= ta
   auto tile_of = [&](int t, int* ta, int* tb) {
     int a = 0;
@@ -78,12 +97,10 @@ __global__ void __launch_bounds__(32 * kGramWarps) gram_kernel(const cpx<R>* __r
     const int64_t s0 = c0 + (int64_t)sl * kSlab;
     if (s0 >= p1) break;
     const int cnt = (int)min((int64_t)kSlab, p1 - s0);
+    copy_slab(sl + 1);                                             // into the buffer read before the last barrier
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
     __syncthreads();
-    for (int e = threadIdx.x; e < k * kSlab; e += blockDim.x) {
-      const int a = e / kSlab, pp = e % kSlab;
-      xs[e] = pp < cnt ? Xj[(int64_t)a * n + s0 + pp] : mk<R>(0, 0);
-    }
-    __syncthreads();
+    const cpx<R>* xs = slabs + (sl & 1) * slab_len;
 #pragma unroll
     for (int q = 0; q < kMaxOwn; ++q) {
       const int t = warp + q * nw;
@@ -114,6 +131,7 @@ __global__ void __launch_bounds__(32 * kGramWarps) gram_kernel(const cpx<R>* __r
       }
       tot[q] += (double)warp_scatter_sum<NV>(v, lane);
     }
+    __syncthreads();
   }
   double* g = reinterpret_cast<double*>(G + ((int64_t)j * n_inst + inst) * k * k);
 #pragma unroll
@@ -188,7 +206,7 @@ cudaError_t launch_gram(const void* X, int n_omega, int k, int64_t n, const int6
   dim3 grid((unsigned)((max_len + per_cta - 1) / per_cta), (unsigned)n_inst, (unsigned)n_omega);
   constexpr int T = gram_tile<R>();
   const int kt = (k + T - 1) / T, tiles = kt * (kt + 1) / 2;
-  const size_t smem = sizeof(cpx<R>) * (size_t)kt * T * kSlab;
+  const size_t smem = 2 * sizeof(cpx<R>) * (size_t)kt * T * kSlab;
   if (smem > 48 * 1024) {
     e = cudaFuncSetAttribute(gram_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

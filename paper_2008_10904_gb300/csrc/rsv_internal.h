@@ -180,7 +180,7 @@ struct rsv_operator_s {
   void* tc_acc = nullptr;       // its FP32 partial-sum accumulators
   // stencil kinds: base-flow fields
   void* fld[8] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-  void* fldp[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};   // ADV3D, FP32: rows padded to 4 cells
+  void* fldp[4] = {nullptr, nullptr, nullptr, nullptr};   // ADV3D, FP32: rows padded to 4 cells
   double c_dx = 0, c_dy = 0, c_dz = 0;
   int nx = 0, ny = 0, nz = 0;
   double visc = 0;

@@ -1324,12 +1324,12 @@ rsv_status build_adv3d(rsv_operator op, const rsv_operator_desc* d) {
   }
   st = upload(op, il.data(), il.size() * sizeof(float), &op->fld[4]);
   const int nxp = (d->nx + 3) / 4 * 4;
-  for (int a = 0; a < 5; ++a) op->fldp[a] = op->fld[a];
+  for (int a = 0; a < 4; ++a) op->fldp[a] = op->fld[a];
   if (st != RSV_OK || nxp == d->nx) return st;
   // the step form's rows are padded to four cells (zeros)
   const size_t rows = (size_t)d->ny * d->nz;
-  for (int a = 0; a < 5; ++a) {
-    const size_t w = (a < 4 ? 1 : 4) * sizeof(float);
+  for (int a = 0; a < 4; ++a) {
+    const size_t w = sizeof(float);
     void* p = nullptr;
     cudaError_t e = cudaMalloc(&p, rows * nxp * w);
     if (e != cudaSuccess) return cuda_fail(e, "operator allocation");

@@ -53,6 +53,13 @@ __device__ __forceinline__ cpx<R> ld_or0(const cpx<R>* p, bool ok) {
   return ok ? *p : mk<R>(0, 0);
 }
 
+// a_j = c1 + cs s_j + cz z_j (one thread per block: the 64-bit remainders of the phases are slow)
+template <typename R>
+__device__ cpx<R> coef_factor(const cpx<R>* tw, int64_t p, int64_t m4, R c1, R cs, R cz) {
+  const cpx<R> s = tw[phase_index(p, 1, m4)], z = tw[phase_index(p, 2, m4)];
+  return mk<R>(c1 + cs * s.re + cz * z.re, cs * s.im + cz * z.im);
+}
+
 // One pass for the frequencies j0 .. j0 + gridDim.y - 1 and the vectors gridDim.z of a 2-D block:
 // out = scale (a_j f + B t), with a_j = (1, s_j, z_j) . coef.  f has the caller's layout (stride
 // f_stride per frequency), t and out the padded one.
@@ -62,16 +69,18 @@ __global__ void __launch_bounds__(256) coef2d_kernel(Grid3<R> g, int j0, const c
                                                      cpx<R>* __restrict__ out, int64_t o_stride,
                                                      const cpx<R>* __restrict__ tw, const int64_t* __restrict__ pj,
                                                      int sgn, int64_t m4, R c1, R cs, R cz, R bscale, R scale) {
+  __shared__ cpx<R> sa;
+  const int w = blockIdx.y, v = blockIdx.z;
+  if (threadIdx.x == 0) sa = coef_factor<R>(tw, sgn * pj[j0 + w], m4, c1, cs, cz);
+  __syncthreads();
+  const cpx<R> a = sa;
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) % g.nxp, j = (blockIdx.x * blockDim.x + threadIdx.x) / g.nxp;
   if (j >= g.ny) return;
-  const int w = blockIdx.y, v = blockIdx.z;
   cpx<R>* o = out + (int64_t)w * o_stride + (int64_t)v * g.ncellp + (int64_t)j * g.nxp + i;
   if (i >= g.nx) {
     *o = mk<R>(0, 0);
     return;
   }
-  const cpx<R> s = tw[phase_index(sgn * pj[j0 + w], 1, m4)], z = tw[phase_index(sgn * pj[j0 + w], 2, m4)];
-  const cpx<R> a = mk<R>(c1 + cs * s.re + cz * z.re, cs * s.im + cz * z.im);
   const cpx<R> fv = f[(int64_t)(j0 + w) * f_stride + (int64_t)v * g.ncell + (int64_t)j * g.nx + i];
   const int pitch = t_is_f ? g.nx : g.nxp;
   const cpx<R>* x = t_is_f ? f + (int64_t)(j0 + w) * f_stride + (int64_t)v * g.ncell
@@ -95,22 +104,23 @@ __global__ void __launch_bounds__(256) coef3d_kernel(Grid3<R> g, int j0, const c
                                                      cpx<R>* __restrict__ out, int64_t o_stride,
                                                      const cpx<R>* __restrict__ tw, const int64_t* __restrict__ pj,
                                                      int sgn, int64_t m4, R c1, R cs, R cz, R bscale, R scale) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int i = (int)(e % g.nxp);
-  const int64_t jk = e / g.nxp;
-  const int j = (int)(jk % g.ny), kz = (int)(jk / g.ny);
-  if (kz >= g.nz) return;
+  __shared__ cpx<R> sa;
   const int w = blockIdx.y, v = blockIdx.z;
+  if (threadIdx.x == 0) sa = coef_factor<R>(tw, sgn * pj[j0 + w], m4, c1, cs, cz);
+  __syncthreads();
+  const cpx<R> a = sa;
+  const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;   // a component's cells number less than 2^31
+  const unsigned jk = e / (unsigned)g.nxp;
+  const int i = (int)(e - jk * (unsigned)g.nxp), j = (int)(jk % (unsigned)g.ny), kz = (int)(jk / (unsigned)g.ny);
+  if (kz >= g.nz) return;
   cpx<R>* o = out + (int64_t)w * o_stride + (int64_t)v * 3 * g.ncellp + e;
   if (i >= g.nx) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) o[c * g.ncellp] = mk<R>(0, 0);
     return;
   }
-  const cpx<R> s = tw[phase_index(sgn * pj[j0 + w], 1, m4)], z = tw[phase_index(sgn * pj[j0 + w], 2, m4)];
-  const cpx<R> a = mk<R>(c1 + cs * s.re + cz * z.re, cs * s.im + cz * z.im);
   const cpx<R>* fv = f + (int64_t)(j0 + w) * f_stride + (int64_t)v * 3 * g.ncell;
-  const int64_t q = jk * g.nx + i;                       // cell in the fields and in f
+  const int64_t q = (int64_t)jk * g.nx + i;              // cell in the fields and in f
   const int64_t pitch = t_is_f ? g.nx : g.nxp, plane = pitch * g.ny, cells = t_is_f ? g.ncell : g.ncellp;
   const cpx<R>* x = (t_is_f ? fv : t + (int64_t)w * t_stride + (int64_t)v * 3 * g.ncellp) + (t_is_f ? q : e);
   const R Uc = g.f0[q], Uw = i > 0 ? g.f0[q - 1] : R(0), Ue = i < g.nx - 1 ? g.f0[q + 1] : R(0);

@@ -5,38 +5,46 @@
 //   half 2:  w3 = u + h/2 A w2   on the tile + 1 halo cell
 //            u' = u + h A w3 + g on the tile
 //
-// A CTA owns a 64 x 8 tile in (x, y) of one vector and a run of planes in z, and streams through z:
-// the first stage's input (u or w2) sits in a ring of four planes with two halo cells in x and y
-// (three in use, the next arriving by asynchronous copies), the first stage's result in a ring of
-// three planes with one halo cell.  At plane p the first stage is evaluated on plane p + 1 and the
-// second on plane p, one barrier apart.  Per step the state-sized arrays cross HBM six times (half 1:
-// u read, w2 written, plus the snapshot on analysed steps; half 2: w2, u and g read, u' written)
-// against eleven for the stage pairs with accumulator and forcing (stencil_kernels.cu).  Cells outside
-// the grid hold zero (homogeneous Dirichlet), in both rings.
+// A CTA owns a 64 x 12 tile in (x, y) of one vector and a run of planes in z, and streams through z.  A
+// thread owns four consecutive x cells of one row of every plane: its own column of the planes below, at
+// and above comes from registers, and only the y neighbours (16-byte loads) and the x neighbours at the
+// ends of shuffles come from shared memory.  Nine warps evaluate the first stage (18 groups x 16 rows with
+// the halo), six the second on the tile, two planes behind; the planes between them pass through a ring
+// of three, one barrier per plane.  All operands arrive by 16-byte asynchronous copies issued a plane
+// ahead; the base flow and u are copied once and read by both stages.  Both stages in the same threads
+// (nine warps at 168 registers) were bound by the latency of 2.25 warps per scheduler: 162 us per step at
+// 256 x 128 x 128; one cell per thread with scalar shared-memory operands took 143 us.
+//
+// Per step the state-sized arrays cross HBM six times (half 1: u read, w2 written, plus the snapshot on
+// analysed steps; half 2: w2, u and g read, u' written) against eleven for the stage pairs with
+// accumulator and forcing (stencil_kernels.cu).  Cells outside the grid hold zero (homogeneous Dirichlet).
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
-#include <mutex>
 
 #include "rsv_ops.h"
 
 namespace rsv {
 namespace {
 
-constexpr int kTX = 64, kTY = 8, kThreads = 256;
-constexpr int kUW = kTX + 8, kUH = kTY + 4;     // input ring: x from X0 - 4 (16-byte aligned), y halo 2
-constexpr int kXW = kTX + 2, kXH = kTY + 2;     // intermediate ring: halo 1
-constexpr int kUP = kUW * kUH, kXP = kXW * kXH;
-constexpr int kRow4 = kUW / 4;
-constexpr int kS1 = (kXP + kThreads - 1) / kThreads, kS2 = kTX * kTY / kThreads;
-constexpr size_t kSmem = sizeof(float) * (4 * 3 * (size_t)kUP + 3 * 3 * (size_t)kXP);
+constexpr int kTX = 64, kTY = 12;
+constexpr int kGX = kTX / 4 + 2, kRY = kTY + 4;   // groups of a row with the halo, rows with the halo
+constexpr int kT1 = kGX * kRY;                    // first-stage threads (288)
+constexpr int kT2 = kTX / 4 * kTY;                // second-stage threads (192)
+constexpr int kThreads = kT1 + kT2;
+constexpr int kMidRing = 3, kFlowRing = 4, kGRing = 2;
+constexpr int in_ring(bool second) { return second ? 3 : 5; }   // half 1's second stage reads u from it
+constexpr size_t half_smem(bool second) {
+  return sizeof(float4) * (kT1 * (size_t)(3 * in_ring(second) + 3 * kMidRing + 4 * kFlowRing + (second ? 3 * kFlowRing : 0)) +
+                           (second ? (size_t)kT2 * 3 * kGRing : 0));
+}
+static_assert(half_smem(true) <= 232448 && half_smem(false) <= 232448, "3-D rings exceed the shared memory of a CTA");
 
 struct Half3D {
   int nx, nxp, ny, nz, kg, zruns;
   int64_t vstride;            // 3 * nxp * ny * nz
   float cdx, nx2, ny2, nz2;   // 1 / (2 dx), visc / d^2
-  const float4* f4;           // base flow per cell: U, dU/dx, dU/dy, dU/dz (rows padded to nxp)
-  const float *U, *Ux, *Uy, *Uz;
+  const float *U, *Ux, *Uy, *Uz;   // base flow, rows padded to nxp
   const float* in;            // u (half 1) or w2 (half 2)
   const float* u;             // half 2: u
   const float* g;             // half 2: g_n (nullable)
@@ -45,68 +53,95 @@ struct Half3D {
   float f1, f2;               // factors of the two stages
 };
 
-// Base flow at one cell: forward advection uses U at the cell, the transposed one U at the x neighbours.
+struct V4 {
+  float v[4];
+};
+__device__ __forceinline__ V4 zero4() {
+  V4 o;
+  o.v[0] = o.v[1] = o.v[2] = o.v[3] = 0.f;
+  return o;
+}
+__device__ __forceinline__ V4 v4(float4 x) {
+  V4 o;
+  o.v[0] = x.x;
+  o.v[1] = x.y;
+  o.v[2] = x.z;
+  o.v[3] = x.w;
+  return o;
+}
+__device__ __forceinline__ float4 f4(const V4& x) { return make_float4(x.v[0], x.v[1], x.v[2], x.v[3]); }
+struct C3 {
+  V4 c[3];
+};
+// Base flow of a group: U with its two x neighbours (transposed advection), gradient.
 struct Flow {
-  float Uc, Uw, Ue, Ux, Uy, Uz;
+  V4 U, Ux, Uy, Uz;
+  float Ul, Ur;
 };
 
+// u0 + f A x of one group: below, centre and above in registers, rows so and no from shared memory, the
+// cells l and r beside the group.
 template <bool ADJ>
-__device__ __forceinline__ Flow load_flow(const Half3D& P, int q, int i, bool ok) {
-  Flow b;
-  if (!ADJ) {   // one 16-byte load of the interleaved fields (the transposed one measured slower so)
-    const float4 v = ok ? __ldg(P.f4 + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-    b.Uc = v.x;
-    b.Uw = b.Ue = 0.f;
-    b.Ux = v.y;
-    b.Uy = v.z;
-    b.Uz = v.w;
-    return b;
+__device__ __forceinline__ void stage3d(const Half3D& P, float f, const C3& xb, const C3& xc, const C3& xt,
+                                        const float4 so[3], const float4 no[3], const float l[3], const float r[3],
+                                        const Flow& w, const C3& u0, C3& o) {
+  const float fz = f * P.nz2, fy = f * P.ny2, fx = f * P.nx2, fc = f * P.cdx;
+  const float cc = -2.f * (fx + fy + fz);
+  float cw[4], ce[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    if (ADJ) {
+      cw[c] = fmaf(-fc, c == 0 ? w.Ul : w.U.v[c - 1], fx);
+      ce[c] = fmaf(fc, c == 3 ? w.Ur : w.U.v[c + 1], fx);
+    } else {
+      cw[c] = fmaf(fc, w.U.v[c], fx);
+      ce[c] = fmaf(-fc, w.U.v[c], fx);
+    }
   }
-  b.Uc = 0.f;
-  b.Uw = (ok && i > 0) ? __ldg(P.U + q - 1) : 0.f;
-  b.Ue = (ok && i < P.nx - 1) ? __ldg(P.U + q + 1) : 0.f;
-  b.Ux = ok ? __ldg(P.Ux + q) : 0.f;
-  b.Uy = ok ? __ldg(P.Uy + q) : 0.f;
-  b.Uz = ok ? __ldg(P.Uz + q) : 0.f;
-  return b;
-}
-
-// 7-point operator at index e of component planes with rows of width W (below, centre, above).
-template <bool ADJ, int W, int PLANE>
-__device__ __forceinline__ void op3d(const float* __restrict__ xb, const float* __restrict__ xc,
-                                     const float* __restrict__ xt, int e, const Flow& b, const Half3D& P, float k[3]) {
-  float cen[3];
-  const float cc = -2.f * (P.nx2 + P.ny2 + P.nz2);
-  const float cw = P.nx2 + P.cdx * (ADJ ? -b.Uw : b.Uc), ce = P.nx2 - P.cdx * (ADJ ? -b.Ue : b.Uc);
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const float* p = xc + c * PLANE;
-    cen[c] = p[e];
-    float a = P.nz2 * (xb[c * PLANE + e] + xt[c * PLANE + e]);
-    a = fmaf(P.ny2, p[e - W] + p[e + W], a);
-    a = fmaf(cw, p[e - 1], a);
-    a = fmaf(ce, p[e + 1], a);
-    k[c] = fmaf(cc, cen[c], a);
+    const V4 s = v4(so[c]), n = v4(no[c]);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      float a = fmaf(fz, xb.c[c].v[k] + xt.c[c].v[k], u0.c[c].v[k]);
+      a = fmaf(fy, s.v[k] + n.v[k], a);
+      a = fmaf(cw[k], k == 0 ? l[c] : xc.c[c].v[k - 1], a);
+      a = fmaf(ce[k], k == 3 ? r[c] : xc.c[c].v[k + 1], a);
+      o.c[c].v[k] = fmaf(cc, xc.c[c].v[k], a);
+    }
   }
-  if (ADJ) {
-    k[0] = fmaf(-b.Ux, cen[0], k[0]);
-    k[1] = fmaf(-b.Uy, cen[0], k[1]);
-    k[2] = fmaf(-b.Uz, cen[0], k[2]);
-  } else {
-    k[0] = fmaf(-b.Ux, cen[0], fmaf(-b.Uy, cen[1], fmaf(-b.Uz, cen[2], k[0])));
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (ADJ) {
+      const float fx0 = -f * xc.c[0].v[k];
+      o.c[0].v[k] = fmaf(w.Ux.v[k], fx0, o.c[0].v[k]);
+      o.c[1].v[k] = fmaf(w.Uy.v[k], fx0, o.c[1].v[k]);
+      o.c[2].v[k] = fmaf(w.Uz.v[k], fx0, o.c[2].v[k]);
+    } else {
+      const float d = fmaf(w.Ux.v[k], xc.c[0].v[k], fmaf(w.Uy.v[k], xc.c[1].v[k], w.Uz.v[k] * xc.c[2].v[k]));
+      o.c[0].v[k] = fmaf(-f, d, o.c[0].v[k]);
+    }
   }
 }
 
-__device__ __forceinline__ void cp16(float* dst, const float* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+// Copies 16 bytes, or writes zeros without reading.
+__device__ __forceinline__ void cp16_zfill(float4* dst, const float* src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src),
+               "r"(ok ? 16 : 0)
                : "memory");
 }
+__device__ __forceinline__ void plane_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(kThreads) : "memory"); }
 
 template <bool ADJ, bool SECOND>
-__global__ void __launch_bounds__(kThreads, 2) adv3d_half_kernel(Half3D P) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float* ring = reinterpret_cast<float*>(smem_raw);   // [4 planes][3 comps][kUP]
-  float* mid = ring + 4 * 3 * kUP;                      // [3 planes][3 comps][kXP]
+__global__ void __launch_bounds__(kThreads, 1) adv3d_half_kernel(Half3D P) {
+  constexpr int kIn = in_ring(SECOND);
+  extern __shared__ __align__(16) float4 smem_raw[];
+  // rings of planes, one slot per first-stage thread
+  float4 (*s_in)[3][kT1] = reinterpret_cast<float4 (*)[3][kT1]>(smem_raw);          // [kIn] input
+  float4 (*s_mid)[3][kT1] = s_in + kIn;                                             // [kMidRing] first stage's result
+  float4 (*s_w)[4][kT1] = reinterpret_cast<float4 (*)[4][kT1]>(s_mid + kMidRing);   // [kFlowRing] base flow
+  float4 (*s_u)[3][kT1] = reinterpret_cast<float4 (*)[3][kT1]>(s_w + kFlowRing);    // [kFlowRing] half 2: u
+  float4 (*s_g)[3][kT2] = reinterpret_cast<float4 (*)[3][kT2]>(s_u + kFlowRing);    // [kGRing] half 2: g
   const int nx = P.nx, ny = P.ny, nz = P.nz;
   const int plane = P.nxp * ny, ncell = plane * nz;
   int b = blockIdx.x;          // vector fastest: neighbouring tiles of all vectors in flight together
@@ -119,158 +154,193 @@ __global__ void __launch_bounds__(kThreads, 2) adv3d_half_kernel(Half3D P) {
   const int cz = b / nty;
   const int z0 = (int)((int64_t)cz * nz / P.zruns), z1 = (int)((int64_t)(cz + 1) * nz / P.zruns);
   const int64_t base = (int64_t)v * P.vstride;
-  const float* __restrict__ in = P.in + base;
-  const float* __restrict__ pu = SECOND ? P.u + base : nullptr;
-  const float* __restrict__ pg = SECOND && P.g ? P.g + base : nullptr;
-  float* __restrict__ out = P.out + base;
-  float* __restrict__ ysnap = !SECOND && P.ysnap ? P.ysnap + base : nullptr;
-  const int tid = threadIdx.x;
+  const bool second = threadIdx.x >= kT1;              // this thread's stage
+  const int t2 = threadIdx.x - kT1, lane = threadIdx.x & 31;
+  const int gx = second ? t2 % (kTX / 4) + 1 : threadIdx.x % kGX, ry = second ? t2 / (kTX / 4) + 2 : threadIdx.x / kGX;
+  const int at = ry * kGX + gx;                        // the group's slot in the planes
+  const int x = X0 - 4 + 4 * gx, y = Y0 - 2 + ry;
+  const bool in_xy = x >= 0 && x < P.nxp && y >= 0 && y < ny;
+  const int xy = in_xy ? y * P.nxp + x : 0;
+  bool cell[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) cell[c] = in_xy && x + c < nx;
+  const bool inner = X0 >= 4 && X0 + kTX + 4 <= nx && Y0 >= 2 && Y0 + kTY + 2 <= ny;   // no cell of the tile outside
   // launched as a programmatic dependent: resident early, waits here before any memory access
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-
-  // per-thread cells, fixed over the planes: (x, y) offset (-1 outside the grid), x index, ring index
-  int xy1[kS1], gi1[kS1], eu1[kS1];
+  auto in_z = [&](int kz) { return kz >= 0 && kz < nz; };
+  auto get3 = [&](const float4 (*s)[kT1]) -> C3 {
+    C3 r;
 #pragma unroll
-  for (int sl = 0; sl < kS1; ++sl) {
-    const int e = tid + sl * kThreads;
-    const int lx = e % kXW, ly = e / kXW;
-    const int gi = X0 - 1 + lx, gj = Y0 - 1 + ly;
-    const bool ok = e < kXP && gi >= 0 && gi < nx && gj >= 0 && gj < ny;
-    xy1[sl] = ok ? gj * P.nxp + gi : -1;
-    gi1[sl] = gi;
-    eu1[sl] = e < kXP ? (ly + 1) * kUW + lx + 3 : kUW + 3;   // a slot past the region evaluates the first cell
-  }
-  int xy2[kS2], gi2[kS2];
+    for (int c = 0; c < 3; ++c) r.c[c] = v4(s[c][at]);
+    return r;
+  };
+  auto get_w = [&](const float4 (*s)[kT1]) -> Flow {
+    Flow w;
+    w.U = v4(s[0][at]);
+    w.Ux = v4(s[1][at]);
+    w.Uy = v4(s[2][at]);
+    w.Uz = v4(s[3][at]);
+    w.Ul = w.Ur = 0.f;
+    return w;
+  };
+  // neighbours of the thread's group in plane s: rows beside it (row 0 and the last one: results unused) and
+  // cells beside it, from the neighbouring lanes where they hold them
+  const int up = ry + 1 < kRY ? at + kGX : at, dn = ry > 0 ? at - kGX : at;
+  const bool edge_l = second ? gx == 1 || lane == 0 : lane == 0, edge_r = second ? gx == kTX / 4 || lane == 31 : lane == 31;
+  auto around = [&](const float4 (*s)[kT1], const C3& xc, float4 so[3], float4 no[3], float l[3], float r[3]) {
 #pragma unroll
-  for (int sl = 0; sl < kS2; ++sl) {
-    const int e = tid + sl * kThreads;
-    const int gi = X0 + e % kTX, gj = Y0 + e / kTX;
-    xy2[sl] = (gi < nx && gj < ny) ? gj * P.nxp + gi : -1;
-    gi2[sl] = gi;
-  }
-
-  // plane kz of the input into ring slot kz & 3, 16-byte chunks wholly inside or outside the padded grid
-  auto load_plane = [&](int kz) {
-    float* dst = ring + (size_t)(kz & 3) * 3 * kUP;
-    const bool zin = kz >= 0 && kz < nz;
-    for (int e = tid; e < 3 * kUH * kRow4; e += kThreads) {
-      const int row = e / kRow4, ch = e - row * kRow4;
-      const int c = row / kUH, ly = row - c * kUH;
-      const int gj = Y0 - 2 + ly, gx = X0 - 4 + 4 * ch;
-      float* d = dst + c * kUP + ly * kUW + 4 * ch;
-      if (zin && gj >= 0 && gj < ny && gx >= 0 && gx < P.nxp)
-        cp16(d, in + c * ncell + kz * plane + gj * P.nxp + gx);
-      else
-        *reinterpret_cast<float4*>(d) = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int c = 0; c < 3; ++c) {
+      so[c] = s[c][dn];
+      no[c] = s[c][up];
+      l[c] = __shfl_up_sync(0xffffffffu, xc.c[c].v[3], 1);
+      r[c] = __shfl_down_sync(0xffffffffu, xc.c[c].v[0], 1);
+      if (edge_l) l[c] = at > 0 ? s[c][at - 1].w : 0.f;
+      if (edge_r) r[c] = at + 1 < kT1 ? s[c][at + 1].x : 0.f;
     }
+  };
+  const C3 zero = {{zero4(), zero4(), zero4()}};
+  // Iteration i = z0 - 1 .. z1 + 1: the first stage on plane i (to z1), the second on plane i - 2 (from z0).
+  // Ring slots of plane k: (k - z0 + 2) mod the ring's length, kept as running indices.
+  const int last = z1 + 1;
+  if (!second) {
+    const float* in = P.in + base + xy;
+    const float* pu = SECOND ? P.u + base + xy : nullptr;
+    auto copy3 = [&](float4 (*s)[kT1], const float* p, int kz, bool ok) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) cp16_zfill(&s[c][at], ok ? p + c * ncell + kz * plane : P.in, ok);
+    };
+    auto copy_in = [&](int kz, int slot) { copy3(s_in[slot], in, kz, in_xy && in_z(kz) && kz <= z1 + 1); };
+    auto copy_wu = [&](int kz, int slot) {
+      const bool ok = in_xy && in_z(kz) && kz <= z1;
+      const int64_t q = ok ? kz * plane + xy : 0;
+      cp16_zfill(&s_w[slot][0][at], P.U + q, ok);
+      cp16_zfill(&s_w[slot][1][at], P.Ux + q, ok);
+      cp16_zfill(&s_w[slot][2][at], P.Uy + q, ok);
+      cp16_zfill(&s_w[slot][3][at], P.Uz + q, ok);
+      if (SECOND) copy3(s_u[slot], pu, kz, ok);
+    };
+    // planes z0 - 2 .. z0 of the input and plane z0 - 1 of the rest; slot of plane z0 - 2 + k is k
+    copy_in(z0 - 2, 0);
+    copy_in(z0 - 1, 1);
+    copy_in(z0, 2);
+    copy_wu(z0 - 1, 1);
     asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  struct In1 {
-    float u[kS1][3];
-    Flow b[kS1];
-  };
-  struct In2 {
-    float u[kS2][3], g[kS2][3];
-    Flow b[kS2];
-  };
-  auto fetch1 = [&](int kz, In1& r) {
-    const bool zin = kz >= 0 && kz < nz;
-#pragma unroll
-    for (int sl = 0; sl < kS1; ++sl) {
-      const bool ok = zin && xy1[sl] >= 0;
-      const int q = kz * plane + xy1[sl];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) r.u[sl][c] = (SECOND && ok) ? __ldg(pu + q + c * ncell) : 0.f;
-      r.b[sl] = load_flow<ADJ>(P, q, gi1[sl], ok);
-    }
-  };
-  auto fetch2 = [&](int kz, In2& r) {
-    const bool zin = kz >= z0 && kz < z1;
-#pragma unroll
-    for (int sl = 0; sl < kS2; ++sl) {
-      const bool ok = zin && xy2[sl] >= 0;
-      const int q = kz * plane + xy2[sl];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        r.u[sl][c] = (SECOND && ok) ? __ldg(pu + q + c * ncell) : 0.f;
-        r.g[sl][c] = (SECOND && ok && pg) ? __ldcs(pg + q + c * ncell) : 0.f;
-      }
-      r.b[sl] = load_flow<ADJ>(P, q, gi2[sl], ok);
-    }
-  };
-  // first stage on plane kz, tile + 1 halo cell, as one straight-line block masked afterwards
-  auto first_stage = [&](int kz, const In1& r) {
-    float* dst = mid + (size_t)(((kz % 3) + 3) % 3) * 3 * kXP;
-    const float* xb = ring + (size_t)((kz - 1) & 3) * 3 * kUP;
-    const float* xc = ring + (size_t)(kz & 3) * 3 * kUP;
-    const float* xt = ring + (size_t)((kz + 1) & 3) * 3 * kUP;
-    const bool zin = kz >= 0 && kz < nz;
-#pragma unroll
-    for (int sl = 0; sl < kS1; ++sl) {
-      const int e = tid + sl * kThreads;
-      const bool ok = zin && xy1[sl] >= 0;
-      float k[3];
-      op3d<ADJ, kUW, kUP>(xb, xc, xt, eu1[sl], r.b[sl], P, k);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const float uu = SECOND ? r.u[sl][c] : xc[c * kUP + eu1[sl]];
-        const float o = ok ? fmaf(P.f1, k[c], uu) : 0.f;
-        if (e < kXP) dst[c * kXP + e] = o;
-      }
-    }
-  };
-  // second stage on plane kz, the tile: every slot is evaluated, only the stores are masked
-  auto second_stage = [&](int kz, const In2& r) {
-    const float* mb = mid + (size_t)((((kz - 1) % 3) + 3) % 3) * 3 * kXP;
-    const float* mc = mid + (size_t)(kz % 3) * 3 * kXP;
-    const float* mt = mid + (size_t)((kz + 1) % 3) * 3 * kXP;
-    const float* uc = ring + (size_t)(kz & 3) * 3 * kUP;
-#pragma unroll
-    for (int sl = 0; sl < kS2; ++sl) {
-      const int e = tid + sl * kThreads;
-      const int tx = e % kTX, ty = e / kTX;
-      const int q = kz * plane + xy2[sl];
-      float k[3];
-      op3d<ADJ, kXW, kXP>(mb, mc, mt, (ty + 1) * kXW + tx + 1, r.b[sl], P, k);
-      if (xy2[sl] < 0) continue;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const float uu = SECOND ? r.u[sl][c] : uc[c * kUP + (ty + 2) * kUW + tx + 4];
-        float o = fmaf(P.f2, k[c], uu);
-        if (SECOND) o += r.g[sl][c];
-        out[q + c * ncell] = o;
-        if (!SECOND && ysnap) __stcs(ysnap + q + c * ncell, uu);
-      }
-    }
-  };
-
-  In1 s1;
-  In2 s2;
-  for (int kz = z0 - 2; kz <= z0 + 1; ++kz) load_plane(kz);
-  fetch1(z0 - 1, s1);
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
-  __syncthreads();
-  first_stage(z0 - 1, s1);
-  fetch1(z0, s1);
-  fetch2(z0, s2);
-  for (int p = z0 - 1; p < z1; ++p) {
-    // plane p + 2 has landed; the slot of plane p - 1 is free and receives plane p + 3
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncthreads();
-    if (p + 3 <= z1 + 1) load_plane(p + 3);
-    first_stage(p + 1, s1);
-    if (p + 2 <= z1) fetch1(p + 2, s1);   // in flight during the barrier and the second stage
-    __syncthreads();
-    if (p >= z0) {
-      second_stage(p, s2);
-      if (p + 1 < z1) fetch2(p + 1, s2);
+    C3 xin[3];
+    xin[0] = get3(s_in[0]);
+    xin[1] = get3(s_in[1]);
+    plane_barrier();
+    int si = 1, sm = 1, sw = 1;    // slots of plane i in the input, result and flow rings
+    for (int i0 = z0 - 1; i0 <= last; i0 += 3) {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const int i = i0 + q;        // planes i - 1, i, i + 1 in xin[q], xin[q + 1], xin[q + 2]
+        if (i > last) break;
+        if (i <= z1) {
+          asm volatile("cp.async.wait_group 0;" ::: "memory");
+          const int sn = si + 1 < kIn ? si + 1 : 0, sn2 = sn + 1 < kIn ? sn + 1 : 0;   // planes i + 1, i + 2
+          const int wn = sw + 1 < kFlowRing ? sw + 1 : 0;
+          xin[(q + 2) % 3] = get3(s_in[sn]);
+          copy_in(i + 2, sn2);
+          copy_wu(i + 1, wn);
+          asm volatile("cp.async.commit_group;" ::: "memory");
+          const C3& c = xin[(q + 1) % 3];
+          float4 so[3], no[3];
+          float l[3], r[3];
+          around(s_in[si], c, so, no, l, r);
+          C3 o;
+          Flow w = get_w(s_w[sw]);
+          if (ADJ) {   // U of the x neighbours: this plane's copies of other warps may still be on their way
+            w.Ul = __shfl_up_sync(0xffffffffu, w.U.v[3], 1);
+            w.Ur = __shfl_down_sync(0xffffffffu, w.U.v[0], 1);
+            const bool ok = in_xy && in_z(i);
+            if (lane == 0) w.Ul = ok && x > 0 ? __ldg(P.U + i * plane + xy - 1) : 0.f;
+            if (lane == 31) w.Ur = ok && x + 4 < P.nxp ? __ldg(P.U + i * plane + xy + 4) : 0.f;
+          }
+          stage3d<ADJ>(P, P.f1, xin[q], c, xin[(q + 2) % 3], so, no, l, r, w, SECOND ? get3(s_u[sw]) : c, o);
+          if (!inner || !in_z(i)) {
+            const bool zin = in_z(i);
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) o.c[k].v[e] = zin && cell[e] ? o.c[k].v[e] : 0.f;
+          }
+#pragma unroll
+          for (int k = 0; k < 3; ++k) s_mid[sm][k][at] = f4(o.c[k]);
+          si = sn;
+          sw = wn;
+          sm = sm + 1 < kMidRing ? sm + 1 : 0;
+        }
+        plane_barrier();
+      }
+    }
+  } else {
+    float* out = P.out + base + xy;
+    float* ysnap = !SECOND && P.ysnap ? P.ysnap + base + xy : nullptr;
+    const float* pg = SECOND && P.g ? P.g + base + xy : nullptr;
+    auto copy_g = [&](int kz) {
+      if (SECOND) {
+        const bool ok = in_xy && pg != nullptr && kz >= z0 && kz < z1;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) cp16_zfill(&s_g[kz & 1][c][t2], ok ? pg + c * ncell + kz * plane : P.in, ok);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    copy_g(z0);
+    C3 mid[3] = {zero, zero, zero};
+    plane_barrier();
+    // slots of plane i - 2 in the result, flow and input rings, of plane i - 1 in the result ring
+    int sm = kMidRing - 1, sw = kFlowRing - 1, si = kIn - 1;
+    for (int i0 = z0 - 1; i0 <= last; i0 += 3) {
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        const int i = i0 + q;        // planes i - 3, i - 2, i - 1 of the first stage's result in mid[q], mid[q + 1], mid[q + 2]
+        if (i > last) break;
+        const int sm1 = sm + 1 < kMidRing ? sm + 1 : 0;
+        if (i >= z0) mid[(q + 2) % 3] = get3(s_mid[sm1]);
+        const int k2 = i - 2;
+        if (k2 >= z0) {
+          asm volatile("cp.async.wait_group 0;" ::: "memory");
+          const C3& c = mid[(q + 1) % 3];
+          float4 so[3], no[3];
+          float l[3], r[3];
+          around(s_mid[sm], c, so, no, l, r);
+          const C3 u0 = SECOND ? get3(s_u[sw]) : get3(s_in[si]);
+          C3 o;
+          Flow w = get_w(s_w[sw]);
+          if (ADJ) {
+            w.Ul = s_w[sw][0][at - 1].w;
+            w.Ur = s_w[sw][0][at + 1].x;
+          }
+          stage3d<ADJ>(P, P.f2, mid[q], c, mid[(q + 2) % 3], so, no, l, r, w, u0, o);
+          if (in_xy) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+              V4 gv = zero4();
+              if (SECOND) gv = v4(s_g[k2 & 1][k][t2]);
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                if (SECOND) o.c[k].v[e] += gv.v[e];
+                if (!inner) o.c[k].v[e] = cell[e] ? o.c[k].v[e] : 0.f;
+              }
+              *reinterpret_cast<float4*>(out + k * ncell + k2 * plane) = f4(o.c[k]);
+              if (!SECOND && ysnap) __stcs(reinterpret_cast<float4*>(ysnap + k * ncell + k2 * plane), f4(u0.c[k]));
+            }
+          }
+          copy_g(k2 + 1);
+        }
+        sm = sm1;
+        sw = sw + 1 < kFlowRing ? sw + 1 : 0;
+        si = si + 1 < kIn ? si + 1 : 0;
+        plane_barrier();
+      }
     }
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-// Runs in z: as many CTAs as fill whole waves of the resident CTAs (runs of at least 4 planes).
+// Runs in z for the least planes of work on one SM (one CTA each), runs of at least 4 planes.
 int zruns_for(int per_run, int nz, int resident) {
   int best = 1;
   double best_t = 1e300;
@@ -286,35 +356,16 @@ int zruns_for(int per_run, int nz, int resident) {
 }
 
 template <bool ADJ, bool SECOND>
-cudaError_t launch_half(rsv_operator op, Half3D P) {
-  // the shared-memory opt-in and the residency are per device, set up once under a lock
-  static std::mutex mu;
-  static int resident_dev[64] = {0};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  int resident = 0;
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    if (dev < 0 || dev >= 64 || resident_dev[dev] == 0) {
-      cudaError_t e = cudaFuncSetAttribute(adv3d_half_kernel<ADJ, SECOND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)kSmem);
-      int per_sm = 0;
-      if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, adv3d_half_kernel<ADJ, SECOND>, kThreads, kSmem);
-      if (e != cudaSuccess) return e;
-      resident = std::max(1, per_sm) * std::max(1, op->sm_count);
-      if (dev >= 0 && dev < 64) resident_dev[dev] = resident;
-    } else {
-      resident = resident_dev[dev];
-    }
-  }
+cudaError_t launch_half(rsv_operator op, const Half3D& P) {
   const int ntx = (P.nx + kTX - 1) / kTX, nty = (P.ny + kTY - 1) / kTY;
-  { const char* zr = getenv("RSV_ZR"); P.zruns = zr ? atoi(zr) : zruns_for(ntx * nty * P.kg, P.nz, resident); }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(ntx * nty) * (unsigned)P.zruns * (unsigned)P.kg);
   cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kSmem;
+  cfg.dynamicSmemBytes = half_smem(SECOND);
   cfg.stream = op->stream;
+  cudaError_t e = cudaFuncSetAttribute(adv3d_half_kernel<ADJ, SECOND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)half_smem(SECOND));
+  if (e != cudaSuccess) return e;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -339,11 +390,11 @@ cudaError_t step_march_3d(rsv_operator op, const MarchTile& t, void* state, cons
   P.nx2 = nu * (1.f / (dx * dx));
   P.ny2 = nu * (1.f / (dy * dy));
   P.nz2 = nu * (1.f / (dz * dz));
-  P.f4 = (const float4*)op->fldp[4];
   P.U = (const float*)op->fldp[0];
   P.Ux = (const float*)op->fldp[1];
   P.Uy = (const float*)op->fldp[2];
   P.Uz = (const float*)op->fldp[3];
+  P.zruns = zruns_for(((P.nx + kTX - 1) / kTX) * ((P.ny + kTY - 1) / kTY) * P.kg, P.nz, std::max(1, op->sm_count));
   const int64_t rows = (int64_t)t.kg * P.vstride;
   float* cur = static_cast<float*>(state);
   float* nxt = cur + rows;

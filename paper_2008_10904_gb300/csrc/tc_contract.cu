@@ -381,9 +381,42 @@ __device__ __forceinline__ void convert_row(const ContractArgs& a, int64_t r0, i
   }
 }
 
-// Accumulator columns [c0, c1) of row r (output columns coff + c): F stores, or FP64
-// accumulator read-modify-writes, 32 columns per tensor-memory load, all loads of a
-// group issued before use.
+// FP32 -> FP64 with integer instructions (exact for zero and normal values).  FP64 instructions issue once
+// per 19 cycles and SM, conversions among them, and the accumulation needs one FP64 addition per value
+// anyway: converting there as well held the FP64 pipe 48% busy and the epilogue at twice its loads' time.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x), m = u & 0x7fffffffu;
+  const uint32_t hi = m < 0x00800000u ? 0u : (m >> 3) + 0x38000000u;
+  return __hiloint2double((int)(hi | (u & 0x80000000u)), m < 0x00800000u ? 0 : (int)(u << 29));
+}
+
+// FP64 accumulators of 16 output columns from column c on (8 frequencies) of row r.
+__device__ __forceinline__ void load_acc16(const ContractArgs& a, int64_t r, int c, double2 old[8]) {
+  const double2* acc = reinterpret_cast<const double2*>(a.out);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int j = (c >> 1) + q;
+    old[q] = (r < a.rows && j < a.n_omega) ? __ldcs(acc + (int64_t)j * a.acc_stride + r) : make_double2(0.0, 0.0);
+  }
+}
+// += v, the columns' sums over the tile.
+__device__ __forceinline__ void add_acc16(const ContractArgs& a, int64_t r, int c, const double2 old[8], const float v[16]) {
+  if (r >= a.rows) return;
+  uint32_t top = 0;
+#pragma unroll
+  for (int q = 0; q < 16; ++q) top = max(top, __float_as_uint(v[q]) & 0x7fffffffu);
+  double2* acc = reinterpret_cast<double2*>(a.out);
+  const bool plain = top < 0x7f800000u;   // no infinity and no NaN
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int j = (c >> 1) + q;
+    if (j >= a.n_omega) continue;
+    const double re = plain ? widen(v[2 * q]) : (double)v[2 * q], im = plain ? widen(v[2 * q + 1]) : (double)v[2 * q + 1];
+    __stcs(acc + (int64_t)j * a.acc_stride + r, make_double2(old[q].x + re, old[q].y + im));
+  }
+}
+
+// Accumulator columns [c0, c1) of row r (output columns coff + c) to F, 32 columns per tensor-memory load.
 template <int W>
 __device__ __forceinline__ void epilogue_cols(const ContractArgs& a, int64_t r, uint32_t tq, int cl, int coff,
                                               bool row_ok) {
@@ -405,21 +438,6 @@ __device__ __forceinline__ void epilogue_cols(const ContractArgs& a, int64_t r, 
     for (int q = 0; q < W; ++q) {
       const int tau = c + q;
       if (tau < a.n_tau) __stcs(F + (int64_t)(a.tau0 + tau) * a.rows + r, v[q]);
-    }
-  } else {
-    double2* __restrict__ acc = reinterpret_cast<double2*>(a.out);
-    double2 old[W / 2];
-#pragma unroll
-    for (int q = 0; q < W / 2; ++q) {
-      const int j = (c >> 1) + q;
-      old[q] = j < a.n_omega ? __ldcs(acc + (int64_t)j * a.acc_stride + r) : make_double2(0.0, 0.0);
-    }
-#pragma unroll
-    for (int q = 0; q < W / 2; ++q) {
-      const int j = (c >> 1) + q;
-      if (j < a.n_omega)
-        __stcs(acc + (int64_t)j * a.acc_stride + r,
-               make_double2(old[q].x + (double)v[2 * q], old[q].y + (double)v[2 * q + 1]));
     }
   }
 }
@@ -600,18 +618,54 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(Contr
     if (!ok) pabort(pb, a.err);
   } else if (warp >= 4 && warp < 12) {  // epilogue: TMEM lane quadrant warp % 4, one half of the columns
     const int q = warp & 3;
+    const bool anal = a.mode == ANAL_C || a.mode == ANAL_R;
     uint32_t tt = 0;
     bool ok = true;
+    // first column of this warp's half and one past its last in column sub-tile h
+    auto half_cols = [&](int h, int* c0, int* c1) {
+      const int nn = h == 0 ? min(256, a.N) : a.N - 256;
+      const int half = round16c((nn + 1) / 2);
+      *c0 = warp < 8 ? 0 : half;
+      *c1 = warp < 8 ? half : nn;
+    };
+    // analysis: the accumulators of the next 16 columns, of this tile or the next one, are in flight while
+    // the current ones are added to and while the tile's products are waited for
+    double2 nxt[8];
+    if (anal) {
+      int c0, c1;
+      half_cols(0, &c0, &c1);
+      if (c0 < c1) load_acc16(a, (int64_t)blockIdx.x * kRowsCta + 32 * q + lane, c0, nxt);
+    }
     for (int64_t t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
       for (int h = 0; h < nsub; ++h, ++tt) {
         const uint32_t buf = tt & 1;
         if (!pwait(&pb->acc_full[buf], (tt >> 1) & 1, abort_flag)) { ok = false; break; }
         tc::tc_fence_after();
-        const int nn = h == 0 ? min(256, a.N) : a.N - 256;
-        const int half = round16c((nn + 1) / 2);
-        const int c0 = warp < 8 ? 0 : half, c1 = warp < 8 ? half : nn;
-        epilogue_tile(a, t * kRowsCta + 32 * q + lane, tmem + ((uint32_t)(32 * q) << 16) + buf * 256u, c0, c1,
-                      256 * h);
+        int c0, c1;
+        half_cols(h, &c0, &c1);
+        const int64_t r = t * kRowsCta + 32 * q + lane;
+        const uint32_t tq = tmem + ((uint32_t)(32 * q) << 16) + buf * 256u;
+        if (anal) {
+          for (int c = c0; c < c1; c += 16) {
+            double2 old[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) old[i] = nxt[i];
+            if (c + 16 < c1) {
+              load_acc16(a, r, 256 * h + c + 16, nxt);
+            } else {
+              int hn = h + 1, n0 = 0, n1 = 0;
+              if (hn < nsub) half_cols(hn, &n0, &n1);
+              const bool same = n0 < n1;   // the next sub-tile of this tile has columns for this warp
+              if (!same) half_cols(hn = 0, &n0, &n1);
+              load_acc16(a, same ? r : r + (int64_t)gridDim.x * kRowsCta, 256 * hn + n0, nxt);
+            }
+            float v[16];
+            tc::tmem_ld16(tq + (uint32_t)c, v);
+            add_acc16(a, r, 256 * h + c, old, v);
+          }
+        } else {
+          epilogue_tile(a, r, tq, c0, c1, 256 * h);
+        }
         tc::tc_fence_before();
         mbar_arrive(&pb->acc_empty[buf]);
       }
