@@ -18,6 +18,7 @@
 // MMAs (3 per K-step: hi*hi, hi*lo, lo*hi).  The epilogue reads tensor memory
 // (one row per thread) and writes F, or adds the tile's sums into the FP64
 // accumulators.  Waits are bounded; a timeout sets the error flag.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -257,9 +258,9 @@ __global__ void __launch_bounds__(256, 1) tc_contract_kernel(ContractArgs a) {
 //
 // One CTA per SM walks the 128-row tiles blockIdx.x, blockIdx.x + gridDim.x, ...
 // with warp roles connected by mbarrier rings:
-//   warp 12              producer: bulk-copies each K chunk of the long operand
-//                        in its storage precision into an 8-deep raw ring, one
-//                        row slice per lane;
+//   warp 12 (one thread) producer: copies each K chunk of the long operand in its
+//                        storage precision into an 8-deep raw ring, one tensor
+//                        copy per chunk;
 //   warp 14 (one thread) producer: bulk-copies the chunk's pre-split twiddles
 //                        into a 2-deep B ring;
 //   warps 0-3            converters: one row each, raw value -> TF32 hi / lo in
@@ -316,64 +317,59 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
 }
 
-// Raw layout of one chunk in shared memory: complex modes [8][128] float2
-// (pair index jj = frequency or step within the chunk), real analysis
-// [16][128] float.  Only the valid pair indices and rows are copied.  Called by the whole warp: lane l
-// issues the copy of pair index l (one thread issuing all 8 or 16 bounded the kernel's chunk rate).
-__device__ __forceinline__ void issue_raw(const ContractArgs& a, int64_t r0, int nr, int kc, unsigned char* raw,
-                                          uint64_t* bar, int lane) {
+// Raw layout of one chunk in shared memory: complex modes [8][128] float2 (pair index jj = frequency or
+// step within the chunk), real analysis [16][128] float: one box of the tensor map, 8 KB.  Rows and pair
+// indices outside the operand come as zeros; snapshots of steps that are not analysed are masked by the
+// converters.  (Row slices by single bulk copies of 512 or 1024 bytes took about 94 cycles each, 1500 per
+// chunk, and bounded the analysis: 54 ms of the 2-D 1024 x 512 x 16 march.)
+__device__ __forceinline__ void issue_raw(const ContractArgs& a, const CUtensorMap* map, int64_t r0, int kc,
+                                          unsigned char* raw, uint64_t* bar) {
   const bool real = a.mode == ANAL_R;
-  const int npair = real ? kKc : kKc / 2;
-  const uint32_t esz = real ? 4 : 8;
-  int lo = kc * npair, hi = lo + npair;
-  if (a.mode == ANAL_C || a.mode == ANAL_R) {
-    lo = max(lo, a.s0);
-    hi = min(hi, a.s1);
-  } else {
-    hi = min(hi, a.n_omega);
-  }
-  const uint32_t bytes_row = (uint32_t)nr * esz;
-  const uint32_t total = hi > lo ? (uint32_t)(hi - lo) * bytes_row : 0u;
-  if (lane == 0) tc::mbar_arrive_expect_tx(bar, total);
-  __syncwarp();
-  const int64_t stride = (a.mode == ANAL_C || a.mode == ANAL_R) ? a.rows : a.src_stride;
-  const int idx = lo + lane;
-  if (idx < hi) {
-    const unsigned char* src = reinterpret_cast<const unsigned char*>(a.src) + ((int64_t)idx * stride + r0) * esz;
-    tc::bulk_g2s(raw + (uint32_t)(idx - kc * npair) * kRowsCta * esz, src, bytes_row, bar);
-  }
+  tc::mbar_arrive_expect_tx(bar, kRawBytes);
+  tc::tensor_g2s(raw, map, (int32_t)(real ? r0 : 2 * r0), kc * (real ? kKc : kKc / 2), bar);
 }
 
-__device__ __forceinline__ void convert_row(const ContractArgs& a, int64_t r0, int kc, int rr, const unsigned char* raw,
+// FP32 -> TF32, round to nearest with ties away from zero, as to_tf32 (integer instructions; a NaN's
+// remainder x - hi is NaN still).
+__device__ __forceinline__ float tf32_hi(float x) { return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u); }
+
+// One row of a chunk.  A warp converts a chunk per scheduler, so its instruction count is the chunk's time:
+// chunks that are valid as a whole take no test per value.
+__device__ __forceinline__ void convert_row(const ContractArgs& a, bool row_ok, int kc, int rr, const unsigned char* raw,
                                             float* A_hi, float* A_lo) {
-  const bool row_ok = r0 + rr < a.rows;
   float x[kKc];
   if (a.mode == ANAL_R) {
-    const float* rv = reinterpret_cast<const float*>(raw);
+    const float* rv = reinterpret_cast<const float*>(raw) + rr;
+    const int s = kc * kKc;
 #pragma unroll
-    for (int kk = 0; kk < kKc; ++kk) {
-      const int s = kc * kKc + kk;
-      x[kk] = (row_ok && s >= a.s0 && s < a.s1) ? rv[kk * kRowsCta + rr] : 0.f;
+    for (int kk = 0; kk < kKc; ++kk) x[kk] = rv[kk * kRowsCta];
+    if (!(row_ok && s >= a.s0 && s + kKc <= a.s1)) {
+#pragma unroll
+      for (int kk = 0; kk < kKc; ++kk) x[kk] = (row_ok && s + kk >= a.s0 && s + kk < a.s1) ? x[kk] : 0.f;
     }
   } else {
-    const float2* rv = reinterpret_cast<const float2*>(raw);
+    const float2* rv = reinterpret_cast<const float2*>(raw) + rr;
+    const int idx = kc * (kKc / 2);
+    const int lo = a.mode == ANAL_C ? a.s0 : 0, hi = a.mode == ANAL_C ? a.s1 : a.n_omega;
 #pragma unroll
     for (int jj = 0; jj < kKc / 2; ++jj) {
-      const int idx = kc * (kKc / 2) + jj;
-      const bool v = row_ok && ((a.mode == ANAL_C) ? (idx >= a.s0 && idx < a.s1) : (idx < a.n_omega));
-      const float2 c = v ? rv[jj * kRowsCta + rr] : make_float2(0.f, 0.f);
+      const float2 c = rv[jj * kRowsCta];
       x[2 * jj] = c.x;
       x[2 * jj + 1] = c.y;
+    }
+    if (!(row_ok && idx >= lo && idx + kKc / 2 <= hi)) {
+#pragma unroll
+      for (int k = 0; k < kKc; ++k) x[k] = (row_ok && idx + k / 2 >= lo && idx + k / 2 < hi) ? x[k] : 0.f;
     }
   }
   // K-major core matrices: 4 consecutive K values of one row are one 16-byte vector
 #pragma unroll
   for (int q = 0; q < kKc / 4; ++q) {
     float4 h, l;
-    h.x = tc::to_tf32(x[4 * q]);
-    h.y = tc::to_tf32(x[4 * q + 1]);
-    h.z = tc::to_tf32(x[4 * q + 2]);
-    h.w = tc::to_tf32(x[4 * q + 3]);
+    h.x = tf32_hi(x[4 * q]);
+    h.y = tf32_hi(x[4 * q + 1]);
+    h.z = tf32_hi(x[4 * q + 2]);
+    h.w = tf32_hi(x[4 * q + 3]);
     l = make_float4(x[4 * q] - h.x, x[4 * q + 1] - h.y, x[4 * q + 2] - h.z, x[4 * q + 3] - h.w);
     const uint32_t o = tc::kmajor_offset(rr, 4 * q, kKc) / 4;
     *reinterpret_cast<float4*>(A_hi + o) = h;
@@ -450,7 +446,8 @@ __device__ __forceinline__ void epilogue_tile(const ContractArgs& a, int64_t r, 
   if (c < c1) epilogue_cols<16>(a, r, tq, c, coff, row_ok);
 }
 
-__global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(ContractArgs a) {
+__global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(ContractArgs a,
+                                                                           const __grid_constant__ CUtensorMap raw_map) {
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* raw = smem;                                                     // [kRawRing][kRawBytes]
   float* sA = reinterpret_cast<float*>(smem + kRawRing * kRawBytes);             // [kAStages][hi, lo][..]
@@ -492,20 +489,16 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(Contr
   const int nsub = a.N > 256 ? 2 : 1;
 
   if (warp == 12) {
-    {  // producer of the long operand (the whole warp)
+    if (lane == 0) {  // producer of the long operand
       uint32_t g = 0;
       bool ok = true;
       for (int64_t t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
         const int64_t r0 = t * kRowsCta;
-        const int nr = (int)min((int64_t)kRowsCta, a.rows - r0);
         for (int h = 0; h < nsub && ok; ++h) {   // the second sub-tile re-reads the rows from L2
           for (int kc = 0; kc < chunks; ++kc, ++g) {
             const uint32_t rs = g % kRawRing, ru = g / kRawRing;
-            if (ru > 0 && !__all_sync(0xffffffffu, pwait(&pb->raw_empty[rs], (ru - 1) & 1, abort_flag))) {
-              ok = false;
-              break;
-            }
-            issue_raw(a, r0, nr, kc, raw + rs * kRawBytes, &pb->raw_full[rs], lane);
+            if (ru > 0 && !pwait(&pb->raw_empty[rs], (ru - 1) & 1, abort_flag)) { ok = false; break; }
+            issue_raw(a, &raw_map, r0, kc, raw + rs * kRawBytes, &pb->raw_full[rs]);
           }
         }
       }
@@ -608,7 +601,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(Contr
           if (!pwait(&pb->raw_full[rs], ru & 1, abort_flag)) { ok = false; break; }
           if (au > 0 && !pwait(&pb->a_empty[as], (au - 1) & 1, abort_flag)) { ok = false; break; }
           float* A_hi = sA + as * 2 * kAStageFloats;
-          convert_row(a, r0, kc, rr, raw + rs * kRawBytes, A_hi, A_hi + kAStageFloats);
+          convert_row(a, r0 + rr < a.rows, kc, rr, raw + rs * kRawBytes, A_hi, A_hi + kAStageFloats);
           tc::fence_proxy_async_smem();
           mbar_arrive(&pb->a_full[as]);
           mbar_arrive(&pb->raw_empty[rs]);
@@ -732,19 +725,45 @@ __global__ void build_b_kernel(ContractArgs a, TileGeom g, const cpx<float>* __r
 
 int round16(int x) { return (x + 15) / 16 * 16; }
 
-// The bulk copies of the pipelined kernel start on 16-byte boundaries and move
-// whole 16-byte units: the long operand's base, its row stride and its row
-// count must keep every copied row slice 16-byte aligned.
-bool pipe_ok(const ContractArgs& a, rsv_operator op) {
+// The driver's tensor-map encoder (null when there is none), through the runtime: no link to the driver.
+using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeTiled encode_tiled() {
+  static const EncodeTiled fn = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+    }
+    return reinterpret_cast<EncodeTiled>(p);
+  }();
+  return fn;
+}
+
+// Tensor map of the long operand for the pipelined kernel: FP32 values, rows fastest, boxes of one K chunk
+// by 128 rows.  False where the operand does not fit one: its base and its row stride in memory must be
+// multiples of 16 bytes and a row of it shorter than 2^32 values.
+bool raw_map_of(const ContractArgs& a, const TileGeom& g, rsv_operator op, CUtensorMap* map) {
   static const int env = [] {
     const char* e = getenv("RSV_CONTRACT_PIPE");
     return e != nullptr && e[0] == '0' ? 0 : 1;
   }();
-  if (!env || op->sm_count <= 0) return false;
-  if ((reinterpret_cast<uintptr_t>(a.src) & 15u) != 0) return false;
-  if (a.mode == ANAL_R) return a.rows % 4 == 0;
-  if (a.mode == ANAL_C) return a.rows % 2 == 0;
-  return a.rows % 2 == 0 && a.src_stride % 2 == 0;
+  if (!env || op->sm_count <= 0 || encode_tiled() == nullptr) return false;
+  const bool real = a.mode == ANAL_R, anal = real || a.mode == ANAL_C;
+  const cuuint64_t vals = (cuuint64_t)a.rows * (real ? 1 : 2);
+  const cuuint64_t stride = (cuuint64_t)(anal ? a.rows : a.src_stride) * (real ? 4 : 8);
+  if ((reinterpret_cast<uintptr_t>(a.src) & 15u) != 0 || stride % 16 != 0 || vals >= ((cuuint64_t)1 << 31) ||
+      stride >= ((cuuint64_t)1 << 40))
+    return false;
+  const cuuint64_t dims[2] = {vals, (cuuint64_t)(anal ? g.steps : a.n_omega)};
+  const cuuint32_t box[2] = {(cuuint32_t)(kRowsCta * (real ? 1 : 2)), (cuuint32_t)(real ? kKc : kKc / 2)};
+  const cuuint32_t unit[2] = {1, 1};
+  return encode_tiled()(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(a.src), dims, &stride, box, unit,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 cudaError_t run(ContractArgs& a, const TileGeom& g, rsv_operator op) {
@@ -762,9 +781,10 @@ cudaError_t run(ContractArgs& a, const TileGeom& g, rsv_operator op) {
     ae = cudaFuncSetAttribute(tc_contract_pipe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem);
   if (ae != cudaSuccess) return ae;
   const int64_t tiles = (a.rows + kRowsCta - 1) / kRowsCta;
-  if (pipe_ok(a, op)) {
+  CUtensorMap map;
+  if (raw_map_of(a, g, op, &map)) {
     const unsigned blocks = (unsigned)std::min<int64_t>(tiles, (int64_t)op->sm_count);
-    tc_contract_pipe_kernel<<<blocks, kPipeThreads, kPipeSmem, op->stream>>>(a);
+    tc_contract_pipe_kernel<<<blocks, kPipeThreads, kPipeSmem, op->stream>>>(a, map);
   } else {
     tc_contract_kernel<<<(unsigned)tiles, 256, kSmem, op->stream>>>(a);
   }
