@@ -421,19 +421,27 @@ __device__ __forceinline__ void epilogue_cols(const ContractArgs& a, int64_t r, 
   else tc::tmem_ld16(tq + (uint32_t)cl, v);
   if (!row_ok) return;
   const int c = coff + cl;
+  // whole groups of stage times step a pointer; only the last one tests each
   if (a.mode == SYNTH_C) {
-    float2* F = reinterpret_cast<float2*>(a.out);
+    const int tau = c >> 1;
+    float2* F = reinterpret_cast<float2*>(a.out) + (int64_t)(a.tau0 + tau) * a.rows + r;
+    if (tau + W / 2 <= a.n_tau) {
 #pragma unroll
-    for (int q = 0; q < W; q += 2) {
-      const int tau = (c + q) >> 1;
-      if (tau < a.n_tau) __stcs(F + (int64_t)(a.tau0 + tau) * a.rows + r, make_float2(v[q], v[q + 1]));
+      for (int q = 0; q < W; q += 2, F += a.rows) __stcs(F, make_float2(v[q], v[q + 1]));
+    } else {
+#pragma unroll
+      for (int q = 0; q < W; q += 2, F += a.rows)
+        if (tau + q / 2 < a.n_tau) __stcs(F, make_float2(v[q], v[q + 1]));
     }
-  } else if (a.mode == SYNTH_R) {
-    float* F = reinterpret_cast<float*>(a.out);
+  } else {
+    float* F = reinterpret_cast<float*>(a.out) + (int64_t)(a.tau0 + c) * a.rows + r;
+    if (c + W <= a.n_tau) {
 #pragma unroll
-    for (int q = 0; q < W; ++q) {
-      const int tau = c + q;
-      if (tau < a.n_tau) __stcs(F + (int64_t)(a.tau0 + tau) * a.rows + r, v[q]);
+      for (int q = 0; q < W; ++q, F += a.rows) __stcs(F, v[q]);
+    } else {
+#pragma unroll
+      for (int q = 0; q < W; ++q, F += a.rows)
+        if (c + q < a.n_tau) __stcs(F, v[q]);
     }
   }
 }
