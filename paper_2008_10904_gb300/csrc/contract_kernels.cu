@@ -185,11 +185,11 @@ __global__ void __launch_bounds__(kTPB) analysis_kernel(TileGeom g, const void* 
 template <typename R>
 __global__ void finish_kernel(const cpx<double>* acc, int64_t acc_stride, int n_omega, int64_t rows, double scale,
                               const double* __restrict__ pscale, int64_t n, cpx<R>* out, int64_t out_stride, int nx,
-                              int nxp) {
+                              int nxp, const int32_t* __restrict__ slot_of_row) {
   const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y;
   if (r >= rows || j >= n_omega) return;
-  const int64_t ra = nx == nxp ? r : r / nx * nxp + r % nx;
+  const int64_t ra = slot_of_row != nullptr ? slot_of_row[r] : nx == nxp ? r : r / nx * nxp + r % nx;
   const cpx<double> v = acc[(int64_t)j * acc_stride + ra];
   const double f = pscale ? scale * pscale[r % n] : scale;
   out[(int64_t)j * out_stride + r] = mk<R>(R(v.re * f), R(v.im * f));
@@ -246,10 +246,10 @@ cudaError_t launch_analysis(const TileGeom& g, const void* Y, int s0, int s1, co
 template <typename R>
 cudaError_t launch_finish(const cpx<double>* acc, int64_t acc_stride, int n_omega, int64_t rows, double scale,
                           void* out, int64_t out_stride, cudaStream_t st, const double* pscale, int64_t n, int nx,
-                          int nxp) {
+                          int nxp, const int32_t* slot_of_row) {
   dim3 grid((unsigned)((rows + 255) / 256), (unsigned)n_omega);
   finish_kernel<R><<<grid, 256, 0, st>>>(acc, acc_stride, n_omega, rows, scale, pscale, n > 0 ? n : rows,
-                                         (cpx<R>*)out, out_stride, nx, nxp);
+                                         (cpx<R>*)out, out_stride, nx, nxp, slot_of_row);
   return cudaGetLastError();
 }
 
@@ -272,9 +272,9 @@ template cudaError_t launch_analysis<double>(const TileGeom&, const void*, int, 
 template cudaError_t launch_analysis<float>(const TileGeom&, const void*, int, int, const void*, const int64_t*,
                                            bool, cpx<double>*, int64_t, cudaStream_t);
 template cudaError_t launch_finish<double>(const cpx<double>*, int64_t, int, int64_t, double, void*, int64_t,
-                                          cudaStream_t, const double*, int64_t, int, int);
+                                          cudaStream_t, const double*, int64_t, int, int, const int32_t*);
 template cudaError_t launch_finish<float>(const cpx<double>*, int64_t, int, int64_t, double, void*, int64_t,
-                                         cudaStream_t, const double*, int64_t, int, int);
+                                         cudaStream_t, const double*, int64_t, int, int, const int32_t*);
 template cudaError_t launch_scale_block<double>(const void*, int64_t, void*, int64_t, int, int64_t, int64_t,
                                                const double*, cudaStream_t);
 template cudaError_t launch_scale_block<float>(const void*, int64_t, void*, int64_t, int, int64_t, int64_t,

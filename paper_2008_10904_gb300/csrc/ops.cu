@@ -182,6 +182,7 @@ size_t stage_scratch_bytes(rsv_operator op, int kg) {
 
 int march_tile_kernels(rsv_operator op, int steps, int kg, bool step_form) {
   if (step_form) {   // 2-D FP32: one launch per step; 3-D: two; FP64: one per stage
+    if (op->kind == RSV_OP_GL1D) return 1;
     if (op->kind == RSV_OP_ADR2D) return op->prec == RSV_PREC_FP32 ? steps + 1 : 4 * steps + 2;
     return 2 * steps + 1;
   }
@@ -220,6 +221,7 @@ rsv_status on_frequencies(rsv_operator op) {
 // ---------------------------------------------------------------------------
 bool step_form_taken(rsv_operator op, int k) {
   if (op->scheme != RSV_SCHEME_RK4 || k > 65535) return false;
+  if (op->kind == RSV_OP_GL1D) return step32_taken(op, k);
   if (op->kind == RSV_OP_ADR2D) {
     const char* e = getenv("RSV_STENCIL_FUSED");
     if (e != nullptr && e[0] == '1') return false;
@@ -234,11 +236,19 @@ bool step_form_taken(rsv_operator op, int k) {
 
 int64_t step_points(rsv_operator op) {
   if (op->kind == RSV_OP_ADR2D || op->kind == RSV_OP_ADV3D) return op->n / op->nx * ((op->nx + 3) / 4 * 4);
-  return op->n;
+  int64_t slots = 0;   // 1-D: whole groups of four, at least one empty slot behind each instance
+  for (int len : op->inst_len) slots += (len + 4) / 4 * 4;
+  return slots;
+}
+
+int64_t step_rows(rsv_operator op, int kg) {
+  if (op->kind == RSV_OP_GL1D && op->p32.kg == kg) return op->p32.slots;
+  return (int64_t)kg * step_points(op);
 }
 
 // A second state buffer and one stage buffer, then (2-D FP64) the stages' row and sponge tables.
 size_t step_scratch_bytes(rsv_operator op, int kg) {
+  if (op->kind == RSV_OP_GL1D) return 0;
   const size_t el = op->prec == RSV_PREC_FP64 ? 8 : 4;
   const size_t tab = op->kind == RSV_OP_ADR2D && el == 8 ? (size_t)(17 * (size_t)op->ny + op->nx) * el : 0;
   return 2 * (size_t)kg * step_points(op) * el + tab;
@@ -258,6 +268,7 @@ rsv_status step_coefficients(rsv_operator op, const void* fhat, int64_t f_stride
   size_t tmp = 0;
   const size_t bytes = step_coef_bytes(op, kg, &tmp);
   rsv_status s = ensure(op->ws_coef, bytes);
+  if (op->kind == RSV_OP_GL1D) return s == RSV_OK ? step32_coefficients(op, fhat, f_stride, kg, adjoint, op->ws_coef.ptr) : s;
   if (s == RSV_OK) s = ensure(op->ws_coef2, tmp);
   if (s != RSV_OK) return s;
   const cudaError_t e = step_coefs_grid<R>(op, fhat, f_stride, kg, adjoint, op->ws_coef.ptr, op->ws_coef2.ptr,
@@ -271,7 +282,7 @@ rsv_status prepare_coefficients(rsv_operator op, const void* fhat, int64_t f_str
   if (step_form) {
     rsv_status s = step_coefficients<R>(op, fhat, f_stride, kg, adjoint);
     *coef = op->ws_coef.ptr;
-    *coef_stride = (int64_t)kg * step_points(op);
+    *coef_stride = step_rows(op, kg);
     *synth_stride = 2;
     return s;
   }
@@ -584,8 +595,10 @@ static cudaError_t march_tile_direct(rsv_operator op, const MarchTile& t, void* 
                                      double* norms) {
   if (t.step_form) {
     if (op->kind == RSV_OP_ADR2D) return step_march_2d<R>(op, t, state, F, Y);
-    if constexpr (sizeof(R) == 4)
+    if constexpr (sizeof(R) == 4) {
       if (op->kind == RSV_OP_ADV3D) return step_march_3d(op, t, state, F, Y);
+      if (op->kind == RSV_OP_GL1D) return step_march_1d32(op, t, state, F, Y);
+    }
     return cudaErrorNotSupported;
   }
   switch (op->kind) {

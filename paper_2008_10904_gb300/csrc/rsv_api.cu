@@ -138,7 +138,7 @@ rsv_operator_s::~rsv_operator_s() {
   }
   if (copy_stream) cudaStreamDestroy(copy_stream);
   if (ws_scaled.ptr) cudaFree(ws_scaled.ptr);
-  for (Workspace* w : {&ws_band[0], &ws_band[1], &ws_part})
+  for (Workspace* w : {&ws_band[0], &ws_band[1], &ws_part, &ws_p32})
     if (w->ptr) cudaFree(w->ptr);
   for (cudaEvent_t e : prof.pool) cudaEventDestroy(e);
 }
@@ -259,6 +259,8 @@ extern "C" rsv_status rsv_describe(rsv_operator op, char* buf, int32_t buflen) {
     if (jump_taken(op, 1))
       path = op->scheme == RSV_SCHEME_CN ? "cuda-core crank-nicolson jump kernels (few pairs, else tile kernel)"
                                          : "cuda-core jump kernels (few pairs, else tile kernel)";
+    else if (step_form_taken(op, 1))
+      path = "cuda-core packed step kernel (sampled forcing: tile kernel)";
     else
       path = op->scheme == RSV_SCHEME_CN ? "cuda-core crank-nicolson tile kernel" : "cuda-core tile kernel";
   }
@@ -292,7 +294,10 @@ extern "C" rsv_status rsv_describe(rsv_operator op, char* buf, int32_t buflen) {
   }
   const char* contract = (op->prec == RSV_PREC_FP32 && !op->tc_contract_disabled) ? "tcgen05" : "cuda-core";
   char packs[96] = "";
-  if (op->kind == RSV_OP_GL1D && op->pack_kg > 0)
+  if (op->kind == RSV_OP_GL1D && op->p32.kg > 0 && op->p32.q > 0)
+    snprintf(packs, sizeof(packs), " packed=%d ctas of %d slots (1024x%d, %d per wave)", op->p32.packs, 1024 * op->p32.q,
+             op->p32.q, op->p32.wave);
+  else if (op->kind == RSV_OP_GL1D && op->pack_kg > 0)
     snprintf(packs, sizeof(packs), " packed=%d ctas of %d slots (%dx%d, %d per wave)", op->pack_count,
              op->pack_threads * op->pack_ppt, op->pack_threads, op->pack_ppt, op->pack_wave);
   else if (op->kind == RSV_OP_GL1D && op->gl_cluster > 0)
@@ -608,6 +613,9 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
   if (trial) {
     S = trial->S;
     kg = trial->kg;
+  } else if (sf && !truncate && tc_contract_segments(op) && !(opts && opts->tile_steps > 0) && op->tuned_k != k) {
+    // one synthesis time per step: as many columns as 2 S + 1 stage times, and half the accumulator traffic
+    S = 2 * (S + 1);
   } else if (jump && !truncate && !(opts && opts->tile_steps > 0) && op->tuned_k != k) {
     // the jumps' launches are short: tiles as long as 128 MB of snapshots, a window at most
     S = (int)std::max<int64_t>(S, std::min<int64_t>(op->n_t, ((int64_t)128 << 20) / ((int64_t)kg * n * 16)));
@@ -653,6 +661,9 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
   cudaError_t e;
   op->last_tile = S;
   op->last_group = kg;
+  // the 1-D step form's groups fill whole packs
+  const bool packed = sf && op->kind == RSV_OP_GL1D;
+  if (packed && (st = step32_packs(op, kg)) != RSV_OK) return st;
   const int64_t rows_max = (int64_t)kg * np;
   if ((st = ensure(op->ws_state, rows_max * se + scratch_bytes(kg))) != RSV_OK) return st;
   if ((st = ensure(op->ws_ftile, (size_t)f_rows(S) * rows_max * se)) != RSV_OK) return st;
@@ -722,7 +733,8 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
   if (host_in && (e = stage_copy(0)) != cudaSuccess) return cuda_fail(e, "staging copy");
   for (int v0 = 0; v0 < (trial ? std::min(kg, k) : k); v0 += kg) {
     const int kv = std::min(kg, k - v0);
-    const int64_t rows = (int64_t)kv * np;
+    if (packed && (st = step32_packs(op, kv)) != RSV_OK) return st;
+    const int64_t rows = sf ? step_rows(op, kv) : (int64_t)kv * np;
     cpx<double>* acc;
     int64_t acc_stride;
     if (acc_in_out) {
@@ -838,7 +850,8 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
       }
       if (truncate && ((n0 + g.steps) % S == 0 || n0 + g.steps == sc.total)) {   // check points: the tile ends
         const int64_t n_end = n0 + g.steps;
-        e = state_sq_norms(op, kv, n_end, np, (double*)op->ws_norm.ptr);
+        e = packed ? step32_sq_norms(op, kv, (double*)op->ws_norm.ptr)
+                   : state_sq_norms(op, kv, n_end, np, (double*)op->ws_norm.ptr);
         if (e == cudaSuccess)
           e = cudaMemcpyAsync(nrm.data(), op->ws_norm.ptr, sizeof(double) * kv, cudaMemcpyDeviceToHost, stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
@@ -868,7 +881,8 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
     if (!truncate) op->last_steps = sc.total;
     void* o = static_cast<char*>(out) + (size_t)v0 * n * ce;
     e = launch_finish<R>(acc, acc_stride, op->n_omega, (int64_t)kv * n, 1.0 / (double)op->n_t, o, (int64_t)k * n, stream,
-                         s_out, n, np == n ? 0 : op->nx, np == n ? 0 : (op->nx + 3) / 4 * 4);
+                         s_out, n, np == n ? 0 : op->nx, np == n ? 0 : (op->nx + 3) / 4 * 4,   // packed: unused
+                         packed ? (const int32_t*)op->p32.slot : nullptr);
     if (e != cudaSuccess) return cuda_fail(e, "finish");
   }
   int flag = 0;

@@ -109,6 +109,13 @@ struct JumpPlan {
   bool built = false;
   void *Tp = nullptr, *T1 = nullptr;
 };
+// Packs of the FP32 1-D step form (step1d32.cu) for groups of kg vectors: CTAs, warps of the widest, the
+// capacity 1024 q they were filled to (0: one pair per pack), CTAs per wave, slots of all, the device maps.
+struct Pack32 {
+  int kg = 0, packs = 0, warps = 0, q = 0, wave = 0;
+  int64_t slots = 0;
+  void *slot = nullptr, *first = nullptr, *off = nullptr;   // slot of each row; row of each slot group; packs' starts
+};
 struct TileGraph {
   TileGraphKey key;
   cudaGraphExec_t exec;
@@ -149,6 +156,8 @@ struct rsv_operator_s {
   int gl_max_n = 0;
   bool tri_real = false;                // every coefficient is real
   rsv::JumpPlan jump[2];                // direct, adjoint (reset with the frequencies)
+  rsv::Pack32 p32;
+  rsv::Workspace ws_p32;
   rsv::Workspace ws_band[2], ws_part;   // step matrices; partial sums of the FP64 analysis
   // packed launch of uneven GL1D batches (built per vector-group size): slot map, CTA count, threads
   // and slots per thread of a CTA, CTAs per wave (SMs x CTAs resident per SM)
@@ -273,11 +282,13 @@ cudaError_t launch_analysis(const TileGeom& g, const void* Y, int s0, int s1, co
                             const int64_t* pj, bool real_state, cpx<double>* acc, int64_t acc_stride,
                             cudaStream_t st);
 // out[j][r] = acc[j][r] * scale (* pscale[r mod n] when given), converted to the element type R; with
-// nx > 0 the accumulator's rows of nx cells are padded to nxp (r counts the unpadded ones)
+// nx > 0 the accumulator's rows of nx cells are padded to nxp (r counts the unpadded ones), with
+// slot_of_row its value r sits at slot_of_row[r]
 template <typename R>
 cudaError_t launch_finish(const cpx<double>* acc, int64_t acc_stride, int n_omega, int64_t rows,
                           double scale, void* out, int64_t out_stride, cudaStream_t st,
-                          const double* pscale = nullptr, int64_t n = 0, int nx = 0, int nxp = 0);
+                          const double* pscale = nullptr, int64_t n = 0, int nx = 0, int nxp = 0,
+                          const int32_t* slot_of_row = nullptr);
 // out[j][r] = in[j][r] * s[r mod n] for j < n_omega, r < rows (in and out may alias)
 template <typename R>
 cudaError_t launch_scale_block(const void* in, int64_t in_stride, void* out, int64_t out_stride, int n_omega,
@@ -286,6 +297,7 @@ cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t st);
 
 // ----- tensor-core contractions (tc_contract.cu), FP32 mode -----------------
 bool tc_contract_supported(rsv_operator op, bool synth);
+bool tc_contract_segments(rsv_operator op);   // tiles of up to 512 values are analysed in two sums
 cudaError_t tc_synth(rsv_operator op, const TileGeom& g, const void* fhat, void* F);
 cudaError_t tc_analysis(rsv_operator op, const TileGeom& g, const void* Y, int s0, int s1, cpx<double>* acc,
                         int64_t acc_stride);

@@ -31,6 +31,7 @@ int march_tile_kernels(rsv_operator op, int steps, int kg, bool step_form = fals
 // vector of its tiles, and its scratch behind the state.
 bool step_form_taken(rsv_operator op, int k);
 int64_t step_points(rsv_operator op);
+int64_t step_rows(rsv_operator op, int kg);   // rows of a group of kg vectors, kg * step_points at most
 size_t step_scratch_bytes(rsv_operator op, int kg);
 // Bytes of transformed coefficients (and their temporary) of one vector group.
 size_t step_coef_bytes(rsv_operator op, int kg, size_t* tmp);
@@ -43,6 +44,13 @@ cudaError_t step_coefs_grid(rsv_operator op, const void* fhat, int64_t f_stride,
 template <typename R>
 cudaError_t step_march_2d(rsv_operator op, const MarchTile& t, void* state, const void* G, void* Y);
 cudaError_t step_march_3d(rsv_operator op, const MarchTile& t, void* state, const void* G, void* Y);
+
+// FP32 1-D marches in packs (step1d32.cu)
+bool step32_taken(rsv_operator op, int k);
+rsv_status step32_packs(rsv_operator op, int kg);
+rsv_status step32_coefficients(rsv_operator op, const void* fhat, int64_t f_stride, int kg, bool adjoint, void* out);
+cudaError_t step_march_1d32(rsv_operator op, const MarchTile& t, void* state, const void* G, void* Y);
+cudaError_t step32_sq_norms(rsv_operator op, int kg, double* d_out);
 
 // FP64 1-D marches of few pairs by jumps over several steps (step1d.cu)
 bool jump_taken(rsv_operator op, int k);

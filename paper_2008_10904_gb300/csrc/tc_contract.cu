@@ -54,6 +54,7 @@ struct ContractArgs {
   const float* B;          // [K / 16][2][kMaxN x 16] pre-split twiddle chunks
   void* out;               // synthesis: F [n_tau][rows]; analysis: acc (cpx<double>) [n_omega][acc_stride]
   int64_t acc_stride;
+  int seg;                 // K chunks summed in one tensor-memory accumulator (pipelined kernel)
   int* err;
 };
 
@@ -395,20 +396,25 @@ __device__ __forceinline__ void load_acc16(const ContractArgs& a, int64_t r, int
     old[q] = (r < a.rows && j < a.n_omega) ? __ldcs(acc + (int64_t)j * a.acc_stride + r) : make_double2(0.0, 0.0);
   }
 }
-// += v, the columns' sums over the tile.
-__device__ __forceinline__ void add_acc16(const ContractArgs& a, int64_t r, int c, const double2 old[8], const float v[16]) {
-  if (r >= a.rows) return;
+// += v, the columns' sums over the tile or a segment of it.
+__device__ __forceinline__ void add_acc16(double2 old[8], const float v[16]) {
   uint32_t top = 0;
 #pragma unroll
   for (int q = 0; q < 16; ++q) top = max(top, __float_as_uint(v[q]) & 0x7fffffffu);
-  double2* acc = reinterpret_cast<double2*>(a.out);
   const bool plain = top < 0x7f800000u;   // no infinity and no NaN
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
+    old[q].x += plain ? widen(v[2 * q]) : (double)v[2 * q];
+    old[q].y += plain ? widen(v[2 * q + 1]) : (double)v[2 * q + 1];
+  }
+}
+__device__ __forceinline__ void store_acc16(const ContractArgs& a, int64_t r, int c, const double2 old[8]) {
+  if (r >= a.rows) return;
+  double2* acc = reinterpret_cast<double2*>(a.out);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
     const int j = (c >> 1) + q;
-    if (j >= a.n_omega) continue;
-    const double re = plain ? widen(v[2 * q]) : (double)v[2 * q], im = plain ? widen(v[2 * q + 1]) : (double)v[2 * q + 1];
-    __stcs(acc + (int64_t)j * a.acc_stride + r, make_double2(old[q].x + re, old[q].y + im));
+    if (j < a.n_omega) __stcs(acc + (int64_t)j * a.acc_stride + r, old[q]);
   }
 }
 
@@ -567,6 +573,8 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(Contr
               break;
             }
             tc::tc_fence_after();
+            const int seg0 = kc >= a.seg ? a.seg : 0;            // first chunk of the segment
+            const uint32_t ds = d + (seg0 > 0 ? 128u : 0u);
             const char* A_hi = reinterpret_cast<const char*>(sA + as * 2 * kAStageFloats);
             const char* A_lo = A_hi + 4 * kAStageFloats;
             const char* B_hi = reinterpret_cast<const char*>(sB + bs * 2 * kBRingFloats);
@@ -577,9 +585,9 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(Contr
               const uint64_t al = tc::smem_desc(A_lo + ks * 256, 128, sbo);
               const uint64_t bh = tc::smem_desc(B_hi + ks * 256, 128, sbo);
               const uint64_t bl = tc::smem_desc(B_lo + ks * 256, 128, sbo);
-              tc::mma_tf32(d, ah, bh, idesc, kc > 0 || ks > 0);
-              tc::mma_tf32(d, ah, bl, idesc, true);
-              tc::mma_tf32(d, al, bh, idesc, true);
+              tc::mma_tf32(ds, ah, bh, idesc, kc > seg0 || ks > 0);
+              tc::mma_tf32(ds, ah, bl, idesc, true);
+              tc::mma_tf32(ds, al, bh, idesc, true);
             }
             tc::mma_commit(&pb->a_empty[as]);
             tc::mma_commit(&pb->b_empty[bs]);
@@ -662,7 +670,12 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(Contr
             }
             float v[16];
             tc::tmem_ld16(tq + (uint32_t)c, v);
-            add_acc16(a, r, 256 * h + c, old, v);
+            add_acc16(old, v);
+            if (a.seg < chunks) {   // the tile's second segment
+              tc::tmem_ld16(tq + 128u + (uint32_t)c, v);
+              add_acc16(old, v);
+            }
+            store_acc16(a, r, 256 * h + c, old);
           }
         } else {
           epilogue_tile(a, r, tq, c0, c1, 256 * h);
@@ -754,12 +767,15 @@ EncodeTiled encode_tiled() {
 // Tensor map of the long operand for the pipelined kernel: FP32 values, rows fastest, boxes of one K chunk
 // by 128 rows.  False where the operand does not fit one: its base and its row stride in memory must be
 // multiples of 16 bytes and a row of it shorter than 2^32 values.
-bool raw_map_of(const ContractArgs& a, const TileGeom& g, rsv_operator op, CUtensorMap* map) {
+bool pipe_enabled(rsv_operator op) {
   static const int env = [] {
     const char* e = getenv("RSV_CONTRACT_PIPE");
     return e != nullptr && e[0] == '0' ? 0 : 1;
   }();
-  if (!env || op->sm_count <= 0 || encode_tiled() == nullptr) return false;
+  return env && op->sm_count > 0 && encode_tiled() != nullptr;
+}
+bool raw_map_of(const ContractArgs& a, const TileGeom& g, rsv_operator op, CUtensorMap* map) {
+  if (!pipe_enabled(op)) return false;
   const bool real = a.mode == ANAL_R, anal = real || a.mode == ANAL_C;
   const cuuint64_t vals = (cuuint64_t)a.rows * (real ? 1 : 2);
   const cuuint64_t stride = (cuuint64_t)(anal ? a.rows : a.src_stride) * (real ? 4 : 8);
@@ -779,6 +795,12 @@ cudaError_t run(ContractArgs& a, const TileGeom& g, rsv_operator op) {
   if (ensure(op->ws_tcb, bbytes) != RSV_OK) return cudaErrorMemoryAllocation;
   a.B = (const float*)op->ws_tcb.ptr;
   a.err = op->d_flag;
+  // Tensor memory sums in FP32 with truncation, a bias that grows with the length of the sum: 2.9e-6 of a
+  // march's result with 254 values, 5.2e-6 with 512.  So an analysis of more than 256 values whose columns
+  // leave room takes two accumulators per tile, added up in FP64.
+  const int chunks = a.K / kKc;
+  const bool anal = a.mode == ANAL_C || a.mode == ANAL_R;
+  a.seg = anal && a.N <= 128 && chunks > 16 ? std::max(16, (chunks + 1) / 2) : chunks;
   const int64_t total = (int64_t)kMaxN * a.K;
   build_b_kernel<<<(unsigned)((total + 255) / 256), 256, 0, op->stream>>>(a, g, (const cpx<float>*)op->d_tw, op->d_pj,
                                                                           op->d_cw, (float*)op->ws_tcb.ptr);
@@ -804,6 +826,10 @@ cudaError_t run(ContractArgs& a, const TileGeom& g, rsv_operator op) {
 bool tc_contract_supported(rsv_operator op, bool synth) {
   if (op->prec != RSV_PREC_FP32 || op->tc_contract_disabled) return false;
   return synth || round16(2 * op->n_omega) <= kMaxN;
+}
+
+bool tc_contract_segments(rsv_operator op) {
+  return tc_contract_supported(op, false) && pipe_enabled(op) && round16(2 * op->n_omega) <= 128;
 }
 
 // Stage times are processed in calls of at most 512 output columns (256 complex).
