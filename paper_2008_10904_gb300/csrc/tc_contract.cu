@@ -51,7 +51,7 @@ struct ContractArgs {
   const void* src;         // coefficients [n_omega][coef_stride] or snapshots [steps][rows]
   int64_t src_stride;
   int s0, s1;              // analysis: valid tile steps [s0, s1)
-  const float* B;          // [K / 16][2][kMaxN x 16] pre-split twiddle chunks
+  const float* B;          // [K / 16][sub-tile of up to 256 columns][hi, lo][columns x 16] pre-split twiddles
   void* out;               // synthesis: F [n_tau][rows]; analysis: acc (cpx<double>) [n_omega][acc_stride]
   int64_t acc_stride;
   int seg;                 // K chunks summed in one tensor-memory accumulator (pipelined kernel)
@@ -166,10 +166,14 @@ __global__ void __launch_bounds__(256, 1) tc_contract_kernel(ContractArgs a) {
       mma_phase[st] ^= 1;
     }
     if (tid == 0) {
-      const float* bsrc = a.B + (size_t)kc * 2 * kBStageFloats;
+      const float* bsrc = a.B + (size_t)kc * 2 * a.N * kKc;
       tc::mbar_arrive_expect_tx(&bars[st], 2 * bchunk_bytes);
-      tc::bulk_g2s(B_hi, bsrc, bchunk_bytes, &bars[st]);
-      tc::bulk_g2s(B_lo, bsrc + kBStageFloats, bchunk_bytes, &bars[st]);
+      for (int nh = 0; nh < a.N; nh += 256) {
+        const int nf = min(256, a.N - nh) * kKc;
+        tc::bulk_g2s(B_hi + nh * kKc, bsrc, 4 * nf, &bars[st]);
+        tc::bulk_g2s(B_lo + nh * kKc, bsrc + nf, 4 * nf, &bars[st]);
+        bsrc += 2 * nf;
+      }
     }
     store_share(a, tid, cur, A_hi, A_lo);
     tc::fence_proxy_async_smem();
@@ -263,10 +267,12 @@ __global__ void __launch_bounds__(256, 1) tc_contract_kernel(ContractArgs a) {
 //                        storage precision into an 8-deep raw ring, one tensor
 //                        copy per chunk;
 //   warp 14 (one thread) producer: bulk-copies the chunk's pre-split twiddles
-//                        into a 2-deep B ring;
-//   warps 0-3            converters: one row each, raw value -> TF32 hi / lo in
-//                        the K-major operand layout (2 stages);
-//   warp 13 (one thread) MMA issuer: 3 TF32 MMAs per K-step and N half into the
+//                        into a 4-deep B ring, one copy per chunk;
+//   warps 0-3            converters: one row each, raw value -> TF32 hi / lo, into
+//                        tensor memory where at most 96 columns leave room for it
+//                        (4 stages), else in the K-major operand layout in shared
+//                        memory (2 stages);
+//   warp 13              MMA issuer: 3 TF32 MMAs per K-step and N half into the
 //                        tile's tensor-memory accumulator, commits release the
 //                        operand stages and, after the last chunk, the tile;
 //   warps 4-11           epilogue: two warps per tensor-memory lane quadrant,
@@ -292,8 +298,8 @@ constexpr int kPipeThreads = 480;                    // 15 warps, roles below
 
 struct PipeBars {
   uint64_t raw_full[kRawRing], raw_empty[kRawRing];
-  uint64_t a_full[kAStages], a_empty[kAStages];
-  uint64_t b_full[kBRing], b_empty[kBRing];
+  uint64_t a_full[kBRing], b_full[kBRing];
+  uint64_t empty[kBRing];               // products of chunk g done: empty[g % kBRing]
   uint64_t acc_full[2], acc_empty[2];   // two tensor-memory accumulators of 256 columns
   int abort_flag;
 };
@@ -307,6 +313,20 @@ static_assert(kPipeSmem + 1024 <= 232448, "pipelined contraction exceeds the sha
 
 __device__ __forceinline__ bool pwait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
   return tc::mbar_wait(bar, parity, 0xFFFFFFFFu, abort_flag);
+}
+
+// One warp waits for two barriers; the same answer in every lane.
+__device__ __forceinline__ bool pwait2(uint64_t* b0, uint32_t p0, uint64_t* b1, uint32_t p1, volatile int* abort_flag) {
+  uint64_t t0 = 0;
+  for (uint32_t i = 0;; ++i) {
+    const bool d0 = tc::mbar_try(b0, p0), d1 = tc::mbar_try(b1, p1);
+    if (__all_sync(0xffffffffu, d0 && d1)) return true;
+    if ((i & 63) == 63) {
+      const uint64_t now = tc::global_ns();
+      if (t0 == 0) t0 = now;
+      if (__any_sync(0xffffffffu, *abort_flag != 0 || now - t0 > tc::kWaitLimitNs)) return false;
+    }
+  }
 }
 
 __device__ __forceinline__ void pabort(PipeBars* pb, int* err) {
@@ -336,9 +356,8 @@ __device__ __forceinline__ float tf32_hi(float x) { return __uint_as_float((__fl
 
 // One row of a chunk.  A warp converts a chunk per scheduler, so its instruction count is the chunk's time:
 // chunks that are valid as a whole take no test per value.
-__device__ __forceinline__ void convert_row(const ContractArgs& a, bool row_ok, int kc, int rr, const unsigned char* raw,
-                                            float* A_hi, float* A_lo) {
-  float x[kKc];
+__device__ __forceinline__ void load_row(const ContractArgs& a, bool row_ok, int kc, int rr, const unsigned char* raw,
+                                         float x[kKc]) {
   if (a.mode == ANAL_R) {
     const float* rv = reinterpret_cast<const float*>(raw) + rr;
     const int s = kc * kKc;
@@ -363,6 +382,8 @@ __device__ __forceinline__ void convert_row(const ContractArgs& a, bool row_ok, 
       for (int k = 0; k < kKc; ++k) x[k] = (row_ok && idx + k / 2 >= lo && idx + k / 2 < hi) ? x[k] : 0.f;
     }
   }
+}
+__device__ __forceinline__ void store_row(const float x[kKc], int rr, float* A_hi, float* A_lo) {
   // K-major core matrices: 4 consecutive K values of one row are one 16-byte vector
 #pragma unroll
   for (int q = 0; q < kKc / 4; ++q) {
@@ -376,6 +397,19 @@ __device__ __forceinline__ void convert_row(const ContractArgs& a, bool row_ok, 
     *reinterpret_cast<float4*>(A_hi + o) = h;
     *reinterpret_cast<float4*>(A_lo + o) = l;
   }
+}
+
+// The same in tensor memory: columns [0, 16) high parts, [16, 32) low parts.
+__device__ __forceinline__ void store_row_tmem(float x[kKc], uint32_t ta) {
+  float h[kKc];
+#pragma unroll
+  for (int k = 0; k < kKc; ++k) {
+    h[k] = tf32_hi(x[k]);
+    x[k] -= h[k];
+  }
+  tc::tmem_st16(ta, h);
+  tc::tmem_st16(ta + 16, x);
+  tc::tmem_wait_st();
 }
 
 // FP32 -> FP64 with integer instructions (exact for zero and normal values).  FP64 instructions issue once
@@ -460,6 +494,15 @@ __device__ __forceinline__ void epilogue_tile(const ContractArgs& a, int64_t r, 
   if (c < c1) epilogue_cols<16>(a, r, tq, c, coff, row_ok);
 }
 
+// kTA: the converted operand in tensor memory (at most 96 columns of a segment, one column sub-tile).  In shared
+// memory a chunk of an analysis with 64 columns moves 76 KB: raw in and out, converted in, read by three
+// products each, twiddles; at 128 bytes per cycle that is most of its time.  In tensor memory 36 KB are left:
+// analysis of the 2-D 1024 x 512 x 16 march 26.4 -> 23.8 ms, of 64 1-D instances x 8 vectors 14.4 -> 12.8 ms.
+constexpr uint32_t kTaCols = 96;                       // columns of a segment's accumulator
+constexpr uint32_t kTaBase = 4 * kTaCols;              // two accumulators of two segments, then the operand's stages
+static_assert(kTaBase + kBRing * 2 * kKc <= 512, "tensor memory");
+
+template <bool kTA>
 __global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(ContractArgs a,
                                                                            const __grid_constant__ CUtensorMap raw_map) {
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -470,19 +513,17 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(Contr
   __shared__ uint32_t tbase;
   volatile int* abort_flag = &pb->abort_flag;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // known to be the warp's: uniform registers
   if (tid == 0) {
     for (int i = 0; i < kRawRing; ++i) {
       tc::mbar_init(&pb->raw_full[i], 1);
       tc::mbar_init(&pb->raw_empty[i], 128);
     }
-    for (int i = 0; i < kAStages; ++i) {
-      tc::mbar_init(&pb->a_full[i], 128);
-      tc::mbar_init(&pb->a_empty[i], 1);
-    }
     for (int i = 0; i < kBRing; ++i) {
+      tc::mbar_init(&pb->a_full[i], 128);
       tc::mbar_init(&pb->b_full[i], 1);
-      tc::mbar_init(&pb->b_empty[i], 1);
+      tc::mbar_init(&pb->empty[i], 1);
     }
     for (int i = 0; i < 2; ++i) {
       tc::mbar_init(&pb->acc_full[i], 1);
@@ -500,7 +541,9 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(Contr
   const int64_t tiles = (a.rows + kRowsCta - 1) / kRowsCta;
   // Each row tile runs as one or two column sub-tiles of at most 256 columns; sub-tiles alternate
   // between the two accumulators, so the products of one overlap the epilogue of the previous one.
-  const int nsub = a.N > 256 ? 2 : 1;
+  const int nsub = !kTA && a.N > 256 ? 2 : 1;
+  constexpr uint32_t kSegCols = kTA ? kTaCols : 128u, kBufCols = 2 * kSegCols;
+  constexpr int kStages = kTA ? kBRing : kAStages;     // of the converted operand
 
   if (warp == 12) {
     if (lane == 0) {  // producer of the long operand
@@ -530,17 +573,14 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(Contr
       bool ok = true;
       for (int64_t t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
         for (int h = 0; h < nsub && ok; ++h) {
-          // rows [256 h, 256 h + nn) of a chunk are one contiguous run of 8-row core-matrix groups
+          // a sub-tile's rows of a chunk, hi and lo, are one contiguous run of 8-row core-matrix groups
           const int nn = h == 0 ? min(256, a.N) : a.N - 256;
           const uint32_t bytes = 4u * (uint32_t)nn * kKc;
           for (int kc = 0; kc < chunks; ++kc, ++g) {
             const uint32_t bs = g % kBRing, bu = g / kBRing;
-            if (bu > 0 && !pwait(&pb->b_empty[bs], (bu - 1) & 1, abort_flag)) { ok = false; break; }
-            float* B_hi = sB + bs * 2 * kBRingFloats;
-            const float* bsrc = a.B + (size_t)kc * 2 * kBStageFloats + (size_t)h * 256 * kKc;
+            if (bu > 0 && !pwait(&pb->empty[bs], (bu - 1) & 1, abort_flag)) { ok = false; break; }
             tc::mbar_arrive_expect_tx(&pb->b_full[bs], 2 * bytes);
-            tc::bulk_g2s(B_hi, bsrc, bytes, &pb->b_full[bs]);
-            tc::bulk_g2s(B_hi + kBRingFloats, bsrc + kBStageFloats, bytes, &pb->b_full[bs]);
+            tc::bulk_g2s(sB + bs * 2 * kBRingFloats, a.B + ((size_t)kc * a.N + 256 * h) * 2 * kKc, 2 * bytes, &pb->b_full[bs]);
           }
         }
       }
@@ -553,56 +593,67 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(Contr
       }
     }
   } else if (warp == 13) {
-    if (lane == 0) {  // MMA issuer
-      uint32_t g = 0, tt = 0;
-      bool ok = true;
-      const uint32_t sbo = (kKc / 4) * 128;
-      for (int64_t t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
-        for (int h = 0; h < nsub; ++h, ++tt) {
-          const uint32_t buf = tt & 1, use = tt >> 1;
-          if (use > 0 && !pwait(&pb->acc_empty[buf], (use - 1) & 1, abort_flag)) { ok = false; break; }
-          tc::tc_fence_after();
-          const int nn = h == 0 ? min(256, a.N) : a.N - 256;
-          const uint32_t idesc = tc::idesc_tf32(128, (uint32_t)nn);
-          const uint32_t d = tmem + buf * 256u;
-          for (int kc = 0; kc < chunks; ++kc, ++g) {
-            const uint32_t as = g % kAStages, au = g / kAStages;
-            const uint32_t bs = g % kBRing, bu = g / kBRing;
-            if (!pwait(&pb->a_full[as], au & 1, abort_flag) || !pwait(&pb->b_full[bs], bu & 1, abort_flag)) {
-              ok = false;
-              break;
-            }
-            tc::tc_fence_after();
-            const int seg0 = kc >= a.seg ? a.seg : 0;            // first chunk of the segment
-            const uint32_t ds = d + (seg0 > 0 ? 128u : 0u);
-            const char* A_hi = reinterpret_cast<const char*>(sA + as * 2 * kAStageFloats);
-            const char* A_lo = A_hi + 4 * kAStageFloats;
-            const char* B_hi = reinterpret_cast<const char*>(sB + bs * 2 * kBRingFloats);
-            const char* B_lo = B_hi + 4 * kBRingFloats;
-#pragma unroll
-            for (int ks = 0; ks < kKc / 8; ++ks) {
-              const uint64_t ah = tc::smem_desc(A_hi + ks * 256, 128, sbo);
-              const uint64_t al = tc::smem_desc(A_lo + ks * 256, 128, sbo);
-              const uint64_t bh = tc::smem_desc(B_hi + ks * 256, 128, sbo);
-              const uint64_t bl = tc::smem_desc(B_lo + ks * 256, 128, sbo);
-              tc::mma_tf32(ds, ah, bh, idesc, kc > seg0 || ks > 0);
-              tc::mma_tf32(ds, ah, bl, idesc, true);
-              tc::mma_tf32(ds, al, bh, idesc, true);
-            }
-            tc::mma_commit(&pb->a_empty[as]);
-            tc::mma_commit(&pb->b_empty[bs]);
+    // MMA issuer: the whole warp walks the chunks, so that addresses and descriptors stay in uniform
+    // registers: with the loop in one lane a chunk's six products took 680 cycles to issue (those analyses
+    // 31.0 and 16.4 ms, 28.8 and 15.6 with one wait and one copy less per chunk, 26.4 and 14.4 like this)
+    uint32_t g = 0, tt = 0;
+    bool ok = true;
+    const bool issue = lane == 0;
+    const uint64_t desc_a = tc::smem_desc(sA, 128, (kKc / 4) * 128), desc_b = tc::smem_desc(sB, 128, (kKc / 4) * 128);
+    for (int64_t t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+      for (int h = 0; h < nsub; ++h, ++tt) {
+        const uint32_t buf = tt & 1, use = tt >> 1;
+        if (use > 0 && !__all_sync(0xffffffffu, pwait(&pb->acc_empty[buf], (use - 1) & 1, abort_flag))) { ok = false; break; }
+        tc::tc_fence_after();
+        const int nn = h == 0 ? min(256, a.N) : a.N - 256;
+        const uint32_t idesc = tc::idesc_tf32(128, (uint32_t)nn);
+        const uint32_t d = tmem + buf * kBufCols;
+        for (int kc = 0; kc < chunks; ++kc, ++g) {
+          const uint32_t as = g % kStages, au = g / kStages;
+          const uint32_t bs = g % kBRing, bu = g / kBRing;
+          if (!pwait2(&pb->a_full[as], au & 1, &pb->b_full[bs], bu & 1, abort_flag)) {
+            ok = false;
+            break;
           }
-          if (!ok) break;
-          tc::mma_commit(&pb->acc_full[buf]);
+          tc::tc_fence_after();
+          const int seg0 = kc >= a.seg ? a.seg : 0;            // first chunk of the segment
+          const uint32_t ds = d + (seg0 > 0 ? kSegCols : 0u);
+          // start addresses (16-byte units) are the descriptors' low bits
+          const uint64_t ah = desc_a + as * (2 * kAStageFloats / 4), al = ah + kAStageFloats / 4;
+          const uint64_t bh = desc_b + bs * (2 * kBRingFloats / 4), bl = bh + nn * (kKc / 4);
+          if (kTA) {
+            const uint32_t ta = tmem + kTaBase + as * (2 * kKc);
+            if (issue) {
+              tc::mma_tf32_ta(ds, ta, bh, idesc, kc > seg0);
+              tc::mma_tf32_ta(ds, ta, bl, idesc, true);
+              tc::mma_tf32_ta(ds, ta + kKc, bh, idesc, true);
+              tc::mma_tf32_ta(ds, ta + 8, bh + 16, idesc, true);
+              tc::mma_tf32_ta(ds, ta + 8, bl + 16, idesc, true);
+              tc::mma_tf32_ta(ds, ta + kKc + 8, bh + 16, idesc, true);
+              tc::mma_commit(&pb->empty[bs]);
+            }
+          } else if (issue) {
+            tc::mma_tf32(ds, ah, bh, idesc, kc > seg0);
+            tc::mma_tf32(ds, ah, bl, idesc, true);
+            tc::mma_tf32(ds, al, bh, idesc, true);
+            tc::mma_tf32(ds, ah + 16, bh + 16, idesc, true);
+            tc::mma_tf32(ds, ah + 16, bl + 16, idesc, true);
+            tc::mma_tf32(ds, al + 16, bh + 16, idesc, true);
+            tc::mma_commit(&pb->empty[bs]);   // frees both operands
+          }
+          __syncwarp();
         }
+        if (!ok) break;
+        if (issue) tc::mma_commit(&pb->acc_full[buf]);
+        __syncwarp();
       }
-      if (!ok) {
-        pabort(pb, a.err);
-        // every MMA issued so far completes before tensor memory is freed: a commit after them
-        // completes the next phase of the current sub-tile's accumulator barrier
-        tc::mma_commit(&pb->acc_full[tt & 1]);
-        tc::mbar_wait(&pb->acc_full[tt & 1], (tt >> 1) & 1, kTries);
-      }
+    }
+    if (!ok && issue) {
+      pabort(pb, a.err);
+      // every MMA issued so far completes before tensor memory is freed: a commit after them
+      // completes the next phase of the current sub-tile's accumulator barrier
+      tc::mma_commit(&pb->acc_full[tt & 1]);
+      tc::mbar_wait(&pb->acc_full[tt & 1], (tt >> 1) & 1, kTries);
     }
   } else if (warp < 4) {  // converters: one row each
     const int rr = tid;
@@ -613,12 +664,22 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(Contr
       for (int h = 0; h < nsub && ok; ++h) {
         for (int kc = 0; kc < chunks; ++kc, ++g) {
           const uint32_t rs = g % kRawRing, ru = g / kRawRing;
-          const uint32_t as = g % kAStages, au = g / kAStages;
-          if (!pwait(&pb->raw_full[rs], ru & 1, abort_flag)) { ok = false; break; }
-          if (au > 0 && !pwait(&pb->a_empty[as], (au - 1) & 1, abort_flag)) { ok = false; break; }
-          float* A_hi = sA + as * 2 * kAStageFloats;
-          convert_row(a, r0 + rr < a.rows, kc, rr, raw + rs * kRawBytes, A_hi, A_hi + kAStageFloats);
-          tc::fence_proxy_async_smem();
+          const uint32_t as = g % kStages, gp = g - kStages;   // gp: the chunk that used the stage before
+          bool got = pwait(&pb->raw_full[rs], ru & 1, abort_flag);
+          if (got && g >= kStages) got = pwait(&pb->empty[gp % kBRing], (gp / kBRing) & 1, abort_flag);
+          if (kTA) got = __all_sync(0xffffffffu, got);   // the stores to tensor memory take whole warps
+          if (!got) { ok = false; break; }
+          float x[kKc];
+          load_row(a, r0 + rr < a.rows, kc, rr, raw + rs * kRawBytes, x);
+          if (kTA) {
+            tc::tc_fence_after();
+            store_row_tmem(x, tmem + kTaBase + as * (2 * kKc) + ((uint32_t)(32 * warp) << 16));
+            tc::tc_fence_before();
+          } else {
+            float* A_hi = sA + as * 2 * kAStageFloats;
+            store_row(x, rr, A_hi, A_hi + kAStageFloats);
+            tc::fence_proxy_async_smem();
+          }
           mbar_arrive(&pb->a_full[as]);
           mbar_arrive(&pb->raw_empty[rs]);
         }
@@ -653,7 +714,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(Contr
         int c0, c1;
         half_cols(h, &c0, &c1);
         const int64_t r = t * kRowsCta + 32 * q + lane;
-        const uint32_t tq = tmem + ((uint32_t)(32 * q) << 16) + buf * 256u;
+        const uint32_t tq = tmem + ((uint32_t)(32 * q) << 16) + buf * kBufCols;
         if (anal) {
           for (int c = c0; c < c1; c += 16) {
             double2 old[8];
@@ -672,7 +733,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(Contr
             tc::tmem_ld16(tq + (uint32_t)c, v);
             add_acc16(old, v);
             if (a.seg < chunks) {   // the tile's second segment
-              tc::tmem_ld16(tq + 128u + (uint32_t)c, v);
+              tc::tmem_ld16(tq + kSegCols + (uint32_t)c, v);
               add_acc16(old, v);
             }
             store_acc16(a, r, 256 * h + c, old);
@@ -696,10 +757,10 @@ __global__ void __launch_bounds__(kPipeThreads, 1) tc_contract_pipe_kernel(Contr
 __global__ void build_b_kernel(ContractArgs a, TileGeom g, const cpx<float>* __restrict__ tw,
                                const int64_t* __restrict__ pj, const float* __restrict__ cw, float* __restrict__ B) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= (int64_t)kMaxN * a.K) return;
+  if (e >= (int64_t)a.N * a.K) return;
   const int nrow = (int)(e / a.K), k = (int)(e % a.K);
   float val = 0.f;
-  if (nrow < a.N) {
+  {
     switch (a.mode) {
       case SYNTH_C: {
         const int tau = nrow >> 1, q = nrow & 1, j = k >> 1, part = k & 1;
@@ -738,10 +799,11 @@ __global__ void build_b_kernel(ContractArgs a, TileGeom g, const cpx<float>* __r
   }
   const float hi = tc::to_tf32(val);
   const int kc = k / kKc, kk = k % kKc;
-  float* chunk = B + (size_t)kc * 2 * kBStageFloats;
-  const uint32_t o = tc::kmajor_offset(nrow, kk, kKc) / 4;
-  chunk[o] = hi;
-  chunk[kBStageFloats + o] = val - hi;
+  const int h0 = nrow < 256 ? 0 : 256, nn = min(256, a.N - h0);
+  float* part = B + ((size_t)kc * a.N + h0) * 2 * kKc;
+  const uint32_t o = tc::kmajor_offset(nrow - h0, kk, kKc) / 4;
+  part[o] = hi;
+  part[(uint32_t)nn * kKc + o] = val - hi;
 }
 
 int round16(int x) { return (x + 15) / 16 * 16; }
@@ -791,7 +853,7 @@ bool raw_map_of(const ContractArgs& a, const TileGeom& g, rsv_operator op, CUten
 }
 
 cudaError_t run(ContractArgs& a, const TileGeom& g, rsv_operator op) {
-  const size_t bbytes = (size_t)(a.K / kKc) * 2 * kBStageFloats * sizeof(float);
+  const size_t bbytes = (size_t)a.K * 2 * a.N * sizeof(float);
   if (ensure(op->ws_tcb, bbytes) != RSV_OK) return cudaErrorMemoryAllocation;
   a.B = (const float*)op->ws_tcb.ptr;
   a.err = op->d_flag;
@@ -801,20 +863,22 @@ cudaError_t run(ContractArgs& a, const TileGeom& g, rsv_operator op) {
   const int chunks = a.K / kKc;
   const bool anal = a.mode == ANAL_C || a.mode == ANAL_R;
   a.seg = anal && a.N <= 128 && chunks > 16 ? std::max(16, (chunks + 1) / 2) : chunks;
-  const int64_t total = (int64_t)kMaxN * a.K;
+  const int64_t total = (int64_t)a.N * a.K;
   build_b_kernel<<<(unsigned)((total + 255) / 256), 256, 0, op->stream>>>(a, g, (const cpx<float>*)op->d_tw, op->d_pj,
                                                                           op->d_cw, (float*)op->ws_tcb.ptr);
   // the shared-memory opt-in is a per-device attribute: set it before every launch (cheap next
   // to a launch that moves gigabytes), so that any device and any thread gets it
   cudaError_t ae = cudaFuncSetAttribute(tc_contract_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-  if (ae == cudaSuccess)
-    ae = cudaFuncSetAttribute(tc_contract_pipe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem);
+  // the converted operand in tensor memory where the accumulators leave room for it
+  const bool ta = a.N <= (int)kTaCols;
+  auto* pipe = ta ? tc_contract_pipe_kernel<true> : tc_contract_pipe_kernel<false>;
+  if (ae == cudaSuccess) ae = cudaFuncSetAttribute(pipe, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPipeSmem);
   if (ae != cudaSuccess) return ae;
   const int64_t tiles = (a.rows + kRowsCta - 1) / kRowsCta;
   CUtensorMap map;
   if (raw_map_of(a, g, op, &map)) {
     const unsigned blocks = (unsigned)std::min<int64_t>(tiles, (int64_t)op->sm_count);
-    tc_contract_pipe_kernel<<<blocks, kPipeThreads, kPipeSmem, op->stream>>>(a, map);
+    pipe<<<blocks, kPipeThreads, kPipeSmem, op->stream>>>(a, map);
   } else {
     tc_contract_kernel<<<(unsigned)tiles, 256, kSmem, op->stream>>>(a);
   }
