@@ -184,17 +184,24 @@ __global__ void __launch_bounds__(256, 1) dense_tc_step_kernel(TcStepArgs a) {
 // (32 real columns), each driven by its own four warps with its own operand
 // buffer, mbarriers, tensor-memory columns and counters, so one chain's
 // hand-off latency overlaps the other chain's work.  Per chain and step:
-//   1. wait until row blocks 2j and 2j+1 have published the state (counter),
-//      bulk-copy the TF32 hi / lo split of the state slice (32 KB);
+//   1. wait until row blocks 2j and 2j+1 have published the state (counters), each by
+//      a warp of its own, which bulk-copies that K half of the TF32 hi / lo split of
+//      the state slice (16 KB);
 //   2. two MMAs per K-step: A_hi x [X_hi | X_lo] (N = 64) and A_lo x X_hi
 //      (N = 32), so the A tile is read from shared memory twice, not three times;
+//      the first half's run while the second half arrives;
 //   3. sum the three product groups out of tensor memory into the CTA's
-//      128 x 32 partial, store it (L2) and count it in the row block's counter;
+//      128 x 32 partial, store it (L2, four columns of all rows side by side, so that
+//      stores and loads fill whole sectors) and count it in the row block's counter;
 //   4. as owner of 64/CS rows of its row block, wait for all CS partials of the
-//      step, bulk-copy its rows of them into shared memory (16 KB), sum them,
-//      apply the RK4 update u <- u + D u + F (the owner keeps
-//      its rows of u in registers for the whole tile), write the snapshot and
-//      the hi / lo split of the new state, and count the publication.
+//      step, load its rows of them, all in flight at once, sum them, apply the RK4
+//      update u <- u + D u + F (the owner keeps its rows of u in registers for the
+//      whole tile), write the snapshot and the hi / lo split of the new state in
+//      16-byte pieces, and count the publication.
+// A step is a chain of latencies (two hand-offs through L2, about 6.7 us at n = 1024
+// with 32 vectors; 8.1 us with the partials fetched by 16 bulk copies of one thread,
+// about 94 cycles each to issue, both row blocks polled in turn by the thread that
+// issues the products, and products issued by a lone lane).
 // Partials, split states and counter targets are double-buffered by step
 // parity: every row block reads every K slice, so no CTA runs more than one
 // step ahead of any other within a chain.  Counters only grow (zeroed at the
@@ -206,14 +213,14 @@ constexpr int kChainN = 2 * kChainVec;               // real columns per chain (
 constexpr int kMaxChains = 2;
 constexpr uint32_t kXcFloats = 2 * kChainN * kTileK; // hi rows [0, 32) then lo rows [32, 64): 8192 floats
 constexpr uint32_t kPartFloats = kM * kChainN;       // 128 x 32 partial of one CTA
-constexpr uint32_t kGFloats = 2 * kTileRows * kChainN;   // the owner's rows of all CS partials: 16 KB
-constexpr uint32_t kSmemPersistent = 4 * (2 * kATileFloats + kMaxChains * (kXcFloats + kGFloats)) + 256;
+constexpr uint32_t kXhFloats = kXcFloats / 2;        // one of its K halves, [64 rows x 64 columns] K-major
+constexpr uint32_t kSmemPersistent = 4 * (2 * kATileFloats + kMaxChains * kXcFloats) + 256;
 constexpr int kMarchThreads = 128 * kMaxChains;
 
 struct TcMarchArgs {
   const float* A;
-  float* X;                 // [chains][2][CS][kXcFloats]
-  float* part;              // [chains][2][MB][CS][kPartFloats]
+  float* X;                 // [chains][2][CS][2 K halves][kXhFloats]
+  float* part;              // [chains][2][MB][CS][kChainN / 4][kM][4]
   int* cnt;                 // [chains][2][MB]  partials stored
   int* ready;               // [chains][MB]     owner publications
   cpx<float>* u;            // [2][kg][n]: state at n0 in slot n0 & 1, written back to slot (n0 + steps) & 1
@@ -238,11 +245,11 @@ __global__ void __launch_bounds__(kMarchThreads, 1) dense_tc_march_kernel(TcMarc
   float* A_hi = reinterpret_cast<float*>(smem);
   float* A_lo = A_hi + kATileFloats;
   float* Xs = A_lo + kATileFloats;                                          // [chain][kXcFloats]
-  float* Gs = Xs + kMaxChains * kXcFloats;                                  // [chain][kGFloats]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(Gs + kMaxChains * kGFloats);  // [0] A, then 3 per chain
+  uint64_t* bars = reinterpret_cast<uint64_t*>(Xs + kMaxChains * kXcFloats);   // [0] A, then 3 per chain
   uint32_t* tbase = reinterpret_cast<uint32_t*>(bars + 1 + 3 * kMaxChains);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // known to be the warp's: uniform registers
   const int chain = warp >> 2;                  // warps 4c .. 4c + 3 drive chain c
   const int ctid = tid & 127;                   // thread index within the chain
   const int MB = a.n / kTileRows;
@@ -268,10 +275,8 @@ __global__ void __launch_bounds__(kMarchThreads, 1) dense_tc_march_kernel(TcMarc
   __syncthreads();
   if (chain < a.chains) {
     float* X_sm = Xs + (size_t)chain * kXcFloats;
-    uint64_t* bar_x = &bars[1 + 3 * chain];
-    uint64_t* bar_m = &bars[2 + 3 * chain];
-    uint64_t* bar_g = &bars[3 + 3 * chain];
-    float* G_sm = Gs + (size_t)chain * kGFloats;   // [CS][re rows, im rows][rpc][kChainN]
+    uint64_t* bar_x = &bars[1 + 3 * chain];       // one per K half
+    uint64_t* bar_m = &bars[3 + 3 * chain];
     const uint32_t tcol = tmem + (uint32_t)(chain * 128);
     const size_t xset = (size_t)a.cs * kXcFloats;                // one parity
     float* Xg = a.X + (size_t)chain * 2 * xset;
@@ -282,36 +287,50 @@ __global__ void __launch_bounds__(kMarchThreads, 1) dense_tc_march_kernel(TcMarc
     const int v0 = chain * kChainVec;
     const uint32_t idesc_hx = tc::idesc_tf32(kM, 2 * kChainN);   // A_hi x [X_hi | X_lo]
     const uint32_t idesc_lx = tc::idesc_tf32(kM, kChainN);       // A_lo x X_hi
-    const uint32_t sbo = (kTileK / 4) * 128;
-    // owner pairs: rows [rpc j, rpc j + rpc) of the row block x 16 vectors, kPairs per thread
+    // owner pairs: rows [rpc j, rpc j + rpc) of the row block x 16 vectors; a warp holds 4 consecutive rows
+    // x 8 vectors of each group of 8 rows
     const int rpc = kTileRows / a.cs;
-    const int npairs = rpc * kChainVec;
+    const int groups = rpc / 8;
     constexpr int kMaxPairs = kTileRows * kChainVec / 128;       // 8 (cs = 1)
-    const int vl = ctid & 15;
+    const int sub = lane >> 3;                                    // row within the four
+    const int vl = 8 * ((warp >> 1) & 1) + (lane & 7);
     const int vg = v0 + vl;
+    const int il0 = rpc * j + 4 * (warp & 1) + sub;               // row of group 0 in the row block
     cpx<float> u_own[kMaxPairs];
 #pragma unroll
     for (int q = 0; q < kMaxPairs; ++q) {
-      const int pidx = ctid + 128 * q;
-      const int i = mb * kTileRows + rpc * j + (pidx >> 4);
-      u_own[q] = (pidx < npairs && vg < a.kg) ? a.u[(size_t)(a.n0 & 1) * rows + (int64_t)vg * a.n + i]
+      const int i = mb * kTileRows + il0 + 8 * q;
+      u_own[q] = (q < groups && vg < a.kg) ? a.u[(size_t)(a.n0 & 1) * rows + (int64_t)vg * a.n + i]
                                                : mk<float>(0.f, 0.f);
     }
-    // X slot layout: hi rows [0, 32) (re of 16 vectors, then im), lo rows [32, 64)
+    // X slot layout: hi rows [0, 32) (re of 16 vectors, then im), lo rows [32, 64), in each K half.  The four
+    // lanes of a vector swap their four values, so that each stores one row's 16 bytes.
     auto write_x = [&](float* xo_par, int i, cpx<float> u1) {
-      const int js = i / kTileK, kk = i % kTileK;
-      float* xo = xo_par + (size_t)js * kXcFloats;
       const float hr = tc::to_tf32(u1.re), hi = tc::to_tf32(u1.im);
-      __stcg(xo + tc::kmajor_offset(vl, kk, kTileK) / 4, hr);
-      __stcg(xo + tc::kmajor_offset(kChainVec + vl, kk, kTileK) / 4, hi);
-      __stcg(xo + tc::kmajor_offset(kChainN + vl, kk, kTileK) / 4, u1.re - hr);
-      __stcg(xo + tc::kmajor_offset(kChainN + kChainVec + vl, kk, kTileK) / 4, u1.im - hi);
+      const float val[4] = {hr, hi, u1.re - hr, u1.im - hi};
+      float got[4];   // from lane sub ^ r
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int w = sub ^ r;
+        const float lo2 = (w & 1) ? val[1] : val[0], hi2 = (w & 1) ? val[3] : val[2];
+        got[r] = __shfl_xor_sync(0xffffffffu, (w & 2) ? hi2 : lo2, 8 * r);
+      }
+      float out[4];   // out[t] = got[t ^ sub]
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const float lo2 = (sub & 1) ? got[t ^ 1] : got[t];
+        const float hi2 = (sub & 1) ? got[(t ^ 3) & 3] : got[(t ^ 2) & 3];
+        out[t] = (sub & 2) ? hi2 : lo2;
+      }
+      const int js = i / kTileK, kk = i % kTileK;
+      float* xo = xo_par + (size_t)js * kXcFloats + (kk >> 6) * kXhFloats;
+      __stcg(reinterpret_cast<float4*>(xo + tc::kmajor_offset(kChainVec * sub + vl, (kk & 63) & ~3, kTileK / 2) / 4),
+             make_float4(out[0], out[1], out[2], out[3]));
     };
     if (a.n0 == 0) {  // publish the initial state's split (later tiles find it from the previous tile)
 #pragma unroll
       for (int q = 0; q < kMaxPairs; ++q) {
-        const int pidx = ctid + 128 * q;
-        if (pidx < npairs) write_x(Xg, mb * kTileRows + rpc * j + (pidx >> 4), u_own[q]);
+        if (q < groups) write_x(Xg, mb * kTileRows + il0 + 8 * q, u_own[q]);
       }
       chain_bar(chain);
       if (ctid == 0) tc::red_release_add(&ready[mb], 1);
@@ -326,44 +345,52 @@ __global__ void __launch_bounds__(kMarchThreads, 1) dense_tc_march_kernel(TcMarc
       cpx<float> fv[kMaxPairs];
 #pragma unroll
       for (int q = 0; q < kMaxPairs; ++q) {
-        const int pidx = ctid + 128 * q;
-        const int i = mb * kTileRows + rpc * j + (pidx >> 4);
-        fv[q] = (Fs != nullptr && pidx < npairs && vg < a.kg)
+        const int i = mb * kTileRows + il0 + 8 * q;
+        fv[q] = (Fs != nullptr && q < groups && vg < a.kg)
                     ? mk<float>(__ldcs(reinterpret_cast<const float*>(Fs + (int64_t)vg * a.n + i)),
                                 __ldcs(reinterpret_cast<const float*>(Fs + (int64_t)vg * a.n + i) + 1))
                     : mk<float>(0.f, 0.f);
       }
-      // 1. the state slice of this step
-      if (ctid == 0) {
-        const int target = a.cs * (int)(n + 1) + ((a.stall && s == 0) ? (1 << 30) : 0);
-        const bool got = tc::spin_until_geq(&ready[2 * j], target, errv, a.wait_ns) &&
-                         tc::spin_until_geq(&ready[2 * j + 1], target, errv, a.wait_ns);
-        if (!got) {
-          atomicExch(a.err, 2);
-          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar_x)) : "memory");
-        } else {
-          tc::fence_proxy_async_global();
-          tc::mbar_arrive_expect_tx(bar_x, 4 * kXcFloats);
-          tc::bulk_g2s(X_sm, Xg + (size_t)par * xset + (size_t)j * kXcFloats, 4 * kXcFloats, bar_x);
-        }
-      }
-      // 2. products
-      if (ctid == 0) {
-        bool okx = tc::mbar_wait(bar_x, (uint32_t)(s & 1), 0xFFFFFFFFu) && *errv == 0;
-        tc::tc_fence_after();
-        if (okx) {
-#pragma unroll 4
-          for (int ks = 0; ks < kTileK / 8; ++ks) {
-            const uint64_t ah = tc::smem_desc(reinterpret_cast<char*>(A_hi) + ks * 256, 128, sbo);
-            const uint64_t al = tc::smem_desc(reinterpret_cast<char*>(A_lo) + ks * 256, 128, sbo);
-            const uint64_t xx = tc::smem_desc(reinterpret_cast<char*>(X_sm) + ks * 256, 128, sbo);
-            tc::mma_tf32(tcol, ah, xx, idesc_hx, ks > 0);
-            tc::mma_tf32(tcol + 2 * kChainN, al, xx, idesc_lx, ks > 0);
+      // 1. the state slice of this step: a row block's columns are one K half, fetched by one of two warps
+      const int wc = warp & 3;
+      if (wc < 2) {
+        if (lane == 0) {
+          const int target = a.cs * (int)(n + 1) + ((a.stall && s == 0) ? (1 << 30) : 0);
+          if (!tc::spin_until_geq(&ready[2 * j + wc], target, errv, a.wait_ns)) {
+            atomicExch(a.err, 2);
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar_x + wc)) : "memory");
+          } else {
+            tc::fence_proxy_async_global();
+            tc::mbar_arrive_expect_tx(bar_x + wc, 4 * kXhFloats);
+            tc::bulk_g2s(X_sm + wc * kXhFloats, Xg + (size_t)par * xset + (size_t)j * kXcFloats + wc * kXhFloats,
+                         4 * kXhFloats, bar_x + wc);
           }
-          tc::mma_commit(bar_m);
-        } else {
-          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar_m)) : "memory");
         }
+        __syncwarp();
+      }
+      // 2. products, issued by a converged warp (descriptors in uniform registers)
+      if (wc == 0) {
+        const uint64_t ah = tc::smem_desc(A_hi, 128, (kTileK / 4) * 128), al = tc::smem_desc(A_lo, 128, (kTileK / 4) * 128);
+        const uint64_t xx = tc::smem_desc(X_sm, 128, (kTileK / 8) * 128);
+        bool okx = true;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          okx = tc::mbar_wait(bar_x + h, (uint32_t)(s & 1), 0xFFFFFFFFu) && okx;
+          if (__all_sync(0xffffffffu, okx && *errv == 0)) {
+            tc::tc_fence_after();
+            if (lane == 0) {
+#pragma unroll
+              for (int ks = 0; ks < kTileK / 16; ++ks) {
+                const uint64_t x = xx + h * (kXhFloats / 4) + ks * 16;
+                tc::mma_tf32(tcol, ah + (8 * h + ks) * 16, x, idesc_hx, h + ks > 0);
+                tc::mma_tf32(tcol + 2 * kChainN, al + (8 * h + ks) * 16, x, idesc_lx, h + ks > 0);
+              }
+            }
+            __syncwarp();
+          }
+        }
+        if (lane == 0) tc::mma_commit(bar_m);
+        __syncwarp();
       }
       ok = tc::mbar_wait(bar_m, (uint32_t)(s & 1), 0xFFFFFFFFu) && ok && *errv == 0;
       tc::tc_fence_after();
@@ -373,62 +400,42 @@ __global__ void __launch_bounds__(kMarchThreads, 1) dense_tc_march_kernel(TcMarc
         const int qw = warp & 3;
         const int row = 32 * qw + lane;
         const uint32_t tl = tcol + ((uint32_t)(32 * qw) << 16);
+        float x0[32], x1[32], x2[32];
+        tc::tmem_ld32(tl, x0);
+        tc::tmem_ld32(tl + kChainN, x1);
+        tc::tmem_ld32(tl + 2 * kChainN, x2);
+        float4* dst = reinterpret_cast<float4*>(pb) + row;   // four columns of all rows side by side
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          float x0[16], x1[16], x2[16];
-          tc::tmem_ld16(tl + 16 * h, x0);
-          tc::tmem_ld16(tl + kChainN + 16 * h, x1);
-          tc::tmem_ld16(tl + 2 * kChainN + 16 * h, x2);
-          float4* dst = reinterpret_cast<float4*>(pb + row * kChainN + 16 * h);
-#pragma unroll
-          for (int c = 0; c < 4; ++c)
-            __stcg(dst + c, make_float4(x0[4 * c] + x1[4 * c] + x2[4 * c], x0[4 * c + 1] + x1[4 * c + 1] + x2[4 * c + 1],
-                                        x0[4 * c + 2] + x1[4 * c + 2] + x2[4 * c + 2],
-                                        x0[4 * c + 3] + x1[4 * c + 3] + x2[4 * c + 3]));
-        }
+        for (int c = 0; c < kChainN / 4; ++c)
+          __stcg(dst + c * kM, make_float4(x0[4 * c] + x1[4 * c] + x2[4 * c], x0[4 * c + 1] + x1[4 * c + 1] + x2[4 * c + 1],
+                                           x0[4 * c + 2] + x1[4 * c + 2] + x2[4 * c + 2],
+                                           x0[4 * c + 3] + x1[4 * c + 3] + x2[4 * c + 3]));
       }
       tc::tc_fence_before();
       chain_bar(chain);
       if (ctid == 0) tc::red_release_add(&cnt[par * MB + mb], 1);
-      // 4. owner: all partials of the row block for this step; the owner's rows of every
-      //    partial (rpc real-part rows and rpc imaginary-part rows) come in by bulk copies
+      // 4. owner: its rows of all partials of the row block for this step
       const float* pbase = partg + ((size_t)par * MB + mb) * a.cs * kPartFloats;
-      if (ctid == 0) {
-        if (!tc::spin_until_geq(&cnt[par * MB + mb], a.cs * (int)((n >> 1) + 1), errv, a.wait_ns)) {
-          atomicExch(a.err, 2);
-          asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar_g)) : "memory");
-        } else {
-          tc::fence_proxy_async_global();
-          const uint32_t rows_bytes = (uint32_t)rpc * kChainN * 4;
-          tc::mbar_arrive_expect_tx(bar_g, 2u * (uint32_t)a.cs * rows_bytes);
-          for (int p = 0; p < a.cs; ++p) {
-            const float* src = pbase + (size_t)p * kPartFloats;
-            float* dst = G_sm + (size_t)p * 2 * rpc * kChainN;
-            tc::bulk_g2s(dst, src + (size_t)(rpc * j) * kChainN, rows_bytes, bar_g);
-            tc::bulk_g2s(dst + rpc * kChainN, src + (size_t)(64 + rpc * j) * kChainN, rows_bytes, bar_g);
-          }
-        }
-      }
-      if (!tc::mbar_wait(bar_g, (uint32_t)(s & 1), 0xFFFFFFFFu)) atomicExch(a.err, 2);
+      if (ctid == 0 && !tc::spin_until_geq(&cnt[par * MB + mb], a.cs * (int)((n >> 1) + 1), errv, a.wait_ns))
+        atomicExch(a.err, 2);
+      chain_bar(chain);
       cpx<float>* Ys = (a.Y != nullptr && s >= a.y_first) ? a.Y + (size_t)s * rows : nullptr;
       float* xo_par = Xg + (size_t)(1 - par) * xset;
 #pragma unroll
       for (int q = 0; q < kMaxPairs; ++q) {
-        const int pidx = ctid + 128 * q;
-        if (pidx < npairs) {
-          const int il = pidx >> 4;
-          const int iloc = rpc * j + il;
+        if (q < groups) {
+          const int iloc = il0 + 8 * q;
           float prr = 0.f, pri = 0.f, pir = 0.f, pii = 0.f;
           float t0[8], t1[8], t2[8], t3[8];
+          // columns [0, 16) times Ur, [16, 32) times Ui; rows iloc real, 64 + iloc imaginary part of D
+          const float* g = pbase + (size_t)((vl >> 2) * kM + iloc) * 4 + (vl & 3);
 #pragma unroll
           for (int p = 0; p < 8; ++p) {
             if (p < a.cs) {
-              const float* gr = G_sm + (size_t)p * 2 * rpc * kChainN + il * kChainN;
-              const float* gi = gr + rpc * kChainN;
-              t0[p] = gr[vl];
-              t1[p] = gr[kChainVec + vl];
-              t2[p] = gi[vl];
-              t3[p] = gi[kChainVec + vl];
+              t0[p] = __ldcg(g + (size_t)p * kPartFloats);
+              t1[p] = __ldcg(g + (size_t)p * kPartFloats + 4 * kM * 4);
+              t2[p] = __ldcg(g + (size_t)p * kPartFloats + 64 * 4);
+              t3[p] = __ldcg(g + (size_t)p * kPartFloats + 4 * kM * 4 + 64 * 4);
             }
           }
 #pragma unroll
@@ -456,9 +463,8 @@ __global__ void __launch_bounds__(kMarchThreads, 1) dense_tc_march_kernel(TcMarc
     const int64_t nend = a.n0 + a.steps;
 #pragma unroll
     for (int q = 0; q < kMaxPairs; ++q) {
-      const int pidx = ctid + 128 * q;
-      const int i = mb * kTileRows + rpc * j + (pidx >> 4);
-      if (pidx < npairs && vg < a.kg) a.u[(size_t)(nend & 1) * rows + (int64_t)vg * a.n + i] = u_own[q];
+      const int i = mb * kTileRows + il0 + 8 * q;
+      if (q < groups && vg < a.kg) a.u[(size_t)(nend & 1) * rows + (int64_t)vg * a.n + i] = u_own[q];
     }
   }
   tc::tc_fence_before();
