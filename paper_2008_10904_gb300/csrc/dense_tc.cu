@@ -180,49 +180,44 @@ __global__ void __launch_bounds__(256, 1) dense_tc_step_kernel(TcStepArgs a) {
 // MB * CS CTAs, one per SM, all resident at once.  CTA (mb, j) keeps the A
 // tile of row block mb and K slice j in shared memory for the whole tile.
 //
-// The test vectors are split into up to two independent chains of 16 vectors
-// (32 real columns), each driven by its own four warps with its own operand
-// buffer, mbarriers, tensor-memory columns and counters, so one chain's
-// hand-off latency overlaps the other chain's work.  Per chain and step:
-//   1. wait until row blocks 2j and 2j+1 have published the state (counters), each by
-//      a warp of its own, which bulk-copies that K half of the TF32 hi / lo split of
-//      the state slice (16 KB);
-//   2. two MMAs per K-step: A_hi x [X_hi | X_lo] (N = 64) and A_lo x X_hi
-//      (N = 32), so the A tile is read from shared memory twice, not three times;
-//      the first half's run while the second half arrives;
-//   3. sum the three product groups out of tensor memory into the CTA's
-//      128 x 32 partial, store it (L2, four columns of all rows side by side, so that
-//      stores and loads fill whole sectors) and count it in the row block's counter;
-//   4. as owner of 64/CS rows of its row block, wait for all CS partials of the
-//      step, load its rows of them, all in flight at once, sum them, apply the RK4
-//      update u <- u + D u + F (the owner keeps its rows of u in registers for the
-//      whole tile), write the snapshot and the hi / lo split of the new state in
-//      16-byte pieces, and count the publication.
-// A step is a chain of latencies (two hand-offs through L2, about 6.7 us at n = 1024
-// with 32 vectors; 8.1 us with the partials fetched by 16 bulk copies of one thread,
-// about 94 cycles each to issue, both row blocks polled in turn by the thread that
-// issues the products, and products issued by a lone lane).
-// Partials, split states and counter targets are double-buffered by step
-// parity: every row block reads every K slice, so no CTA runs more than one
-// step ahead of any other within a chain.  Counters only grow (zeroed at the
-// start of a march).  Spins are bounded in time and stop once any CTA has set
-// the error flag.
+// Two hand-offs per step pass through L2: the partial sums of a row block's CS
+// CTAs to the owners of its rows, and the owners' new state to the CTAs of its
+// K slice.  Every value travels with the number of its step in one 8-byte word
+// (16-byte accesses carry two of them), and the receiver loads until the numbers
+// are right: no counter, no fence and no copy stands between a store and the load
+// that wants it.  Per step, with C = 32 or 64 real columns (16 or 32 vectors):
+//   1. the eight worker warps load the state slice (128 x C), split it into TF32
+//      hi / lo and store it as the K-major operand, one K half after the other;
+//   2. warp 8 issues two MMAs per K-step, A_hi x [X_hi | X_lo] (N = 2 C) and
+//      A_lo x X_hi (N = C), the first half's while the second is converted: the A
+//      tile is read from shared memory twice, for all vectors at once;
+//   3. the workers sum the three product groups out of tensor memory and store the
+//      CTA's 128 x C partial;
+//   4. as owner of 64/CS rows of its row block, each thread loads its rows of the
+//      CS partials, all in flight at once, sums them in order, applies the RK4
+//      update u <- u + D u + F (u stays in registers for the whole tile), writes
+//      the snapshot and the new state.
+// Both buffers alternate by step parity.  A CTA stores step n + 2's values only
+// after it has received the state n + 2, which depends on every CTA's partials of
+// step n + 1 and those on every owner's state n + 1: all loads of step n are over.
+// The numbers start at 1; the buffers are zeroed at the start of a march.  Loads
+// that wait are bounded in time and stop once any CTA has set the error flag.
+// A step is a chain of latencies: n = 1024, 32 vectors, 13188 steps march in
+// 66 ms.  With counters (fence, add, poll and bulk copy per hand-off) and two
+// chains of 16 vectors that took turns on the tensor cores 88 ms; of 6.7 us per
+// step 1.4 us were fences, 1.8 us polls and 2 us products.
 // ---------------------------------------------------------------------------
-constexpr int kChainVec = 16;                        // vectors per chain
-constexpr int kChainN = 2 * kChainVec;               // real columns per chain (re, im)
-constexpr int kMaxChains = 2;
-constexpr uint32_t kXcFloats = 2 * kChainN * kTileK; // hi rows [0, 32) then lo rows [32, 64): 8192 floats
-constexpr uint32_t kPartFloats = kM * kChainN;       // 128 x 32 partial of one CTA
-constexpr uint32_t kXhFloats = kXcFloats / 2;        // one of its K halves, [64 rows x 64 columns] K-major
-constexpr uint32_t kSmemPersistent = 4 * (2 * kATileFloats + kMaxChains * kXcFloats) + 256;
-constexpr int kMarchThreads = 128 * kMaxChains;
+constexpr int kMaxCols = 64;                               // real columns: (re, im) of 32 vectors
+constexpr int kWorkers = 256;
+constexpr int kMarchThreads = kWorkers + 32;               // and the warp that issues the products
+constexpr uint32_t kXsFloats = kTileK * kMaxCols * 2;      // a slice's words: [K / 2][C] x 2 (value, number)
+constexpr uint32_t kPartFloats = kM * kMaxCols * 2;        // a partial's words: [C / 2][128 rows] x 2
+constexpr uint32_t kSmemPersistent = 4 * (2 * kATileFloats + 2 * kMaxCols * kTileK) + 256;
 
 struct TcMarchArgs {
   const float* A;
-  float* X;                 // [chains][2][CS][2 K halves][kXhFloats]
-  float* part;              // [chains][2][MB][CS][kChainN / 4][kM][4]
-  int* cnt;                 // [chains][2][MB]  partials stored
-  int* ready;               // [chains][MB]     owner publications
+  float* X;                 // [2][CS][kXsFloats]
+  float* part;              // [2][MB][CS][kPartFloats]
   cpx<float>* u;            // [2][kg][n]: state at n0 in slot n0 & 1, written back to slot (n0 + steps) & 1
   const cpx<float>* F;      // [steps][kg][n] or null
   cpx<float>* Y;            // [steps][kg][n] or null
@@ -230,34 +225,71 @@ struct TcMarchArgs {
   int steps;
   int64_t n_forced;
   int y_first;
-  int n, kg, cs, chains;
+  int n, kg, cs;
   int* err;
-  uint64_t wait_ns;         // limit of each wait on another CTA's counter
-  int stall;                // test hook: the first state wait of the tile targets a count nobody reaches
+  uint64_t wait_ns;         // limit of each wait on another CTA's values
+  int stall;                // test hook: the first state wait of the tile wants a number nobody writes
 };
 
-__device__ __forceinline__ void chain_bar(int chain) {
-  asm volatile("bar.sync %0, 128;" ::"r"(1 + chain) : "memory");
+// Two (value, number) words, each of them one access of 8 bytes.
+__device__ __forceinline__ void words_store(float* p, float v0, float v1, uint32_t number) {
+  const uint64_t hi = (uint64_t)number << 32;
+  asm volatile("st.relaxed.gpu.global.v2.b64 [%0], {%1, %2};" ::"l"(p), "l"(hi | __float_as_uint(v0)),
+               "l"(hi | __float_as_uint(v1))
+               : "memory");
+}
+__device__ __forceinline__ void words_load(const float* p, uint64_t w[2]) {
+  asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(w[0]), "=l"(w[1]) : "l"(p) : "memory");
+}
+__device__ __forceinline__ float word_value(uint64_t w) { return __uint_as_float((uint32_t)w); }
+
+// Load again what has not got its number yet, until all have; false on the time limit or another CTA's error.
+template <int M, typename At>
+__device__ __forceinline__ bool words_wait(uint64_t (*w)[2], int count, uint32_t number, At at, const volatile int* err,
+                                           uint64_t limit_ns) {
+  uint64_t t0 = 0;
+  for (uint32_t tries = 0;; ++tries) {
+    bool all = true;
+#pragma unroll
+    for (int i = 0; i < M; ++i) {
+      if (i < count && ((uint32_t)(w[i][0] >> 32) != number || (uint32_t)(w[i][1] >> 32) != number)) {
+        all = false;
+        words_load(at(i), w[i]);
+      }
+    }
+    if (all) return true;
+    if ((tries & 15) == 15) {
+      if (*err != 0) return false;
+      const uint64_t now = tc::global_ns();
+      if (t0 == 0) t0 = now;
+      else if (now - t0 > limit_ns) return false;
+    }
+  }
 }
 
+template <int C, int kMaxGroups>   // real columns; groups of eight owner rows at most (1: CS = 8)
 __global__ void __launch_bounds__(kMarchThreads, 1) dense_tc_march_kernel(TcMarchArgs a) {
   extern __shared__ __align__(1024) unsigned char smem[];
   float* A_hi = reinterpret_cast<float*>(smem);
   float* A_lo = A_hi + kATileFloats;
-  float* Xs = A_lo + kATileFloats;                                          // [chain][kXcFloats]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(Xs + kMaxChains * kXcFloats);   // [0] A, then 3 per chain
-  uint32_t* tbase = reinterpret_cast<uint32_t*>(bars + 1 + 3 * kMaxChains);
+  float* X_sm = A_lo + kATileFloats;                                    // [K half][hi rows [0, C), lo rows [C, 2 C)][64]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(X_sm + 2 * kMaxCols * kTileK);   // A; X halves; products
+  uint32_t* tbase = reinterpret_cast<uint32_t*>(bars + 4);
+  volatile int* dead = reinterpret_cast<volatile int*>(tbase + 1);   // a wait of this CTA has run out: no values from here on
+  constexpr uint32_t kHalf = 2 * C * (kTileK / 2);                       // floats of a K half of the operand
 
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // known to be the warp's: uniform registers
-  const int chain = warp >> 2;                  // warps 4c .. 4c + 3 drive chain c
-  const int ctid = tid & 127;                   // thread index within the chain
   const int MB = a.n / kTileRows;
   const int mb = blockIdx.x / a.cs;
   const int j = blockIdx.x % a.cs;
   const volatile int* errv = a.err;
   if (tid == 0) {
-    for (int b = 0; b < 1 + 3 * kMaxChains; ++b) tc::mbar_init(&bars[b], 1);
+    tc::mbar_init(&bars[0], 1);
+    tc::mbar_init(&bars[1], kWorkers / 32);
+    tc::mbar_init(&bars[2], kWorkers / 32);
+    tc::mbar_init(&bars[3], 1);
+    *dead = 0;
     tc::fence_mbar_init();
   }
   if (warp == 0) tc::tmem_alloc(tbase, 256);
@@ -273,206 +305,214 @@ __global__ void __launch_bounds__(kMarchThreads, 1) dense_tc_march_kernel(TcMarc
   }
   bool ok = tc::mbar_wait(&bars[0], 0, 0xFFFFFFFFu);   // this CTA's own copy: never abandoned early
   __syncthreads();
-  if (chain < a.chains) {
-    float* X_sm = Xs + (size_t)chain * kXcFloats;
-    uint64_t* bar_x = &bars[1 + 3 * chain];       // one per K half
-    uint64_t* bar_m = &bars[3 + 3 * chain];
-    const uint32_t tcol = tmem + (uint32_t)(chain * 128);
-    const size_t xset = (size_t)a.cs * kXcFloats;                // one parity
-    float* Xg = a.X + (size_t)chain * 2 * xset;
-    float* partg = a.part + (size_t)chain * 2 * MB * a.cs * kPartFloats;
-    int* cnt = a.cnt + chain * 2 * MB;
-    int* ready = a.ready + chain * MB;
+  uint64_t* bar_x = &bars[1];       // one per K half
+  uint64_t* bar_m = &bars[3];
+  const uint64_t own_ns = 2 * a.wait_ns + tc::kWaitLimitNs;   // waits on this CTA's own warps outlast theirs on others
+
+  if (warp == kWorkers / 32) {
+    // 2. products, issued by a converged warp (descriptors in uniform registers)
+    const uint32_t idesc_hx = tc::idesc_tf32(kM, 2 * C);   // A_hi x [X_hi | X_lo]
+    const uint32_t idesc_lx = tc::idesc_tf32(kM, C);       // A_lo x X_hi
+    const uint64_t ah = tc::smem_desc(A_hi, 128, (kTileK / 4) * 128), al = tc::smem_desc(A_lo, 128, (kTileK / 4) * 128);
+    const uint64_t xx = tc::smem_desc(X_sm, 128, (kTileK / 8) * 128);
+    for (int s = 0; s < a.steps; ++s) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const bool here = tc::mbar_wait(bar_x + h, (uint32_t)(s & 1), 0xFFFFFFFFu, nullptr, own_ns);
+        ok = __all_sync(0xffffffffu, here) && ok;
+        tc::tc_fence_after();
+        if (ok && lane == 0 && *dead == 0) {
+#pragma unroll
+          for (int ks = 0; ks < kTileK / 16; ++ks) {
+            const uint64_t x = xx + h * (kHalf / 4) + ks * 16;
+            tc::mma_tf32(tmem, ah + (8 * h + ks) * 16, x, idesc_hx, h + ks > 0);
+            tc::mma_tf32(tmem + 2 * C, al + (8 * h + ks) * 16, x, idesc_lx, h + ks > 0);
+          }
+        }
+        __syncwarp();
+      }
+      if (lane == 0) tc::mma_commit(bar_m);
+      __syncwarp();
+    }
+  } else {
     const int64_t rows = (int64_t)a.kg * a.n;
-    const int v0 = chain * kChainVec;
-    const uint32_t idesc_hx = tc::idesc_tf32(kM, 2 * kChainN);   // A_hi x [X_hi | X_lo]
-    const uint32_t idesc_lx = tc::idesc_tf32(kM, kChainN);       // A_lo x X_hi
-    // owner pairs: rows [rpc j, rpc j + rpc) of the row block x 16 vectors; a warp holds 4 consecutive rows
-    // x 8 vectors of each group of 8 rows
-    const int rpc = kTileRows / a.cs;
-    const int groups = rpc / 8;
-    constexpr int kMaxPairs = kTileRows * kChainVec / 128;       // 8 (cs = 1)
-    const int sub = lane >> 3;                                    // row within the four
-    const int vl = 8 * ((warp >> 1) & 1) + (lane & 7);
-    const int vg = v0 + vl;
-    const int il0 = rpc * j + 4 * (warp & 1) + sub;               // row of group 0 in the row block
-    cpx<float> u_own[kMaxPairs];
+    // owner pairs: rows [rpc j, rpc j + rpc) of the row block, eight at a time, x 16 or 32 vectors
+    const int groups = kTileRows / a.cs / 8;
+    const int vg = 4 * warp + (lane >> 3);
+    const bool owner = 4 * warp < C / 2;                          // a whole warp
+    const int il0 = (kTileRows / a.cs) * j + (lane & 7);          // row of group 0 in the row block
+    cpx<float> u_own[kMaxGroups];
 #pragma unroll
-    for (int q = 0; q < kMaxPairs; ++q) {
+    for (int q = 0; q < kMaxGroups; ++q) {
       const int i = mb * kTileRows + il0 + 8 * q;
-      u_own[q] = (q < groups && vg < a.kg) ? a.u[(size_t)(a.n0 & 1) * rows + (int64_t)vg * a.n + i]
-                                               : mk<float>(0.f, 0.f);
+      u_own[q] = (owner && q < groups && vg < a.kg) ? a.u[(size_t)(a.n0 & 1) * rows + (int64_t)vg * a.n + i]
+                                                    : mk<float>(0.f, 0.f);
     }
-    // X slot layout: hi rows [0, 32) (re of 16 vectors, then im), lo rows [32, 64), in each K half.  The four
-    // lanes of a vector swap their four values, so that each stores one row's 16 bytes.
-    auto write_x = [&](float* xo_par, int i, cpx<float> u1) {
-      const float hr = tc::to_tf32(u1.re), hi = tc::to_tf32(u1.im);
-      const float val[4] = {hr, hi, u1.re - hr, u1.im - hi};
-      float got[4];   // from lane sub ^ r
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int w = sub ^ r;
-        const float lo2 = (w & 1) ? val[1] : val[0], hi2 = (w & 1) ? val[3] : val[2];
-        got[r] = __shfl_xor_sync(0xffffffffu, (w & 2) ? hi2 : lo2, 8 * r);
-      }
-      float out[4];   // out[t] = got[t ^ sub]
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const float lo2 = (sub & 1) ? got[t ^ 1] : got[t];
-        const float hi2 = (sub & 1) ? got[(t ^ 3) & 3] : got[(t ^ 2) & 3];
-        out[t] = (sub & 2) ? hi2 : lo2;
-      }
-      const int js = i / kTileK, kk = i % kTileK;
-      float* xo = xo_par + (size_t)js * kXcFloats + (kk >> 6) * kXhFloats;
-      __stcg(reinterpret_cast<float4*>(xo + tc::kmajor_offset(kChainVec * sub + vl, (kk & 63) & ~3, kTileK / 2) / 4),
-             make_float4(out[0], out[1], out[2], out[3]));
+    // State words of a slice: [K / 4][pair of the four][C] x (two K values); two neighbouring rows swap their
+    // halves, so that each stores one column's two values.
+    auto write_x = [&](int par, int i, cpx<float> u1, uint32_t number) {
+      const bool odd = lane & 1;
+      const float got = __shfl_xor_sync(0xffffffffu, odd ? u1.re : u1.im, 1);
+      const int kk = i % kTileK, c = 2 * vg + (odd ? 1 : 0);
+      float* x = a.X + ((size_t)par * a.cs + i / kTileK) * kXsFloats;
+      words_store(x + ((kk >> 1) * C + c) * 4, odd ? got : u1.re, odd ? u1.im : got, number);
     };
-    if (a.n0 == 0) {  // publish the initial state's split (later tiles find it from the previous tile)
+    if (a.n0 == 0 && owner) {  // publish the initial state (later tiles find it from the previous tile)
 #pragma unroll
-      for (int q = 0; q < kMaxPairs; ++q) {
-        if (q < groups) write_x(Xg, mb * kTileRows + il0 + 8 * q, u_own[q]);
-      }
-      chain_bar(chain);
-      if (ctid == 0) tc::red_release_add(&ready[mb], 1);
+      for (int q = 0; q < kMaxGroups; ++q)
+        if (q < groups) write_x(0, mb * kTileRows + il0 + 8 * q, u_own[q], 1u);
     }
-    // Every thread of the chain runs every step (named barriers need all 128);
-    // after an error the waits return at once and the flag reports the failure.
+    constexpr int kUnits = (kTileK / 2) * C / 4 / kWorkers;   // groups of four K values of a half per thread: 2 or 4
+    const int col = tid % C, kq0 = tid / C;
+    // Every warp runs every step; after an error the waits return at once and the flag reports the failure.
     for (int s = 0; s < a.steps; ++s) {
       const int64_t n = a.n0 + s;
       const int par = (int)(n & 1);
-      // forcing of this step for the owned pairs: loads in flight during the MMA phase
+      const uint32_t number = (uint32_t)(n + 1);
+      // forcing of this step for the owned pairs: loads in flight during the products
       const cpx<float>* Fs = (a.F != nullptr && n < a.n_forced) ? a.F + (size_t)s * rows : nullptr;
-      cpx<float> fv[kMaxPairs];
+      cpx<float> fv[kMaxGroups];
 #pragma unroll
-      for (int q = 0; q < kMaxPairs; ++q) {
+      for (int q = 0; q < kMaxGroups; ++q) {
         const int i = mb * kTileRows + il0 + 8 * q;
-        fv[q] = (Fs != nullptr && q < groups && vg < a.kg)
-                    ? mk<float>(__ldcs(reinterpret_cast<const float*>(Fs + (int64_t)vg * a.n + i)),
-                                __ldcs(reinterpret_cast<const float*>(Fs + (int64_t)vg * a.n + i) + 1))
-                    : mk<float>(0.f, 0.f);
-      }
-      // 1. the state slice of this step: a row block's columns are one K half, fetched by one of two warps
-      const int wc = warp & 3;
-      if (wc < 2) {
-        if (lane == 0) {
-          const int target = a.cs * (int)(n + 1) + ((a.stall && s == 0) ? (1 << 30) : 0);
-          if (!tc::spin_until_geq(&ready[2 * j + wc], target, errv, a.wait_ns)) {
-            atomicExch(a.err, 2);
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar_x + wc)) : "memory");
-          } else {
-            tc::fence_proxy_async_global();
-            tc::mbar_arrive_expect_tx(bar_x + wc, 4 * kXhFloats);
-            tc::bulk_g2s(X_sm + wc * kXhFloats, Xg + (size_t)par * xset + (size_t)j * kXcFloats + wc * kXhFloats,
-                         4 * kXhFloats, bar_x + wc);
-          }
+        fv[q] = mk<float>(0.f, 0.f);
+        if (Fs != nullptr && owner && q < groups && vg < a.kg) {
+          const float2 f = __ldcs(reinterpret_cast<const float2*>(Fs + (int64_t)vg * a.n + i));
+          fv[q] = mk<float>(f.x, f.y);
         }
-        __syncwarp();
       }
-      // 2. products, issued by a converged warp (descriptors in uniform registers)
-      if (wc == 0) {
-        const uint64_t ah = tc::smem_desc(A_hi, 128, (kTileK / 4) * 128), al = tc::smem_desc(A_lo, 128, (kTileK / 4) * 128);
-        const uint64_t xx = tc::smem_desc(X_sm, 128, (kTileK / 8) * 128);
-        bool okx = true;
+      // 1. the state slice of this step
+      {
+        const float* xs = a.X + ((size_t)par * a.cs + j) * kXsFloats;
+        const uint32_t want = number + ((a.stall && s == 0) ? (1u << 30) : 0u);
+        auto at = [&](int h, int i) {   // load i of half h: unit i / 2, K pair i % 2
+          return xs + (((kTileK / 8) * h + kq0 + (kWorkers / C) * (i >> 1)) * 2 + (i & 1)) * C * 4 + col * 4;
+        };
+        uint64_t w[2][2 * kUnits][2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int i = 0; i < 2 * kUnits; ++i) words_load(at(h, i), w[h][i]);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          okx = tc::mbar_wait(bar_x + h, (uint32_t)(s & 1), 0xFFFFFFFFu) && okx;
-          if (__all_sync(0xffffffffu, okx && *errv == 0)) {
-            tc::tc_fence_after();
-            if (lane == 0) {
+          if (!words_wait<2 * kUnits>(w[h], 2 * kUnits, want, [&](int i) { return at(h, i); }, errv, a.wait_ns)) {
+            atomicExch(a.err, 2);
+            *dead = 1;
+          }
 #pragma unroll
-              for (int ks = 0; ks < kTileK / 16; ++ks) {
-                const uint64_t x = xx + h * (kXhFloats / 4) + ks * 16;
-                tc::mma_tf32(tcol, ah + (8 * h + ks) * 16, x, idesc_hx, h + ks > 0);
-                tc::mma_tf32(tcol + 2 * kChainN, al + (8 * h + ks) * 16, x, idesc_lx, h + ks > 0);
-              }
+          for (int t = 0; t < kUnits; ++t) {
+            float v[4], hi[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              v[e] = word_value(w[h][2 * t + (e >> 1)][e & 1]);
+              hi[e] = tc::to_tf32(v[e]);
+            }
+            const int kk = 4 * (kq0 + (kWorkers / C) * t);
+            float* x = X_sm + h * kHalf;
+            *reinterpret_cast<float4*>(x + tc::kmajor_offset(col, kk, kTileK / 2) / 4) =
+                make_float4(hi[0], hi[1], hi[2], hi[3]);
+            *reinterpret_cast<float4*>(x + tc::kmajor_offset(C + col, kk, kTileK / 2) / 4) =
+                make_float4(v[0] - hi[0], v[1] - hi[1], v[2] - hi[2], v[3] - hi[3]);
+          }
+          tc::fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar_x + h)) : "memory");
+        }
+      }
+      ok = tc::mbar_wait(bar_m, (uint32_t)(s & 1), 0xFFFFFFFFu, nullptr, own_ns) && ok;
+      const bool live = ok && *dead == 0;   // else zeros go out and the state stays
+      __syncwarp();
+      tc::tc_fence_after();
+      // 3. partial: hi*hi + hi*lo + lo*hi, one row and half of the columns per thread
+      {
+        constexpr int W = C / 2;
+        const int row = 32 * (warp & 3) + lane, c0 = W * (warp >> 2);
+        const uint32_t tl = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0;
+        float x0[W], x1[W], x2[W];
+        if constexpr (W == 32) {
+          tc::tmem_ld32(tl, x0);
+          tc::tmem_ld32(tl + C, x1);
+          tc::tmem_ld32(tl + 2 * C, x2);
+        } else {
+          tc::tmem_ld16(tl, x0);
+          tc::tmem_ld16(tl + C, x1);
+          tc::tmem_ld16(tl + 2 * C, x2);
+        }
+        tc::tc_fence_before();
+        float* pb = a.part + (((size_t)par * MB + mb) * a.cs + j) * kPartFloats + ((size_t)(c0 / 2) * kM + row) * 4;
+#pragma unroll
+        for (int c = 0; c < W; c += 2)
+          words_store(pb + (size_t)(c / 2) * kM * 4, live ? x0[c] + x1[c] + x2[c] : 0.f,
+                      live ? x0[c + 1] + x1[c + 1] + x2[c + 1] : 0.f, number);
+      }
+      // 4. owner: its rows of all partials of the row block for this step
+      if (owner) {
+        cpx<float>* Ys = (a.Y != nullptr && s >= a.y_first) ? a.Y + (size_t)s * rows : nullptr;
+        const float* pbase = a.part + ((size_t)par * MB + mb) * a.cs * kPartFloats;
+#pragma unroll
+        for (int q = 0; q < kMaxGroups; ++q) {
+          if (q < groups) {
+            const int iloc = il0 + 8 * q;
+            // rows iloc: Re D times (Ur, Ui); rows 64 + iloc: Im D
+            auto at = [&](int i) {
+              return pbase + (size_t)(i >> 1) * kPartFloats + ((size_t)vg * kM + iloc + 64 * (i & 1)) * 4;
+            };
+            uint64_t w[16][2];
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              if (i < 2 * a.cs) words_load(at(i), w[i]);
+            bool got = live;
+            if (!words_wait<16>(w, 2 * a.cs, number, at, errv, a.wait_ns)) {
+              atomicExch(a.err, 2);
+              *dead = 1;
+              got = false;
             }
             __syncwarp();
+            float prr = 0.f, pri = 0.f, pir = 0.f, pii = 0.f;
+#pragma unroll
+            for (int p = 0; p < 8; ++p) {
+              if (p < a.cs) {
+                prr += word_value(w[2 * p][0]);
+                pri += word_value(w[2 * p][1]);
+                pir += word_value(w[2 * p + 1][0]);
+                pii += word_value(w[2 * p + 1][1]);
+              }
+            }
+            const int i = mb * kTileRows + iloc;
+            const cpx<float> u0 = u_own[q];
+            cpx<float> u1 = mk<float>(u0.re + (prr - pii) + fv[q].re, u0.im + (pri + pir) + fv[q].im);
+            if (vg >= a.kg) u1 = mk<float>(0.f, 0.f);
+            if (!got) u1 = u0;
+            write_x(1 - par, i, u1, number + 1);
+            if (Ys != nullptr && vg < a.kg)
+              __stcs(reinterpret_cast<float2*>(Ys + (int64_t)vg * a.n + i), make_float2(u0.re, u0.im));
+            u_own[q] = u1;
           }
         }
-        if (lane == 0) tc::mma_commit(bar_m);
-        __syncwarp();
       }
-      ok = tc::mbar_wait(bar_m, (uint32_t)(s & 1), 0xFFFFFFFFu) && ok && *errv == 0;
-      tc::tc_fence_after();
-      // 3. partial: hi*hi + hi*lo + lo*hi, one row per thread
-      float* pb = partg + (((size_t)par * MB + mb) * a.cs + j) * kPartFloats;
-      {
-        const int qw = warp & 3;
-        const int row = 32 * qw + lane;
-        const uint32_t tl = tcol + ((uint32_t)(32 * qw) << 16);
-        float x0[32], x1[32], x2[32];
-        tc::tmem_ld32(tl, x0);
-        tc::tmem_ld32(tl + kChainN, x1);
-        tc::tmem_ld32(tl + 2 * kChainN, x2);
-        float4* dst = reinterpret_cast<float4*>(pb) + row;   // four columns of all rows side by side
-#pragma unroll
-        for (int c = 0; c < kChainN / 4; ++c)
-          __stcg(dst + c * kM, make_float4(x0[4 * c] + x1[4 * c] + x2[4 * c], x0[4 * c + 1] + x1[4 * c + 1] + x2[4 * c + 1],
-                                           x0[4 * c + 2] + x1[4 * c + 2] + x2[4 * c + 2],
-                                           x0[4 * c + 3] + x1[4 * c + 3] + x2[4 * c + 3]));
-      }
-      tc::tc_fence_before();
-      chain_bar(chain);
-      if (ctid == 0) tc::red_release_add(&cnt[par * MB + mb], 1);
-      // 4. owner: its rows of all partials of the row block for this step
-      const float* pbase = partg + ((size_t)par * MB + mb) * a.cs * kPartFloats;
-      if (ctid == 0 && !tc::spin_until_geq(&cnt[par * MB + mb], a.cs * (int)((n >> 1) + 1), errv, a.wait_ns))
-        atomicExch(a.err, 2);
-      chain_bar(chain);
-      cpx<float>* Ys = (a.Y != nullptr && s >= a.y_first) ? a.Y + (size_t)s * rows : nullptr;
-      float* xo_par = Xg + (size_t)(1 - par) * xset;
-#pragma unroll
-      for (int q = 0; q < kMaxPairs; ++q) {
-        if (q < groups) {
-          const int iloc = il0 + 8 * q;
-          float prr = 0.f, pri = 0.f, pir = 0.f, pii = 0.f;
-          float t0[8], t1[8], t2[8], t3[8];
-          // columns [0, 16) times Ur, [16, 32) times Ui; rows iloc real, 64 + iloc imaginary part of D
-          const float* g = pbase + (size_t)((vl >> 2) * kM + iloc) * 4 + (vl & 3);
-#pragma unroll
-          for (int p = 0; p < 8; ++p) {
-            if (p < a.cs) {
-              t0[p] = __ldcg(g + (size_t)p * kPartFloats);
-              t1[p] = __ldcg(g + (size_t)p * kPartFloats + 4 * kM * 4);
-              t2[p] = __ldcg(g + (size_t)p * kPartFloats + 64 * 4);
-              t3[p] = __ldcg(g + (size_t)p * kPartFloats + 4 * kM * 4 + 64 * 4);
-            }
-          }
-#pragma unroll
-          for (int p = 0; p < 8; ++p) {
-            if (p < a.cs) {
-              prr += t0[p];
-              pri += t1[p];
-              pir += t2[p];
-              pii += t3[p];
-            }
-          }
-          const int i = mb * kTileRows + iloc;
-          const cpx<float> u0 = u_own[q];
-          cpx<float> u1 = mk<float>(u0.re + (prr - pii) + fv[q].re, u0.im + (pri + pir) + fv[q].im);
-          if (vg >= a.kg) u1 = mk<float>(0.f, 0.f);
-          if (Ys != nullptr && vg < a.kg) __stcs(reinterpret_cast<float2*>(Ys + (int64_t)vg * a.n + i), make_float2(u0.re, u0.im));
-          write_x(xo_par, i, u1);
-          u_own[q] = u1;
-        }
-      }
-      chain_bar(chain);
-      if (ctid == 0) tc::red_release_add(&ready[mb], 1);
     }
     // state at the end of the tile
     const int64_t nend = a.n0 + a.steps;
 #pragma unroll
-    for (int q = 0; q < kMaxPairs; ++q) {
+    for (int q = 0; q < kMaxGroups; ++q) {
       const int i = mb * kTileRows + il0 + 8 * q;
-      if (q < groups && vg < a.kg) a.u[(size_t)(nend & 1) * rows + (int64_t)vg * a.n + i] = u_own[q];
+      if (owner && q < groups && vg < a.kg) a.u[(size_t)(nend & 1) * rows + (int64_t)vg * a.n + i] = u_own[q];
     }
   }
+  if (!ok && lane == 0) atomicExch(a.err, 2);
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
   if (warp == 0) tc::tmem_dealloc(tmem, 256);
-  if (!ok && (tid & 127) == 0) atomicExch(a.err, 2);
 }
+
+void (*march_kernel(int n, int kg))(TcMarchArgs) {
+  if (n / kTileK == 8) return kg <= 16 ? dense_tc_march_kernel<32, 1> : dense_tc_march_kernel<64, 1>;
+  return kg <= 16 ? dense_tc_march_kernel<32, 8> : dense_tc_march_kernel<64, 8>;
+}
+
+// Partial words of all CTAs, two step parities.
+size_t part_bytes(int n) { return (size_t)2 * (n / kTileRows) * (n / kTileK) * kPartFloats * sizeof(float); }
 
 // A tiles from the FP64 matrix (conj-transposed for the adjoint): tile (mb, j) rows
 // r < 64: Re M[64 mb + r][128 j + k], r >= 64: Im M[64 mb + r - 64][128 j + k]; hi/lo TF32 split.
@@ -536,23 +576,20 @@ rsv_status dense_tc_prepare(rsv_operator op, const void* d64_direct) {
   }
   cudaError_t e = cudaFuncSetAttribute(dense_tc_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)kSmemBytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(dense_tc_march_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kSmemPersistent);
+  for (auto* k : {march_kernel(n, 16), march_kernel(n, 32)})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemPersistent);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "tensor-core tiles");
   // The persistent tile kernel needs all of its CTAs resident at once (one per SM).
   op->tc_persistent = false;
   const int MB = n / kTileRows;
-  if (!op->d_ready) {
-    e = cudaMalloc(&op->d_ready, sizeof(int) * kMaxChains * 3 * MB);
-    if (e == cudaSuccess) op->dev.push_back(op->d_ready);
-    if (e == cudaSuccess) e = cudaMalloc(&op->tc_acc, sizeof(float) * kMaxChains * 2 * MB * cs * kPartFloats);
+  if (!op->tc_acc) {
+    e = cudaMalloc(&op->tc_acc, part_bytes(n));
     if (e == cudaSuccess) op->dev.push_back(op->tc_acc);
     if (e != cudaSuccess) return cuda_fail(e, "tensor-core march buffers");
   }
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, dense_tc_march_kernel, kMarchThreads, kSmemPersistent);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, march_kernel(n, 32), kMarchThreads, kSmemPersistent);
   if (e != cudaSuccess) {
     cudaGetLastError();
     per_sm = 0;
@@ -563,10 +600,8 @@ rsv_status dense_tc_prepare(rsv_operator op, const void* d64_direct) {
   return RSV_OK;
 }
 
-// Operand buffers of the persistent kernel (per chain, two step parities).
-size_t dense_tc_chain_x_bytes(rsv_operator op) {
-  return (size_t)kMaxChains * 2 * (op->n / kTileK) * kXcFloats * sizeof(float);
-}
+// State words of the persistent kernel (two step parities).
+size_t dense_tc_chain_x_bytes(rsv_operator op) { return (size_t)2 * (op->n / kTileK) * kXsFloats * sizeof(float); }
 
 // A whole tile of steps in one persistent launch (requires op->tc_persistent).
 cudaError_t dense_tc_march_tile(rsv_operator op, int kg, bool adjoint, int64_t n0, int steps, int64_t n_forced,
@@ -578,8 +613,6 @@ cudaError_t dense_tc_march_tile(rsv_operator op, int kg, bool adjoint, int64_t n
   a.A = (const float*)op->tc_tiles[adjoint ? 1 : 0];
   a.X = (float*)xbuf;
   a.part = (float*)op->tc_acc;
-  a.cnt = (int*)op->d_ready;                       // [chains][2][MB]
-  a.ready = (int*)op->d_ready + kMaxChains * 2 * MB;  // [chains][MB]
   a.u = (cpx<float>*)state;
   a.F = (const cpx<float>*)F;
   a.Y = (cpx<float>*)Y;
@@ -590,16 +623,16 @@ cudaError_t dense_tc_march_tile(rsv_operator op, int kg, bool adjoint, int64_t n
   a.n = n;
   a.kg = kg;
   a.cs = cs;
-  a.chains = (kg + kChainVec - 1) / kChainVec;
   a.err = op->d_flag;
   a.wait_ns = op->wait_limit_ns;
   a.stall = op->test_stall_wait ? 1 : 0;
   cudaError_t e = cudaSuccess;
   if (n0 == 0) {
-    e = cudaMemsetAsync(op->d_ready, 0, sizeof(int) * kMaxChains * 3 * MB, op->stream);
+    e = cudaMemsetAsync(xbuf, 0, dense_tc_chain_x_bytes(op), op->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(op->tc_acc, 0, part_bytes(n), op->stream);
   }
   if (e != cudaSuccess) return e;
-  dense_tc_march_kernel<<<MB * cs, kMarchThreads, kSmemPersistent, op->stream>>>(a);
+  march_kernel(n, kg)<<<MB * cs, kMarchThreads, kSmemPersistent, op->stream>>>(a);
   return cudaGetLastError();
 }
 

@@ -185,8 +185,7 @@ struct rsv_operator_s {
   uint64_t wait_limit_ns = 2000000000ull;  // limit of each cross-CTA wait (RSV_WAIT_LIMIT_NS)
   bool test_stall_wait = false;  // test hook (RSV_TEST_STALL_WAIT=1): a wait on a count nobody reaches
   int tc_max_clusters = 0;      // resident CTAs of the persistent tile kernel on this GPU
-  void* d_ready = nullptr;      // per-block step counters and arrival counters of the persistent tile kernel
-  void* tc_acc = nullptr;       // its FP32 partial-sum accumulators
+  void* tc_acc = nullptr;       // its partial sums
   // stencil kinds: base-flow fields
   void* fld[8] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   void* fldp[4] = {nullptr, nullptr, nullptr, nullptr};   // ADV3D, FP32: rows padded to 4 cells

@@ -242,40 +242,6 @@ __device__ __forceinline__ float ld_peer_f32(uint32_t addr) {
   return v;
 }
 
-// Cross-CTA step counters (global memory, GPU scope).
-__device__ __forceinline__ int ld_acquire(const int* p) {
-  int v;
-  asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_release(int* p, int v) {
-  asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-// Release-ordered atomic add without a return value (fire and forget).
-__device__ __forceinline__ void red_release_add(int* p, int v) {
-  asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-// Spin (one thread) until *p >= target, bounded by limit_ns; also stops once *err != 0.
-__device__ __forceinline__ bool spin_until_geq(const int* p, int target, const volatile int* err,
-                                               uint64_t limit_ns = kWaitLimitNs) {
-  uint64_t t0 = 0;
-  for (uint32_t i = 0;; ++i) {
-    if (ld_acquire(p) >= target) return true;
-    if ((i & 15) == 15) {
-      if (*err != 0) return false;
-      const uint64_t now = global_ns();
-      if (t0 == 0) t0 = now;
-      else if (now - t0 > limit_ns) return false;
-    }
-  }
-}
-
-// Generic-proxy global writes become visible to the async proxy (bulk copies), and back.
-__device__ __forceinline__ void fence_proxy_async_global() {
-  asm volatile("fence.proxy.async.global;" ::: "memory");
-}
-
 // FP32 -> TF32 (round to nearest, ties away), result in an FP32 register with the low bits clear.
 __device__ __forceinline__ float to_tf32(float x) {
   uint32_t r;
