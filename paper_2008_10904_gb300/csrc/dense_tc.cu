@@ -3,7 +3,7 @@
 //   u_{n+1} = u_n + D u_n + F_n      (D = RK4 step polynomial minus identity, see dense_kernels.cu)
 //
 // D u is computed as the real GEMM  [Dr; Di] (2n x n)  x  [Ur | Ui] (n x 2kg):
-// rows 0..63 of a CTA's A tile are 64 rows of Re D, rows 64..127 the same rows
+// rows 2 r of a CTA's A tile are 64 rows of Re D, rows 2 r + 1 the same rows
 // of Im D, and  Re(Du) = DrUr - DiUi,  Im(Du) = DrUi + DiUr.  Operands are
 // split into TF32 pairs (x = hi + lo, hi = tf32(x)) and three MMAs
 // (hi*hi + hi*lo + lo*hi) give FP32-level products with FP32 accumulation in
@@ -15,8 +15,7 @@
 // slice (hi, lo: 2 x 32 KB) into shared memory, issues 16 K-steps x 3 MMAs
 // (M = 128, N = 64, K = 8) from one thread, reads the 128 x 64 partial from
 // tensor memory and exchanges it through distributed shared memory: CTA j
-// sums over the cluster the partials of its 64/CS complex rows (stacked rows
-// r and 64 + r) and
+// sums over the cluster the partials of its 64/CS complex rows and
 // writes the new state, the snapshot, and the TF32 split of the new state
 // in the operand layout of the next step.  All waits are bounded; a timeout
 // sets the error flag.
@@ -121,7 +120,7 @@ __global__ void __launch_bounds__(256, 1) dense_tc_step_kernel(TcStepArgs a) {
   tc::cluster_sync();
 
   // cluster reduction + RK4 update: CTA j owns complex rows [rpc j, rpc j + rpc) of the
-  // cluster's 64-row block (rpc = 64 / cs), i.e. stacked rows iloc and 64 + iloc
+  // cluster's 64-row block (rpc = 64 / cs), i.e. stacked rows 2 iloc and 2 iloc + 1
   {
     const int rpc = kTileRows / a.cs;
     for (int pidx = tid; pidx < rpc * 32; pidx += blockDim.x) {
@@ -134,10 +133,10 @@ __global__ void __launch_bounds__(256, 1) dense_tc_step_kernel(TcStepArgs a) {
 #pragma unroll
         for (int p = 0; p < 8; ++p) {
           if (p < a.cs) {
-            rr[p] = tc::ld_peer_f32(tc::map_peer(&red[iloc * kRedLd + v], p));
-            ri[p] = tc::ld_peer_f32(tc::map_peer(&red[iloc * kRedLd + 32 + v], p));
-            ir[p] = tc::ld_peer_f32(tc::map_peer(&red[(64 + iloc) * kRedLd + v], p));
-            ix[p] = tc::ld_peer_f32(tc::map_peer(&red[(64 + iloc) * kRedLd + 32 + v], p));
+            rr[p] = tc::ld_peer_f32(tc::map_peer(&red[2 * iloc * kRedLd + v], p));
+            ri[p] = tc::ld_peer_f32(tc::map_peer(&red[2 * iloc * kRedLd + 32 + v], p));
+            ir[p] = tc::ld_peer_f32(tc::map_peer(&red[(2 * iloc + 1) * kRedLd + v], p));
+            ix[p] = tc::ld_peer_f32(tc::map_peer(&red[(2 * iloc + 1) * kRedLd + 32 + v], p));
           }
         }
 #pragma unroll
@@ -191,8 +190,8 @@ __global__ void __launch_bounds__(256, 1) dense_tc_step_kernel(TcStepArgs a) {
 //   2. warp 8 issues two MMAs per K-step, A_hi x [X_hi | X_lo] (N = 2 C) and
 //      A_lo x X_hi (N = C), the first half's while the second is converted: the A
 //      tile is read from shared memory twice, for all vectors at once;
-//   3. the workers sum the three product groups out of tensor memory and store the
-//      CTA's 128 x C partial;
+//   3. the workers sum the three product groups out of tensor memory, combine them to
+//      Re (D u) and Im (D u) and store the CTA's 64 x C partial;
 //   4. as owner of 64/CS rows of its row block, each thread loads its rows of the
 //      CS partials, all in flight at once, sums them in order, applies the RK4
 //      update u <- u + D u + F (u stays in registers for the whole tile), writes
@@ -203,15 +202,16 @@ __global__ void __launch_bounds__(256, 1) dense_tc_step_kernel(TcStepArgs a) {
 // The numbers start at 1; the buffers are zeroed at the start of a march.  Loads
 // that wait are bounded in time and stop once any CTA has set the error flag.
 // A step is a chain of latencies: n = 1024, 32 vectors, 13188 steps march in
-// 66 ms.  With counters (fence, add, poll and bulk copy per hand-off) and two
+// 57 ms.  With counters (fence, add, poll and bulk copy per hand-off) and two
 // chains of 16 vectors that took turns on the tensor cores 88 ms; of 6.7 us per
-// step 1.4 us were fences, 1.8 us polls and 2 us products.
+// step 1.4 us were fences, 1.8 us polls and 2 us products.  Partials of separate Re D and
+// Im D rows, twice as many words: 66 ms.
 // ---------------------------------------------------------------------------
 constexpr int kMaxCols = 64;                               // real columns: (re, im) of 32 vectors
 constexpr int kWorkers = 256;
 constexpr int kMarchThreads = kWorkers + 32;               // and the warp that issues the products
 constexpr uint32_t kXsFloats = kTileK * kMaxCols * 2;      // a slice's words: [K / 2][C] x 2 (value, number)
-constexpr uint32_t kPartFloats = kM * kMaxCols * 2;        // a partial's words: [C / 2][128 rows] x 2
+constexpr uint32_t kPartFloats = kM * kMaxCols;            // a partial's words: [C / 4][64 rows x 2 vectors] x (re, im)
 constexpr uint32_t kSmemPersistent = 4 * (2 * kATileFloats + 2 * kMaxCols * kTileK) + 256;
 
 struct TcMarchArgs {
@@ -439,11 +439,20 @@ __global__ void __launch_bounds__(kMarchThreads, 1) dense_tc_march_kernel(TcMarc
           tc::tmem_ld16(tl + 2 * C, x2);
         }
         tc::tc_fence_before();
-        float* pb = a.part + (((size_t)par * MB + mb) * a.cs + j) * kPartFloats + ((size_t)(c0 / 2) * kM + row) * 4;
+        // Neighbouring lanes hold a row of Re D and of Im D: they swap the products of one vector each, and the
+        // sums of half as many values go out
+        const bool odd = lane & 1;
+        float* pb = a.part + (((size_t)par * MB + mb) * a.cs + j) * kPartFloats + ((size_t)(c0 / 4) * kM + row) * 4;
 #pragma unroll
-        for (int c = 0; c < W; c += 2)
-          words_store(pb + (size_t)(c / 2) * kM * 4, live ? x0[c] + x1[c] + x2[c] : 0.f,
-                      live ? x0[c + 1] + x1[c + 1] + x2[c + 1] : 0.f, number);
+        for (int c = 0; c < W; c += 4) {
+          float y[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) y[e] = x0[c + e] + x1[c + e] + x2[c + e];
+          const float g0 = __shfl_xor_sync(0xffffffffu, odd ? y[0] : y[2], 1);
+          const float g1 = __shfl_xor_sync(0xffffffffu, odd ? y[1] : y[3], 1);
+          const float re = odd ? g0 - y[3] : y[0] - g1, im = odd ? g1 + y[2] : y[1] + g0;
+          words_store(pb + (size_t)(c / 4) * kM * 4, live ? re : 0.f, live ? im : 0.f, number);
+        }
       }
       // 4. owner: its rows of all partials of the row block for this step
       if (owner) {
@@ -453,34 +462,31 @@ __global__ void __launch_bounds__(kMarchThreads, 1) dense_tc_march_kernel(TcMarc
         for (int q = 0; q < kMaxGroups; ++q) {
           if (q < groups) {
             const int iloc = il0 + 8 * q;
-            // rows iloc: Re D times (Ur, Ui); rows 64 + iloc: Im D
-            auto at = [&](int i) {
-              return pbase + (size_t)(i >> 1) * kPartFloats + ((size_t)vg * kM + iloc + 64 * (i & 1)) * 4;
+            auto at = [&](int p) {
+              return pbase + (size_t)p * kPartFloats + ((size_t)(vg >> 1) * kM + 2 * iloc + (vg & 1)) * 4;
             };
-            uint64_t w[16][2];
+            uint64_t w[8][2];
 #pragma unroll
-            for (int i = 0; i < 16; ++i)
-              if (i < 2 * a.cs) words_load(at(i), w[i]);
+            for (int p = 0; p < 8; ++p)
+              if (p < a.cs) words_load(at(p), w[p]);
             bool got = live;
-            if (!words_wait<16>(w, 2 * a.cs, number, at, errv, a.wait_ns)) {
+            if (!words_wait<8>(w, a.cs, number, at, errv, a.wait_ns)) {
               atomicExch(a.err, 2);
               *dead = 1;
               got = false;
             }
             __syncwarp();
-            float prr = 0.f, pri = 0.f, pir = 0.f, pii = 0.f;
+            float pr = 0.f, pi = 0.f;
 #pragma unroll
             for (int p = 0; p < 8; ++p) {
               if (p < a.cs) {
-                prr += word_value(w[2 * p][0]);
-                pri += word_value(w[2 * p][1]);
-                pir += word_value(w[2 * p + 1][0]);
-                pii += word_value(w[2 * p + 1][1]);
+                pr += word_value(w[p][0]);
+                pi += word_value(w[p][1]);
               }
             }
             const int i = mb * kTileRows + iloc;
             const cpx<float> u0 = u_own[q];
-            cpx<float> u1 = mk<float>(u0.re + (prr - pii) + fv[q].re, u0.im + (pri + pir) + fv[q].im);
+            cpx<float> u1 = mk<float>(u0.re + pr + fv[q].re, u0.im + pi + fv[q].im);
             if (vg >= a.kg) u1 = mk<float>(0.f, 0.f);
             if (!got) u1 = u0;
             write_x(1 - par, i, u1, number + 1);
@@ -515,7 +521,7 @@ void (*march_kernel(int n, int kg))(TcMarchArgs) {
 size_t part_bytes(int n) { return (size_t)2 * (n / kTileRows) * (n / kTileK) * kPartFloats * sizeof(float); }
 
 // A tiles from the FP64 matrix (conj-transposed for the adjoint): tile (mb, j) rows
-// r < 64: Re M[64 mb + r][128 j + k], r >= 64: Im M[64 mb + r - 64][128 j + k]; hi/lo TF32 split.
+// r even: Re M[64 mb + r / 2][128 j + k], r odd: Im; hi/lo TF32 split.
 __global__ void arrange_a_kernel(int n, int cs, const cpx<double>* __restrict__ M, bool conj_t, float* __restrict__ out) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // over (mb, j, r, k)
   const int64_t total = (int64_t)(n / kTileRows) * cs * kM * kTileK;
@@ -524,9 +530,9 @@ __global__ void arrange_a_kernel(int n, int cs, const cpx<double>* __restrict__ 
   const int r = (int)((e / kTileK) % kM);
   const int j = (int)((e / ((int64_t)kTileK * kM)) % cs);
   const int mb = (int)(e / ((int64_t)kTileK * kM * cs));
-  const int row = mb * kTileRows + (r & 63), col = j * kTileK + k;
+  const int row = mb * kTileRows + (r >> 1), col = j * kTileK + k;
   const cpx<double> m = conj_t ? conjg(M[(int64_t)col * n + row]) : M[(int64_t)row * n + col];
-  const double x = (r < 64) ? m.re : m.im;
+  const double x = (r & 1) == 0 ? m.re : m.im;
   const float hi = tc::to_tf32((float)x);
   const float lo = (float)(x - (double)hi);
   float* tile = out + ((size_t)mb * cs + j) * 2 * kATileFloats;
