@@ -927,7 +927,7 @@ __global__ void __launch_bounds__(NT, MINB) adv3d_pair_kernel(StGeom g, Pair3D P
 
 // ---------------------------------------------------------------------------
 // 2-D system, FP32: RK4 in two launches per step, each fusing a pair of stages (the scheme of the
-// 3-D pair kernels above, on one plane).  A CTA owns a 64 x 32 tile of one vector: the pair's
+// 3-D pair kernels above, on one plane).  A CTA owns a 64 x 32 or 64 x 8 tile of one vector: the pair's
 // stencil input (u or x3) is copied with a halo of two cells into shared memory (16-byte
 // asynchronous copies of rows from x = X0 - 4), the first stage is evaluated on the tile and a
 // one-cell halo into a second shared array, the second stage on the tile.  Per step the
@@ -935,9 +935,9 @@ __global__ void __launch_bounds__(NT, MINB) adv3d_pair_kernel(StGeom g, Pair3D P
 // written, plus the snapshot on analysed steps; pair B: x3, u, acc and two forcing samples read,
 // u' written) against about 20 for the four single-stage kernels.  Cells outside the grid hold zero.
 // ---------------------------------------------------------------------------
-constexpr int k2TX = 64, k2TY = 32, k2Threads = 256;
-constexpr int k2UW = k2TX + 8, k2UH = k2TY + 4;     // input tile: x from X0 - 4, y halo 2
-constexpr int k2XW = k2TX + 2, k2XH = k2TY + 2;     // first-stage tile: halo 1
+constexpr int k2TX = 64, k2Threads = 256;           // tiles of 32 or 8 rows
+constexpr int k2UW = k2TX + 8;                      // input tile: x from X0 - 4, y halo 2
+constexpr int k2XW = k2TX + 2;                      // first-stage tile: halo 1
 
 // Sponge rate at cell (gi, gj) with precomputed 1 / sponge_cells (the same values as sponge()).
 __device__ __forceinline__ float sponge_fast(int gi, int gj, const StGeom& g, float inv_s) {
@@ -947,13 +947,13 @@ __device__ __forceinline__ float sponge_fast(int gi, int gj, const StGeom& g, fl
   return (float)g.sponge_amp * t * t;
 }
 
-// Shared-memory tiles of the 2-D pair kernel (floats): the stencil input (rows Y0-2 .. Y0+33, x from
-// X0-4, 72 wide), the first stage's forcing and (pair B) state on its halo region (rows Y0-1 ..
-// Y0+32, 72 wide), the first-stage result (66 x 34), and the second stage's forcing and (pair B)
-// accumulator on the tile (64 x 32).  Every global read of the kernel is one of these 16-byte
+// Shared-memory tiles of the 2-D pair kernel (floats): the stencil input (TY + 4 rows from Y0-2, x from
+// X0-4, 72 wide), the first stage's forcing and (pair B) state on its halo region (TY + 2
+// rows, 72 wide), the first-stage result (66 wide), and the second stage's forcing and (pair B)
+// accumulator on the tile.  Every global read of the kernel is one of these 16-byte
 // asynchronous copies, issued together at the start.
-constexpr int k2HW = k2UW, k2HH = k2XH;            // halo-region tiles: 72 x 34
-constexpr int k2Smem = (k2UH * k2UW + 2 * k2HH * k2HW + k2XH * k2XW + 2 * k2TX * k2TY) * 4;
+constexpr int k2HW = k2UW;                         // halo-region tiles
+constexpr int k2_smem(int ty) { return ((ty + 4) * k2UW + 2 * (ty + 2) * k2HW + (ty + 2) * k2XW + 2 * k2TX * ty) * 4; }
 
 // Copies rows [y0, y0 + nrow) x [x0, x0 + 4 nch) of a field into a tile with rows of width w (16-byte
 // chunks, wholly inside the grid or zero).
@@ -971,8 +971,9 @@ __device__ __forceinline__ void tile_copy(float* t, int w, const float* src, int
 }
 
 // Requires nx % 4 == 0 (16-byte rows of the tiles and of the second stage's float4 stores).
-template <bool PAIR_B>
+template <bool PAIR_B, int k2TY>
 __global__ void __launch_bounds__(k2Threads) adr2d_pair_kernel(StGeom g, Pair3D P) {
+  constexpr int k2UH = k2TY + 4, k2XH = k2TY + 2, k2HH = k2XH;
   extern __shared__ __align__(16) unsigned char smem2[];
   float* tin = reinterpret_cast<float*>(smem2);        // [k2UH][k2UW]
   float* ta = tin + k2UH * k2UW;                        // [k2HH][k2HW] forcing of the first stage
@@ -1002,12 +1003,6 @@ __global__ void __launch_bounds__(k2Threads) adr2d_pair_kernel(StGeom g, Pair3D 
   const float c1 = PAIR_B ? h : 0.5f * h;
   const float c2 = PAIR_B ? h / 6.f : 0.5f * h;
   const int tid = threadIdx.x;
-  tile_copy(tin, k2UW, P.in + base, X0 - 4, k2UW / 4, Y0 - 2, k2UH, nx, ny, tid);
-  tile_copy(ta, k2HW, P.fa ? P.fa + base : nullptr, X0 - 4, k2HW / 4, Y0 - 1, k2HH, nx, ny, tid);
-  if (PAIR_B) tile_copy(tu, k2HW, P.u + base, X0 - 4, k2HW / 4, Y0 - 1, k2HH, nx, ny, tid);
-  tile_copy(tb, k2TX, P.fb ? P.fb + base : nullptr, X0, k2TX / 4, Y0, k2TY, nx, ny, tid);
-  if (PAIR_B) tile_copy(tc, k2TX, P.acc + base, X0, k2TX / 4, Y0, k2TY, nx, ny, tid);
-  asm volatile("cp.async.commit_group;" ::: "memory");
   if (tid < k2XH) {   // row coefficients of rows Y0 - 1 .. Y0 + k2TY
     const int gj = min(max(Y0 - 1 + tid, 0), ny - 1);
     const float* U = reinterpret_cast<const float*>(g.f0);
@@ -1017,6 +1012,15 @@ __global__ void __launch_bounds__(k2Threads) adr2d_pair_kernel(StGeom g, Pair3D 
     rowc[tid][1] = -ux * i2dx + nu * idx2;
     rowc[tid][2] = -2.f * nu * (idx2 + idy2) + __ldg(rr + gj);
   }
+  // Launched as a programmatic dependent of the previous pair kernel: nothing above touches what that one writes.
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  tile_copy(tin, k2UW, P.in + base, X0 - 4, k2UW / 4, Y0 - 2, k2UH, nx, ny, tid);
+  tile_copy(ta, k2HW, P.fa ? P.fa + base : nullptr, X0 - 4, k2HW / 4, Y0 - 1, k2HH, nx, ny, tid);
+  if (PAIR_B) tile_copy(tu, k2HW, P.u + base, X0 - 4, k2HW / 4, Y0 - 1, k2HH, nx, ny, tid);
+  tile_copy(tb, k2TX, P.fb ? P.fb + base : nullptr, X0, k2TX / 4, Y0, k2TY, nx, ny, tid);
+  if (PAIR_B) tile_copy(tc, k2TX, P.acc + base, X0, k2TX / 4, Y0, k2TY, nx, ny, tid);
+  asm volatile("cp.async.commit_group;" ::: "memory");
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
   // first stage on the tile and a one-cell halo: x_mid = u + c1 (A x + f_a); zero outside the grid
@@ -1081,14 +1085,34 @@ __global__ void __launch_bounds__(k2Threads) adr2d_pair_kernel(StGeom g, Pair3D 
   }
 }
 
+template <bool PAIR_B, int TY>
+cudaError_t launch_pair2d_ty(rsv_operator op, const StGeom& g, const Pair3D& P, unsigned blocks) {
+  constexpr int smem = k2_smem(TY);
+  // per-device attribute: set before every launch (cheap next to a pass over the field)
+  cudaError_t e = cudaFuncSetAttribute(adr2d_pair_kernel<PAIR_B, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(k2Threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = op->stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, adr2d_pair_kernel<PAIR_B, TY>, g, P);
+}
+
+// Tiles of 32 rows where they come to two CTAs per SM; a smaller field is bound by the latency of a CTA's chain
+// of copies and stages and takes tiles of 8 (256 x 128, 4 vectors, 765 steps: 7.3 ms by 64 CTAs of 32 rows in
+// ordinary launches, 4.0 ms like this as programmatic dependents).
 template <bool PAIR_B>
 cudaError_t launch_pair2d(rsv_operator op, const StGeom& g, const Pair3D& P) {
-  // per-device attribute: set before every launch (cheap next to a pass over the field)
-  cudaError_t e = cudaFuncSetAttribute(adr2d_pair_kernel<PAIR_B>, cudaFuncAttributeMaxDynamicSharedMemorySize, k2Smem);
-  if (e != cudaSuccess) return e;
-  const unsigned ntx = (unsigned)((g.nx + k2TX - 1) / k2TX), nty = (unsigned)((g.ny + k2TY - 1) / k2TY);
-  adr2d_pair_kernel<PAIR_B><<<ntx * nty * (unsigned)g.kg, k2Threads, k2Smem, op->stream>>>(g, P);
-  return cudaGetLastError();
+  const unsigned cols = (unsigned)((g.nx + k2TX - 1) / k2TX) * (unsigned)g.kg;
+  const unsigned b32 = cols * (unsigned)((g.ny + 31) / 32);
+  if (b32 >= 2u * (unsigned)std::max(1, op->sm_count)) return launch_pair2d_ty<PAIR_B, 32>(op, g, P, b32);
+  return launch_pair2d_ty<PAIR_B, 8>(op, g, P, cols * (unsigned)((g.ny + 7) / 8));
 }
 
 // Resident CTAs per SM the pair kernels are compiled for: 2 (no spills, the default) or 3 (80
