@@ -16,18 +16,15 @@ namespace {
 
 constexpr int kMaxK = 32;
 
-// One CTA per (frequency, instance, chunk of points).  The CTA stages the k vectors of 256 points at a
-// time in shared memory (each value read once from HBM, the next slab in flight during the current one).  The k x k Gram is Hermitian and cut into
-// tiles of T x T pairs on and above the diagonal, one or a few per warp: a lane holds the T x T sums of
-// its points (every 32nd), so that 2 T loads feed T^2 complex multiply-adds.  The lanes' sums over a slab
-// (8 points each) are added up across the warp by a halving exchange that leaves one of the 2 T^2 values
-// per lane, which goes on in FP64 across the slabs.  One FP64 atomic per value and chunk.  k = 16, 4.2 M points, FP32: 0.22 ms (one pair per thread: 0.70).
+// FP64: one CTA per (frequency, instance, chunk of points).  The CTA stages the k vectors of 256 points at a
+// time in shared memory (each value read once from HBM, the next slab in flight during the current one).  The
+// k x k Gram is Hermitian and cut into tiles of T x T pairs on and above the diagonal, one or a few per warp: a
+// lane holds the T x T sums of its points (every 32nd), so that 2 T loads feed T^2 complex multiply-adds.  The
+// lanes' sums over a slab are added up across the warp by a halving exchange that leaves one of the 2 T^2
+// values per lane.  One FP64 atomic per value and chunk.
 constexpr int kSlab = 256;
 constexpr int kSlabsPerCta = 8;
 constexpr int kGramWarps = 12;
-
-template <typename R>
-constexpr int gram_tile() { return sizeof(R) == 4 ? 4 : 2; }
 
 // v[0 .. N-1] of every lane summed over the warp; lane l returns the sum of value l mod N.
 template <int N, typename R>
@@ -47,12 +44,19 @@ __device__ __forceinline__ R warp_scatter_sum(R* v, int lane) {
   return r;
 }
 
-template <typename R>
-__global__ void __launch_bounds__(32 * kGramWarps) gram_kernel(const cpx<R>* __restrict__ X, int k, int64_t n,
-                                                              const int64_t* __restrict__ inst_off, int n_inst,
-                                                              cpx<double>* __restrict__ G) {
-  constexpr int T = gram_tile<R>(), NV = 2 * T * T;
-  constexpr int kMaxOwn = sizeof(R) == 4 ? 3 : 12;                 // tiles per warp at k = 32
+__device__ __forceinline__ void gram_tile_of(int t, int kt, int T, int* ta, int* tb) {   // rows ta, columns tb >= ta
+  int a = 0;
+  while (t >= kt - a) t -= kt - a++;
+  *ta = a * T;
+  *tb = (a + t) * T;
+}
+
+__global__ void __launch_bounds__(32 * kGramWarps) gram64_kernel(const cpx<double>* __restrict__ X, int k, int64_t n,
+                                                                const int64_t* __restrict__ inst_off, int n_inst,
+                                                                cpx<double>* __restrict__ G) {
+  using R = double;
+  constexpr int T = 2, NV = 2 * T * T;
+  constexpr int kMaxOwn = 12;                                       // tiles per warp at k = 32
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cpx<R>* slabs = reinterpret_cast<cpx<R>*>(smem_raw);             // [2][kt T][kSlab], rows from k on zero
   const int inst = blockIdx.y;
@@ -83,13 +87,7 @@ __global__ void __launch_bounds__(32 * kGramWarps) gram_kernel(const cpx<R>* __r
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   copy_slab(0);
-  // this warp's tiles warp, warp + nw, ...: rows ta, columns tb >= ta
-  auto tile_of = [&](int t, int* ta, int* tb) {
-    int a = 0;
-    while (t >= kt - a) t -= kt - a++;
-    *ta = a * T;
-    *tb = (a + t) * T;
-  };
+  // this warp's tiles warp, warp + nw, ...
   double tot[kMaxOwn];
 #pragma unroll
   for (int q = 0; q < kMaxOwn; ++q) tot[q] = 0.0;
@@ -106,7 +104,7 @@ __global__ void __launch_bounds__(32 * kGramWarps) gram_kernel(const cpx<R>* __r
       const int t = warp + q * nw;
       if (t >= tiles) break;
       int ta, tb;
-      tile_of(t, &ta, &tb);
+      gram_tile_of(t, kt, T, &ta, &tb);
       R v[NV];
 #pragma unroll
       for (int i = 0; i < NV; ++i) v[i] = R(0);
@@ -139,13 +137,113 @@ __global__ void __launch_bounds__(32 * kGramWarps) gram_kernel(const cpx<R>* __r
     const int t = warp + q * nw;
     if (t >= tiles) break;
     int ta, tb;
-    tile_of(t, &ta, &tb);
+    gram_tile_of(t, kt, T, &ta, &tb);
     const double s = tot[q];
     if (lane >= NV) continue;
     const int pair = lane >> 1, a = ta + pair / T, b = tb + pair % T;
     if (a >= k || b >= k) continue;
     atomicAdd(g + 2 * (a * k + b) + (lane & 1), s);
     if (ta != tb) atomicAdd(g + 2 * (b * k + a) + (lane & 1), (lane & 1) ? -s : s);   // the mirrored tile
+  }
+}
+
+// FP32: sums over a slab of 256 points in FP32, point after point, then FP64 across slabs.  That order is part of
+// the result (another one moves the triangular factors by 3e-8), and it is a chain of 512 multiply-adds, so the
+// parallelism is across slabs and pairs: a lane takes a slab of its own and a 4 x 4 tile of pairs, 8 loads per
+// point for 64 multiply-adds in 32 independent chains.  A CTA holds 32 slabs, eight points of each at a time in
+// shared memory (rows of 9, so that the lanes' loads fall in different banks; the next eight in flight).
+// 16 x 16 x 262,144: 1.40 ms per CholeskyQR2 call (a pair per thread with all loads its own: 3.1).
+constexpr int kG32Pts = 8, kG32Ld = kG32Pts + 1;
+
+template <int kOwnTiles>   // tiles per warp
+__global__ void __launch_bounds__(32 * kGramWarps) gram32_kernel(const cpx<float>* __restrict__ X, int k, int64_t n,
+                                                                const int64_t* __restrict__ inst_off, int n_inst,
+                                                                cpx<double>* __restrict__ G) {
+  constexpr int T = 4, NV = 2 * T * T;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  cpx<float>* bufs = reinterpret_cast<cpx<float>*>(smem_raw);      // [2][kt T][32 slabs][kG32Ld], rows from k on zero
+  const int inst = blockIdx.y;
+  const int j = blockIdx.z;
+  const int64_t p0 = inst_off[inst], p1 = inst_off[inst + 1];
+  const int64_t c0 = p0 + (int64_t)blockIdx.x * kSlab * 32;
+  if (c0 >= p1) return;
+  const cpx<float>* Xj = X + (int64_t)j * k * n;
+  const int kt = (k + T - 1) / T, tiles = kt * (kt + 1) / 2;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int buf_len = kt * T * 32 * kG32Ld;
+  for (int e = threadIdx.x; e < (kt * T - k) * 32 * kG32Ld; e += blockDim.x)
+    bufs[k * 32 * kG32Ld + e] = bufs[buf_len + k * 32 * kG32Ld + e] = mk<float>(0.f, 0.f);
+  const int rounds = (int)((min((int64_t)kSlab, p1 - c0) + kG32Pts - 1) / kG32Pts);
+  // points [8 s, 8 s + 8) of every slab, zeros past the instance's end
+  auto copy_round = [&](int s) {
+    if (s < rounds) {
+      cpx<float>* dst = bufs + (s & 1) * buf_len;
+      for (int e = threadIdx.x; e < k * 32 * kG32Pts; e += blockDim.x) {
+        const int a = e / (32 * kG32Pts), sl = e / kG32Pts % 32, pp = e % kG32Pts;
+        const int64_t p = c0 + (int64_t)sl * kSlab + s * kG32Pts + pp;
+        const bool in = p < p1;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(
+                         (uint32_t)__cvta_generic_to_shared(dst + (a * 32 + sl) * kG32Ld + pp)),
+                     "l"(Xj + (int64_t)a * n + (in ? p : c0)), "r"(in ? 8 : 0)
+                     : "memory");
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  copy_round(0);
+  float v[kOwnTiles][NV];
+  int ta[kOwnTiles], tb[kOwnTiles];
+#pragma unroll
+  for (int q = 0; q < kOwnTiles; ++q) {
+    ta[q] = tb[q] = 0;
+    if (warp + q * nw < tiles) gram_tile_of(warp + q * nw, kt, T, &ta[q], &tb[q]);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) v[q][i] = 0.f;
+  }
+  for (int s = 0; s < rounds; ++s) {
+    copy_round(s + 1);                                             // into the buffer read before the last barrier
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncthreads();
+    const cpx<float>* xs = bufs + (s & 1) * buf_len + lane * kG32Ld;
+#pragma unroll
+    for (int q = 0; q < kOwnTiles; ++q) {
+      if (warp + q * nw >= tiles) break;
+      const cpx<float>* xa = xs + ta[q] * 32 * kG32Ld;
+      const cpx<float>* xb = xs + tb[q] * 32 * kG32Ld;
+#pragma unroll
+      for (int pp = 0; pp < kG32Pts; ++pp) {
+        cpx<float> a[T], b[T];
+#pragma unroll
+        for (int i = 0; i < T; ++i) {
+          a[i] = xa[i * 32 * kG32Ld + pp];
+          b[i] = xb[i * 32 * kG32Ld + pp];
+        }
+#pragma unroll
+        for (int i = 0; i < T; ++i)
+#pragma unroll
+          for (int l = 0; l < T; ++l) {
+            float& re = v[q][2 * (i * T + l)];
+            float& im = v[q][2 * (i * T + l) + 1];
+            re = fmaf(a[i].re, b[l].re, fmaf(a[i].im, b[l].im, re));
+            im = fmaf(a[i].re, b[l].im, fmaf(-a[i].im, b[l].re, im));
+          }
+      }
+    }
+    __syncthreads();
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  double* g = reinterpret_cast<double*>(G + ((int64_t)j * n_inst + inst) * k * k);
+#pragma unroll
+  for (int q = 0; q < kOwnTiles; ++q) {
+    if (warp + q * nw >= tiles) break;
+    double d[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) d[i] = (double)v[q][i];
+    const double t = warp_scatter_sum<NV>(d, lane);                // value `lane` over the slabs
+    const int pair = lane >> 1, a = ta[q] + pair / T, b = tb[q] + pair % T;
+    if (a >= k || b >= k) continue;
+    atomicAdd(g + 2 * (a * k + b) + (lane & 1), t);
+    if (ta[q] != tb[q]) atomicAdd(g + 2 * (b * k + a) + (lane & 1), (lane & 1) ? -t : t);   // the mirrored tile
   }
 }
 
@@ -202,16 +300,23 @@ cudaError_t launch_gram(const void* X, int n_omega, int k, int64_t n, const int6
   cudaError_t e = cudaMemsetAsync(G, 0, sizeof(cpx<double>) * (size_t)n_omega * n_inst * k * k, st);
   if (e != cudaSuccess) return e;
   // chunks per instance: enough for the longest instance (short instances return early)
-  const int64_t per_cta = (int64_t)kSlab * kSlabsPerCta;
+  constexpr bool f32 = sizeof(R) == 4;
+  constexpr int T = f32 ? 4 : 2;
+  const int64_t per_cta = (int64_t)kSlab * (f32 ? 32 : kSlabsPerCta);
   dim3 grid((unsigned)((max_len + per_cta - 1) / per_cta), (unsigned)n_inst, (unsigned)n_omega);
-  constexpr int T = gram_tile<R>();
   const int kt = (k + T - 1) / T, tiles = kt * (kt + 1) / 2;
-  const size_t smem = 2 * sizeof(cpx<R>) * (size_t)kt * T * kSlab;
+  const size_t smem = 2 * sizeof(cpx<R>) * (size_t)kt * T * (f32 ? 32 * kG32Ld : kSlab);
+  void (*kernel)(const cpx<R>*, int, int64_t, const int64_t*, int, cpx<double>*);
+  if constexpr (f32)
+    kernel = tiles <= kGramWarps ? gram32_kernel<1> : gram32_kernel<3>;
+  else
+    kernel = gram64_kernel;
   if (smem > 48 * 1024) {
-    e = cudaFuncSetAttribute(gram_kernel<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  gram_kernel<R><<<grid, 32 * (tiles < kGramWarps ? tiles : kGramWarps), smem, st>>>((const cpx<R>*)X, k, n, inst_off, n_inst, G);
+  const int warps = tiles > kGramWarps ? kGramWarps : f32 && tiles < 4 ? 4 : tiles;   // FP32: four share the copies
+  kernel<<<grid, 32 * warps, smem, st>>>((const cpx<R>*)X, k, n, inst_off, n_inst, G);
   return cudaGetLastError();
 }
 
