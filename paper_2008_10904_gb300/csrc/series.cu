@@ -94,29 +94,46 @@ __device__ void derivs(const T* src, int64_t stride, int64_t n_in, int rev, int6
 
 // F[tau][r] = g(t) at t = (q0 + tau) h / 2: the interpolant on the interval of the sample
 // spacing d = every h that holds t, the last sample at its own time, zero after it.
+// A thread takes one row and one interval (up to 16 stage times of it): the samples and derivatives of its two ends are read and formed
+// once for these stage times, and what is left per value is the polynomial and the store
+// (a thread per value, with its 64-bit divisions and up to ten sample reads: 1.13 ms for 769 stage times of
+// 131,072 rows; 0.35 ms like this, 403 MB written).  Block (x: rows, y: pieces of the
+// intervals from q0's on).
+constexpr int kPieceTimes = 16;
+
 template <typename T, typename R>
-__global__ void series_forcing_kernel(const T* __restrict__ src, int64_t stride, int64_t n_in, int rev, int every,
-                                      int kind, int64_t q0, int n_tau, int64_t rows, T* __restrict__ F) {
-  const int64_t total = (int64_t)n_tau * rows;
+__global__ void __launch_bounds__(256) series_forcing_kernel(const T* __restrict__ src, int64_t stride, int64_t n_in,
+                                                             int rev, int every, int kind, int64_t q0, int n_tau,
+                                                             int64_t rows, T* __restrict__ F) {
+  const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (r >= rows) return;
   const int64_t span = 2 * (int64_t)every;
   const int64_t q_end = span * (n_in - 1);
-  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t tau = idx / rows;
-    const int64_t r = idx - tau * rows;
-    const int64_t q = q0 + tau;
-    T out = zero_of<T>();
-    if (q < q_end) {
-      const int64_t i = q / span;
+  const int64_t pieces = (span + kPieceTimes - 1) / kPieceTimes;
+  for (int64_t y = blockIdx.y;; y += gridDim.y) {
+    const int64_t i = q0 / span + y / pieces, p0 = i * span + y % pieces * kPieceTimes;
+    if (i * span >= q0 + n_tau) break;
+    const int64_t qa = max(q0, p0), qb = min(q0 + n_tau, min(p0 + kPieceTimes, (i + 1) * span));
+    if (qa >= qb) continue;
+    T* f = F + (qa - q0) * rows + r;
+    if (i >= n_in - 1) {
+      for (int64_t q = qa; q < qb; ++q, f += rows)
+        *f = q == q_end ? sample(src, stride, n_in, rev, n_in - 1, r) : zero_of<T>();
+      continue;
+    }
+    const T x0 = sample(src, stride, n_in, rev, i, r);
+    const T x1 = sample(src, stride, n_in, rev, i + 1, r);
+    T v0 = zero_of<T>(), v1 = v0, a0 = v0, a1 = v0;
+    if (kind != 0) {
+      derivs<T, R>(src, stride, n_in, rev, i, r, kind, &v0, &a0);
+      derivs<T, R>(src, stride, n_in, rev, i + 1, r, kind, &v1, &a1);
+    }
+    for (int64_t q = qa; q < qb; ++q, f += rows) {
       const R s = R(q - i * span) / R(span);
-      const T x0 = sample(src, stride, n_in, rev, i, r);
-      const T x1 = sample(src, stride, n_in, rev, i + 1, r);
+      T out;
       if (kind == 0) {
         out = add(scl(R(1) - s, x0), scl(s, x1));
       } else {
-        T v0, v1, a0, a1;
-        derivs<T, R>(src, stride, n_in, rev, i, r, kind, &v0, &a0);
-        derivs<T, R>(src, stride, n_in, rev, i + 1, r, kind, &v1, &a1);
         const R s2 = s * s, s3 = s2 * s;
         if (kind == 1) {   // cubic Hermite: values and first derivatives at both ends
           const R h00 = R(2) * s3 - R(3) * s2 + R(1), h10 = s3 - R(2) * s2 + s;
@@ -133,10 +150,8 @@ __global__ void series_forcing_kernel(const T* __restrict__ src, int64_t stride,
           out = add(add(add(scl(b0, x0), scl(b1, v0)), scl(b2, a0)), add(add(scl(b5, x1), scl(b4, v1)), scl(b3, a1)));
         }
       }
-    } else if (q == q_end) {
-      out = sample(src, stride, n_in, rev, n_in - 1, r);
+      *f = out;
     }
-    F[idx] = out;
   }
 }
 
@@ -421,7 +436,10 @@ rsv_status series_march_impl(rsv_operator op, bool adjoint, int k, const void* i
       if (forced) {
         ProfScope ps(op, PROF_SYNTH);
         const int n_tau = 2 * steps + 1;
-        series_forcing_kernel<T, R><<<grid_for((int64_t)n_tau * rows, thr, op->sm_count), thr, 0, st>>>(
+        const int64_t span = 2 * (int64_t)every, pieces = (span + kPieceTimes - 1) / kPieceTimes;
+        const int64_t ny = ((2 * n0 + n_tau - 1) / span - 2 * n0 / span + 1) * pieces;
+        const dim3 grid((unsigned)((rows + 255) / 256), (unsigned)std::min<int64_t>(ny, 65535));
+        series_forcing_kernel<T, R><<<grid, 256, 0, st>>>(
             static_cast<const T*>(forcing) + (int64_t)v0 * n, out_stride, n_in, reverse_in ? 1 : 0, every, o.interp,
             2 * n0, n_tau, rows, static_cast<T*>(op->ws_ftile.ptr));
         if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "series forcing");
