@@ -119,6 +119,14 @@ __device__ __forceinline__ void adv3d_apply(const R* __restrict__ xv, int i, int
   }
 }
 
+// The stage kernels are launched as programmatic dependents of each other: a CTA may be resident before the
+// previous stage ends, waits for it here, ahead of every access, and then lets the next stage launch (171 x 129,
+// 2 vectors, 676 sampled steps: 6.0 -> 5.5 ms).
+__device__ __forceinline__ void wait_for_previous_stage() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Stage update at one state value given k (without forcing) and the forcing value.
 template <typename R, int STAGE>
 __device__ __forceinline__ void stage_update(int64_t p, R k, const R* __restrict__ u, R* __restrict__ acc,
@@ -147,6 +155,7 @@ __global__ void __launch_bounds__(256) adr2d_stage_kernel(StGeom g, const R* __r
   const int j = blockIdx.y * 8 + threadIdx.y;
   const int v = blockIdx.z;
   if (i >= g.nx || j >= g.ny) return;
+  wait_for_previous_stage();
   const int64_t base = (int64_t)v * g.n;
   const int64_t p = base + (int64_t)j * g.nx + i;
   R k = adr2d_apply<R>(xin + base, i, j, g);
@@ -162,6 +171,7 @@ __global__ void __launch_bounds__(256) adv3d_stage_kernel(StGeom g, const R* __r
   const int jz = blockIdx.y * 8 + threadIdx.y;  // (j, kz) flattened
   const int v = blockIdx.z;
   if (i >= g.nx || jz >= g.ny * g.nz) return;
+  wait_for_previous_stage();
   const int j = jz % g.ny, kz = jz / g.ny;
   const int64_t base = (int64_t)v * g.n;
   const int64_t ncell = (int64_t)g.nx * g.ny * g.nz;
@@ -243,6 +253,7 @@ __global__ void __launch_bounds__(256) adr2d_stage4_kernel(StGeom g, const float
   const int j = blockIdx.y * 8 + threadIdx.y;
   const int v = blockIdx.z;
   if (i0 >= g.nx || j >= g.ny) return;
+  wait_for_previous_stage();
   const int nx = g.nx, ny = g.ny;
   const int64_t base = (int64_t)v * g.n;
   const float* xv = xin + base;
@@ -284,6 +295,7 @@ __global__ void __launch_bounds__(256) adv3d_stage4_kernel(StGeom g, const S* __
   const int i0 = 4 * ((cb % nxb) * 32 + threadIdx.x);
   const int jz = (cb / nxb) * 8 + threadIdx.y;
   if (i0 >= g.nx || jz >= g.ny * g.nz) return;
+  wait_for_previous_stage();
   const int nx = g.nx, ny = g.ny, nz = g.nz;
   const int j = jz % ny, kz = jz / ny;
   const int64_t base = (int64_t)v * g.n;
@@ -1219,6 +1231,20 @@ bool adr2d_fused_enabled() {
   return e != nullptr && e[0] == '1';
 }
 
+template <typename K, typename... A>
+cudaError_t launch_stage_kernel(rsv_operator op, K kernel, dim3 grid, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(32, 8);
+  cfg.stream = op->stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 template <typename R, int STAGE>
 cudaError_t launch_stage(rsv_operator op, const StGeom& g, const R* xin, const R* u, R* acc, const R* f, R* xout,
                          R* ysnap, R h) {
@@ -1232,28 +1258,26 @@ cudaError_t launch_stage(rsv_operator op, const StGeom& g, const R* xin, const R
     const unsigned gx = (unsigned)((g.nx / 4 + 31) / 32);
     if (op->kind == RSV_OP_ADR2D) {
       dim3 grid(gx, (unsigned)((g.ny + 7) / 8), (unsigned)g.kg);
-      adr2d_stage4_kernel<STAGE><<<grid, dim3(32, 8), 0, op->stream>>>(g, xi, uu, ac, ff, xo, ys, (float)h);
+      return launch_stage_kernel(op, adr2d_stage4_kernel<STAGE>, grid, g, xi, uu, ac, ff, xo, ys, (float)h);
     } else {
       const unsigned blocks = gx * (unsigned)((g.ny * g.nz + 7) / 8) * (unsigned)g.kg;
       if (op->bf16_state) {
         // xin, u, xout hold BF16 values at the FP32 slots' addresses
-        adv3d_stage4_kernel<STAGE, __nv_bfloat16><<<blocks, dim3(32, 8), 0, op->stream>>>(
-            g, reinterpret_cast<const __nv_bfloat16*>(xin), reinterpret_cast<const __nv_bfloat16*>(u), ac, ff,
-            reinterpret_cast<__nv_bfloat16*>(xout), ys, (float)h);
+        return launch_stage_kernel(op, adv3d_stage4_kernel<STAGE, __nv_bfloat16>, dim3(blocks), g,
+                                   reinterpret_cast<const __nv_bfloat16*>(xin), reinterpret_cast<const __nv_bfloat16*>(u),
+                                   ac, ff, reinterpret_cast<__nv_bfloat16*>(xout), ys, (float)h);
       } else {
-        adv3d_stage4_kernel<STAGE, float><<<blocks, dim3(32, 8), 0, op->stream>>>(g, xi, uu, ac, ff, xo, ys, (float)h);
+        return launch_stage_kernel(op, adv3d_stage4_kernel<STAGE, float>, dim3(blocks), g, xi, uu, ac, ff, xo, ys, (float)h);
       }
     }
-    return cudaGetLastError();
   }
   if (op->kind == RSV_OP_ADR2D) {
     dim3 grid((unsigned)((g.nx + 31) / 32), (unsigned)((g.ny + 7) / 8), (unsigned)g.kg);
-    adr2d_stage_kernel<R, STAGE><<<grid, dim3(32, 8), 0, op->stream>>>(g, xin, u, acc, f, xout, ysnap, h);
+    return launch_stage_kernel(op, adr2d_stage_kernel<R, STAGE>, grid, g, xin, (const R*)u, acc, f, xout, ysnap, h);
   } else {
     dim3 grid((unsigned)((g.nx + 31) / 32), (unsigned)((g.ny * g.nz + 7) / 8), (unsigned)g.kg);
-    adv3d_stage_kernel<R, STAGE><<<grid, dim3(32, 8), 0, op->stream>>>(g, xin, u, acc, f, xout, ysnap, h);
+    return launch_stage_kernel(op, adv3d_stage_kernel<R, STAGE>, grid, g, xin, (const R*)u, acc, f, xout, ysnap, h);
   }
-  return cudaGetLastError();
 }
 
 }  // namespace
