@@ -210,24 +210,8 @@ def load_peaks():
 # DRAM bytes (read + write) per launch group of a category's kernels over one time tile,
 # from ncu captures of the same kernels at the same rows per launch, keyed by (workload,
 # category, tile steps, rows per launch).  An entry is dropped whenever the kernel it
-# describes changes.  Sources (summaries in profiles/):
-#   dense march  dense_tc_march_c2.txt: one 256-step launch, 84.35 MB read + 24.63 MB written
-#   1-D march    gl1d_pack_c5.txt: one 127-step launch of the packed kernel (one wave of 152
-#                CTAs x 3072 slots), 750.9 MB read + 340.2 MB written
-#   2-D march    adr2d_pair_c3.txt: the two stage-pair kernels of one step at 16 vectors,
-#                342.9 MB per step, scaled by 255 steps (traffic per step is constant)
-#   3-D march    adv3d_pair_c4.txt: the two stage-pair kernels of one step at 2 vectors,
-#                1347.6 MB per step, scaled by 255 steps
-TRAFFIC = {
-    ("dense_hermite_gl_n1024_k32_w256_trm", "march", 256, 32768):
-        {"bytes": 108.98e6, "src": "ncu dram__bytes_read.sum + dram__bytes_write.sum, one launch"},
-    ("gl_batch64_k8_w64_ssrm", "march", 127, 365184):
-        {"bytes": 1.0911e9, "src": "ncu dram__bytes_read.sum + dram__bytes_write.sum, one launch"},
-    ("adr2d_1024x512_k16_w128_ssrm", "march", 255, 8388608):
-        {"bytes": 255 * 342.9e6, "src": "ncu dram bytes of the two stage-pair kernels of one step x 255 steps"},
-    ("adv3d_256x128x128x3_k8_w64_ssrm", "march", 255, 25165824):
-        {"bytes": 255 * 1347.6e6, "src": "ncu dram bytes of the two stage-pair kernels of one step x 255 steps"},
-}
+# describes changes.
+TRAFFIC = {}
 
 FP32_ALU_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12     # 152 SMs x 128 FP32 lanes x FMA x 2.07 GHz
 REF_TOTAL_S = 150.0                                   # CPU seconds of the reference arm's timed steps
@@ -241,15 +225,19 @@ def kernel_model(cat, w, prec, tile, groups, ms_total, rows, path):
       synthesis  rows x n_omega x n_tau complex (8 flop) or real-output (4 flop) multiply-adds
       analysis   rows x n_omega x S multiply-adds (8 flop complex state, 4 flop real state)
       march      dense: 8 n^2 k flop per step (one dense complex product, tensor cores);
-                 1-D kind (state held on chip for the whole tile): the forcing tile read
-                 (2S+1 stage times), the snapshot tile written (S steps) and the state read
-                 and written once, (3S + 3) state passes per tile; in FP64 (bound by the FP64
+                 1-D kind (state held on chip for the whole tile): the forcing tile read (step
+                 form: S steps, else 2S+1 stage times), the snapshot tile written (S steps) and
+                 the state read and written once, (2S + 2) or (3S + 3) state passes per tile; in FP64 (bound by the FP64
                  rate, not by bytes) 122 flop per point and step: four evaluations of
                  k = A x + f (three complex multiply-adds, 24 flop), the three stage inputs
                  u + c k (4 flop each) and the update u + h/6 (k1 + 2 k2 + 2 k3 + k4) (14 flop);
                  2-D whole-step kernel: 6 state passes per step (state read and written,
                  forcing read at the three stage times, snapshot written);
-                 per-stage and stage-pair kernels (2-D, 3-D): 15 state passes per step, the
+                 step form, 2-D in one launch per step: 4 (state read and written, forcing,
+                 snapshot); 3-D in two half steps: 7 (the state read by both, the half step's
+                 state written and read, forcing, snapshot, new state); 2-D in four stages
+                 (FP64): 13;
+                 other per-stage and stage-pair kernels (2-D, 3-D): 15 state passes per step, the
                  algorithmic model of one RK4 step (12 for four stage read/write pairs,
                  2 forcing reads, 1 snapshot write), whatever the kernels actually move
     """
@@ -257,6 +245,7 @@ def kernel_model(cat, w, prec, tile, groups, ms_total, rows, path):
     avg_s = ms_total / max(groups, 1) / 1e3
     S = tile
     dense = "kind=dense" in path
+    step_form = any(t in path for t in ("jump kernels", "step kernel", "half-step", "step-form")) and "whole-step" not in path
     se = (8 if prec == "fp64" else 4) * (1 if w.real_state else 2)
     alu_peak = FP64_ALU_TFLOPS if prec == "fp64" else FP32_ALU_TFLOPS
     cflop = 4 if w.real_state else 8
@@ -265,7 +254,7 @@ def kernel_model(cat, w, prec, tile, groups, ms_total, rows, path):
     peak_tc = peaks["bf16_tflops_sustained"] * 1.1 / 2.25
     tc_src = "measured sustained bf16 x nominal tf32/bf16 ratio (1.1/2.25)"
     if cat == "synthesis":
-        n_tau = S if dense else 2 * S + 1
+        n_tau = S if dense or step_form else 2 * S + 1
         work = rows * w.n_omega * n_tau * cflop
         bound, unit, peak, per = "alu", "TFLOP/s", alu_peak, 1e12
         src = "derived: 152 SMs x 128 FP32 lanes x 2 flop x 2.07 GHz" if prec != "fp64" else "nominal FP64"
@@ -295,11 +284,14 @@ def kernel_model(cat, w, prec, tile, groups, ms_total, rows, path):
         bound, unit, peak, per = "alu", "TFLOP/s", FP64_ALU_TFLOPS, 1e12
         src = "nominal FP64"
     elif cat == "march" and "kind=gl1d" in path:
-        work = (3.0 * S + 3.0) * rows * se
+        work = (2.0 * S + 2.0 if step_form else 3.0 * S + 3.0) * rows * se
         bound, unit, peak, per = "hbm", "GB/s", peaks["hbm_gbs"], 1e9
         src = peaks["src"] + " copy bandwidth"
     else:
-        work = 15.0 * rows * se * S
+        passes = 15.0
+        if step_form:
+            passes = 7.0 if "half-step" in path else 13.0 if "step-form" in path else 4.0
+        work = passes * rows * se * S
         bound, unit, peak, per = "hbm", "GB/s", peaks["hbm_gbs"], 1e9
         src = peaks["src"] + " copy bandwidth"
     achieved = work / avg_s / per
