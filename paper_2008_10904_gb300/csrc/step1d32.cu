@@ -12,9 +12,9 @@
 // copies.  The tiles (forcing, snapshots, transformed coefficients, accumulators) keep the packs' slot
 // order, so that every access is a 16-byte one and the contractions always take their pipelined kernel.
 // One forcing per step instead of stage times halves the forcing tile and its synthesis.  FP32 issue bounds
-// it (about 62 multiply-adds per point and step): 64 instances of 256 to 2048 points, 8 vectors, 10822 steps
-// march in 25.4 ms and are synthesised in 8.5 ms; one stage per barrier, a point per thread and three
-// forcings per step took 44.7 and 16.7 ms, the whole call 79.6 ms instead of 50.8.
+// it (about 62 multiply-adds per point and step, issue 49% with one CTA per SM and one barrier per step): 64
+// instances of 256 to 2048 points, 8 vectors, 10822 steps march in 25.4 ms and are synthesised in 8.3 ms; one
+// stage per barrier, a point per thread and three forcings per step took 44.7 and 16.7 ms.
 #include <algorithm>
 #include <cstdlib>
 #include <functional>
