@@ -201,26 +201,30 @@ cudaError_t synth64(rsv_operator op, const TileGeom& g, const void* coef, void* 
   return cudaGetLastError();
 }
 
-// Runs an analysis of `steps` steps is split into: enough warps for four per SM and scheduler, few
-// enough that a run has at least two slices.
-static int analysis64_runs(rsv_operator op, int64_t rows, int steps) {
-  const int64_t warps = ((rows + 31) / 32) * ((op->n_omega + kJ - 1) / kJ);
+// Runs an analysis of `steps` steps is split into: enough warps for four per SM and scheduler with a
+// single vector of `points` points, few enough that a run has at least two slices.  Not a function of the
+// vectors in the group: the order of the sums is the same however a block is cut into groups, and the
+// partial sums of a smaller group fit where a larger one's did.
+static int analysis64_runs(rsv_operator op, int64_t points, int steps) {
+  const int64_t warps = ((points + 31) / 32) * ((op->n_omega + kJ - 1) / kJ);
   const int slices = (steps + kSlice - 1) / kSlice;
   const int64_t want = (16 * (int64_t)std::max(1, op->sm_count) + warps - 1) / warps;
   return (int)std::max<int64_t>(1, std::min<int64_t>(want, slices / 2));
 }
 
-size_t analysis64_part_bytes(rsv_operator op, int64_t rows, int steps) {
-  const int runs = analysis64_runs(op, rows, steps);
+size_t analysis64_part_bytes(rsv_operator op, int64_t rows, int64_t points, int steps) {
+  const int runs = analysis64_runs(op, points, steps);
   return runs > 1 ? (size_t)runs * op->n_omega * rows * sizeof(cd) : 0;
 }
 
-// acc += the Fourier sums of the tile steps [s0, s1); part: analysis64_part_bytes(s1 - s0) bytes or more.
-cudaError_t analysis64(rsv_operator op, const TileGeom& g, const void* Y, int s0, int s1, cpx<double>* acc,
-                       int64_t acc_stride, void* part) {
+// acc += the Fourier sums of the tile steps [s0, s1) of vectors of `points` points; part: a buffer of part_bytes,
+// analysis64_part_bytes(s1 - s0) or more (InvalidValue otherwise).
+cudaError_t analysis64(rsv_operator op, const TileGeom& g, int64_t points, const void* Y, int s0, int s1,
+                       cpx<double>* acc, int64_t acc_stride, void* part, size_t part_bytes) {
   if (s1 <= s0) return cudaSuccess;
+  if (analysis64_part_bytes(op, g.rows, points, s1 - s0) > part_bytes) return cudaErrorInvalidValue;
   const int slices = (s1 - s0 + kSlice - 1) / kSlice;
-  int runs = analysis64_runs(op, g.rows, s1 - s0);
+  int runs = analysis64_runs(op, points, s1 - s0);
   const int per = (slices + runs - 1) / runs;
   runs = (slices + per - 1) / per;
   const int64_t rg = (g.rows + 31) / 32;

@@ -617,8 +617,9 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
     // one synthesis time per step: as many columns as 2 S + 1 stage times, and half the accumulator traffic
     S = 2 * (S + 1);
   } else if (jump && !truncate && !(opts && opts->tile_steps > 0) && op->tuned_k != k) {
-    // the jumps' launches are short: tiles as long as 128 MB of snapshots, a window at most
-    S = (int)std::max<int64_t>(S, std::min<int64_t>(op->n_t, ((int64_t)128 << 20) / ((int64_t)kg * n * 16)));
+    // the jumps' launches are short: tiles as long as 128 MB of all k vectors' snapshots (the same ones
+    // however the block is cut into groups), a window at most
+    S = (int)std::max<int64_t>(S, std::min<int64_t>(op->n_t, ((int64_t)128 << 20) / ((int64_t)k * n * 16)));
   }
   // rows of the forcing tile: steps and stage times, whole steps only, or whole steps and jumps
   auto f_rows = [&](int s_) -> int64_t { return jump ? s_ + s_ / jp + jp + 1 : sf ? s_ : 2 * (int64_t)s_ + 1; };
@@ -641,7 +642,7 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
         b += (double)tmp;
       }
       if (jump) b += 2.0 * op->n_omega * rows_ * sizeof(cpx<double>);
-      if (op->prec == RSV_PREC_FP64) b += (double)analysis64_part_bytes(op, (int64_t)rows_, s_);
+      if (op->prec == RSV_PREC_FP64) b += (double)analysis64_part_bytes(op, (int64_t)rows_, np, s_);
       if (s_in) b += (double)op->n_omega * rows_ * coef_bytes(op);
       if (op->kind == RSV_OP_DENSE) b += 2.0 * op->n_omega * rows_ * 2 * sizeof(R);
       if (host_in) b += 2.0 * op->n_omega * rows_ * coef_bytes(op);   // staging buffers
@@ -674,7 +675,7 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
     if ((st = ensure(op->ws_coef, cb)) != RSV_OK || (st = ensure(op->ws_coef2, cb)) != RSV_OK) return st;
   }
   if (op->prec == RSV_PREC_FP64) {
-    const size_t pb = analysis64_part_bytes(op, rows_max, S);
+    const size_t pb = analysis64_part_bytes(op, rows_max, np, S);
     if (pb > 0 && (st = ensure(op->ws_part, pb)) != RSV_OK) return st;
   }
   if (!acc_in_out && (st = ensure(op->ws_acc, (size_t)op->n_omega * rows_max * sizeof(cpx<double>))) != RSV_OK)
@@ -839,9 +840,10 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
           ProfScope ps(op, PROF_ANALYSIS, 2);
           e = tc_analysis(op, g, op->ws_ysnap.ptr, y_first, g.steps, acc, acc_stride);
         } else {
-          ProfScope ps(op, PROF_ANALYSIS, sizeof(R) == 8 && analysis64_part_bytes(op, rows, g.steps - y_first) > 0 ? 2 : 1);
+          ProfScope ps(op, PROF_ANALYSIS, sizeof(R) == 8 && analysis64_part_bytes(op, rows, np, g.steps - y_first) > 0 ? 2 : 1);
           if (sizeof(R) == 8)
-            e = analysis64(op, g, op->ws_ysnap.ptr, y_first, g.steps, acc, acc_stride, op->ws_part.ptr);
+            e = analysis64(op, g, np, op->ws_ysnap.ptr, y_first, g.steps, acc, acc_stride, op->ws_part.ptr,
+                           op->ws_part.bytes);
           else
             e = launch_analysis<R>(g, op->ws_ysnap.ptr, y_first, g.steps, op->d_tw, op->d_pj, op->real_state, acc,
                                    acc_stride, stream);

@@ -61,9 +61,9 @@ cudaError_t jump_march(rsv_operator op, TileGeom g, bool adjoint, int kg, int st
 
 // FP64 contractions at whole steps (contract64.cu)
 cudaError_t synth64(rsv_operator op, const TileGeom& g, const void* coef, void* F);
-size_t analysis64_part_bytes(rsv_operator op, int64_t rows, int steps);
-cudaError_t analysis64(rsv_operator op, const TileGeom& g, const void* Y, int s0, int s1, cpx<double>* acc,
-                       int64_t acc_stride, void* part);
+size_t analysis64_part_bytes(rsv_operator op, int64_t rows, int64_t points, int steps);
+cudaError_t analysis64(rsv_operator op, const TileGeom& g, int64_t points, const void* Y, int s0, int s1,
+                       cpx<double>* acc, int64_t acc_stride, void* part, size_t part_bytes);
 
 // S RK4 steps of the operator's stage kernel(s) on the state block (kg vectors).
 template <typename R>
