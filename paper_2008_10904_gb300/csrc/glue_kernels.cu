@@ -16,7 +16,7 @@ namespace {
 
 constexpr int kMaxK = 32;
 
-// FP64: one CTA per (frequency, instance, chunk of points).  The CTA stages the k vectors of 256 points at a
+// FP64: one CTA per (frequency, instance, chunk of points).  The CTA stages the k vectors of 256 (128) points at a
 // time in shared memory (each value read once from HBM, the next slab in flight during the current one).  The
 // k x k Gram is Hermitian and cut into tiles of T x T pairs on and above the diagonal, one or a few per warp: a
 // lane holds the T x T sums of its points (every 32nd), so that 2 T loads feed T^2 complex multiply-adds.  The
@@ -25,6 +25,10 @@ constexpr int kMaxK = 32;
 constexpr int kSlab = 256;
 constexpr int kSlabsPerCta = 8;
 constexpr int kGramWarps = 12;
+// Two slabs of more than 28 vectors exceed the shared memory of a CTA: these take slabs of half the points.
+constexpr int kWideK = 28, kWideSlab = kSlab / 2;
+constexpr size_t gram64_smem(int rows, int slab) { return 2 * sizeof(cpx<double>) * (size_t)rows * slab; }
+static_assert(gram64_smem(kWideK, kSlab) <= 232448 && gram64_smem(kMaxK, kWideSlab) <= 232448, "FP64 Gram slabs");
 
 // v[0 .. N-1] of every lane summed over the warp; lane l returns the sum of value l mod N.
 template <int N, typename R>
@@ -51,6 +55,7 @@ __device__ __forceinline__ void gram_tile_of(int t, int kt, int T, int* ta, int*
   *tb = (a + t) * T;
 }
 
+template <int kSlab64, int kSlabs64>   // points per slab, slabs per CTA
 __global__ void __launch_bounds__(32 * kGramWarps) gram64_kernel(const cpx<double>* __restrict__ X, int k, int64_t n,
                                                                 const int64_t* __restrict__ inst_off, int n_inst,
                                                                 cpx<double>* __restrict__ G) {
@@ -58,26 +63,26 @@ __global__ void __launch_bounds__(32 * kGramWarps) gram64_kernel(const cpx<doubl
   constexpr int T = 2, NV = 2 * T * T;
   constexpr int kMaxOwn = 12;                                       // tiles per warp at k = 32
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cpx<R>* slabs = reinterpret_cast<cpx<R>*>(smem_raw);             // [2][kt T][kSlab], rows from k on zero
+  cpx<R>* slabs = reinterpret_cast<cpx<R>*>(smem_raw);             // [2][kt T][kSlab64], rows from k on zero
   const int inst = blockIdx.y;
   const int j = blockIdx.z;
   const int64_t p0 = inst_off[inst], p1 = inst_off[inst + 1];
-  const int64_t c0 = p0 + (int64_t)blockIdx.x * kSlab * kSlabsPerCta;
+  const int64_t c0 = p0 + (int64_t)blockIdx.x * kSlab64 * kSlabs64;
   if (c0 >= p1) return;
   const cpx<R>* Xj = X + (int64_t)j * k * n;
   const int kt = (k + T - 1) / T, tiles = kt * (kt + 1) / 2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const int slab_len = kt * T * kSlab;
-  for (int e = threadIdx.x; e < (kt * T - k) * kSlab; e += blockDim.x)
-    slabs[k * kSlab + e] = slabs[slab_len + k * kSlab + e] = mk<R>(0, 0);
+  const int slab_len = kt * T * kSlab64;
+  for (int e = threadIdx.x; e < (kt * T - k) * kSlab64; e += blockDim.x)
+    slabs[k * kSlab64 + e] = slabs[slab_len + k * kSlab64 + e] = mk<R>(0, 0);
   // asynchronous copies of slab sl into its buffer (zeros past the instance's end); nothing past the chunk
   auto copy_slab = [&](int sl) {
-    const int64_t s0 = c0 + (int64_t)sl * kSlab;
-    if (sl < kSlabsPerCta && s0 < p1) {
-      const int cnt = (int)min((int64_t)kSlab, p1 - s0);
+    const int64_t s0 = c0 + (int64_t)sl * kSlab64;
+    if (sl < kSlabs64 && s0 < p1) {
+      const int cnt = (int)min((int64_t)kSlab64, p1 - s0);
       cpx<R>* dst = slabs + (sl & 1) * slab_len;
-      for (int e = threadIdx.x; e < k * kSlab; e += blockDim.x) {
-        const int a = e / kSlab, pp = e % kSlab;
+      for (int e = threadIdx.x; e < k * kSlab64; e += blockDim.x) {
+        const int a = e / kSlab64, pp = e % kSlab64;
         const cpx<R>* src = Xj + (int64_t)a * n + s0 + (pp < cnt ? pp : 0);
         asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"((uint32_t)__cvta_generic_to_shared(dst + e)),
                      "l"(src), "n"(sizeof(cpx<R>)), "r"(pp < cnt ? (int)sizeof(cpx<R>) : 0)
@@ -91,10 +96,10 @@ __global__ void __launch_bounds__(32 * kGramWarps) gram64_kernel(const cpx<doubl
   double tot[kMaxOwn];
 #pragma unroll
   for (int q = 0; q < kMaxOwn; ++q) tot[q] = 0.0;
-  for (int sl = 0; sl < kSlabsPerCta; ++sl) {
-    const int64_t s0 = c0 + (int64_t)sl * kSlab;
+  for (int sl = 0; sl < kSlabs64; ++sl) {
+    const int64_t s0 = c0 + (int64_t)sl * kSlab64;
     if (s0 >= p1) break;
-    const int cnt = (int)min((int64_t)kSlab, p1 - s0);
+    const int cnt = (int)min((int64_t)kSlab64, p1 - s0);
     copy_slab(sl + 1);                                             // into the buffer read before the last barrier
     asm volatile("cp.async.wait_group 1;" ::: "memory");
     __syncthreads();
@@ -108,14 +113,14 @@ __global__ void __launch_bounds__(32 * kGramWarps) gram64_kernel(const cpx<doubl
       R v[NV];
 #pragma unroll
       for (int i = 0; i < NV; ++i) v[i] = R(0);
-      const cpx<R>* xa = xs + ta * kSlab + lane;
-      const cpx<R>* xb = xs + tb * kSlab + lane;
+      const cpx<R>* xa = xs + ta * kSlab64 + lane;
+      const cpx<R>* xb = xs + tb * kSlab64 + lane;
       for (int pp = 0; pp < cnt; pp += 32) {                      // points past cnt are zero
         cpx<R> a[T], b[T];
 #pragma unroll
         for (int i = 0; i < T; ++i) {
-          a[i] = xa[i * kSlab + pp];
-          b[i] = xb[i * kSlab + pp];
+          a[i] = xa[i * kSlab64 + pp];
+          b[i] = xb[i * kSlab64 + pp];
         }
 #pragma unroll
         for (int i = 0; i < T; ++i)
@@ -305,12 +310,14 @@ cudaError_t launch_gram(const void* X, int n_omega, int k, int64_t n, const int6
   const int64_t per_cta = (int64_t)kSlab * (f32 ? 32 : kSlabsPerCta);
   dim3 grid((unsigned)((max_len + per_cta - 1) / per_cta), (unsigned)n_inst, (unsigned)n_omega);
   const int kt = (k + T - 1) / T, tiles = kt * (kt + 1) / 2;
-  const size_t smem = 2 * sizeof(cpx<R>) * (size_t)kt * T * (f32 ? 32 * kG32Ld : kSlab);
+  const bool wide = kt * T > kWideK;
+  const size_t smem =
+      f32 ? 2 * sizeof(cpx<R>) * (size_t)kt * T * 32 * kG32Ld : gram64_smem(kt * T, wide ? kWideSlab : kSlab);
   void (*kernel)(const cpx<R>*, int, int64_t, const int64_t*, int, cpx<double>*);
   if constexpr (f32)
     kernel = tiles <= kGramWarps ? gram32_kernel<1> : gram32_kernel<3>;
   else
-    kernel = gram64_kernel;
+    kernel = wide ? gram64_kernel<kWideSlab, kSlabsPerCta * kSlab / kWideSlab> : gram64_kernel<kSlab, kSlabsPerCta>;
   if (smem > 48 * 1024) {
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
