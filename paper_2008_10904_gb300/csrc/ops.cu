@@ -211,6 +211,9 @@ int march_tile_kernels(rsv_operator op, int steps, int kg, bool step_form) {
 
 rsv_status on_frequencies(rsv_operator op) {
   for (JumpPlan& p : op->jump) p = JumpPlan();
+  for (TileGraph& g : op->tile_graphs)   // the captured launches carry the step h
+    if (g.exec) cudaGraphExecDestroy(g.exec);
+  op->tile_graphs.clear();
   if (op->kind == RSV_OP_DENSE) return dense_on_frequencies(op);
   if (op->kind == RSV_OP_GL1D && op->scheme == RSV_SCHEME_CN) return gl1d_cn_factors(op);
   return RSV_OK;
@@ -658,7 +661,8 @@ static cudaError_t march_tile_direct(rsv_operator op, const MarchTile& t, void* 
 // forced steps of the tile), and a sequence met a second time is captured once into a graph on a
 // private stream and replayed on the operator's stream from then on.  The first meeting runs the
 // launches directly (one-time set-up such as shared-memory opt-ins stays outside any capture).  A
-// capture that fails falls back to direct launches for that sequence.  RSV_TILE_GRAPHS=0 disables.
+// capture that fails falls back to direct launches for that sequence.  The launches carry the step h, so
+// a new frequency grid drops all of them (on_frequencies).  RSV_TILE_GRAPHS=0 disables.
 // ---------------------------------------------------------------------------
 static bool tile_graphs_enabled(rsv_operator op) {
   static const bool env = [] {
