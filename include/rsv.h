@@ -346,8 +346,9 @@ rsv_status rsv_march_adjoint_host(rsv_operator op, const void* y_hat_host, int32
                                   void* w_hat);
 
 /* Measured choice of the march's time-tile length and vector-group size for
- * marches of k vectors with these options.  Candidates: the default tile and
- * half of it, times groups of k, k/2, k/4 and 1 vectors that fit in device
+ * marches of k vectors with these options.  Candidates: the tile such a march
+ * takes untuned (the default tile where the march is no longer) and half of
+ * it, times groups of k, k/2, k/4 and 1 vectors that fit in device
  * memory next to what is allocated; each is timed on one synthesised, marched
  * and analysed tile of the first vector group of f_hat (device [n_omega][k][n],
  * the block a following march will use; nothing is written to it), and the

@@ -576,6 +576,21 @@ static void march_scalings(rsv_operator op, int scaling, bool adjoint, const dou
   }
 }
 
+// Tile length of a march of k vectors that neither its options nor rsv_autotune set.
+static int untuned_tile(rsv_operator op, int k, bool truncate) {
+  const int S = default_tile_steps(op);
+  if (truncate) return S;   // the tile ends are the check points
+  // one synthesis time per step: as many columns as 2 S + 1 stage times, and half the accumulator traffic
+  if (step_form_taken(op, k) && tc_contract_segments(op)) return 2 * (S + 1);
+  // the jumps' launches are short: tiles as long as 128 MB of all k vectors' snapshots (the same ones
+  // however the block is cut into groups), a window at most
+  if (jump_taken(op, k))
+    return (int)std::max<int64_t>(S, std::min<int64_t>(op->n_t, ((int64_t)128 << 20) / ((int64_t)k * op->n * 16)));
+  return S;
+}
+
+static bool truncates(const rsv_march_opts* o) { return o != nullptr && o->variant == RSV_TRM && o->tail_tol > 0.0; }
+
 // A timed trial of one tile configuration for rsv_autotune: the first vector group of kg vectors,
 // one forced and analysed time tile of S steps, accumulators in the workspace, nothing written to
 // the caller; *ms receives the device time of the tile's launches.
@@ -600,26 +615,20 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
   const int jp = jump ? jump_plan(op, adjoint).p : 1;
   const int64_t np = sf ? step_points(op) : n;     // points per vector of the march's tiles
   // TRM truncation by the state norm: per-vector peak over the tile ends so far
-  const bool truncate = opts != nullptr && opts->variant == RSV_TRM && opts->tail_tol > 0.0;
+  const bool truncate = truncates(opts);
   auto scratch_bytes = [&](int kg_) { return sf ? step_scratch_bytes(op, kg_) : stage_scratch_bytes(op, kg_); };
   const bool acc_in_out = op->prec == RSV_PREC_FP64 && trial == nullptr && np == n;
   // Tile length S and vector-group size kg: the requested / default tile and all k vectors, shrunk
   // (kg halved, then S down to 16) until the march workspace fits in 90% of the device memory not
   // held by others.
-  int S = (opts && opts->tile_steps > 0) ? opts->tile_steps
-                                         : (op->tuned_k == k ? op->tuned_tile : default_tile_steps(op));
-  int kg = (op->tuned_k == k && !(opts && opts->tile_steps > 0)) ? op->tuned_group : k;
+  const bool tuned = op->tuned_k == k && !(opts && opts->tile_steps > 0);
+  int S = (opts && opts->tile_steps > 0) ? opts->tile_steps : untuned_tile(op, k, truncate);
+  if (tuned) S = truncate ? std::min(S, op->tuned_tile) : op->tuned_tile;   // check points no further apart
+  int kg = tuned ? op->tuned_group : k;
   if (opts && opts->group_vectors > 0) kg = std::min(kg, (int)opts->group_vectors);
   if (trial) {
     S = trial->S;
     kg = trial->kg;
-  } else if (sf && !truncate && tc_contract_segments(op) && !(opts && opts->tile_steps > 0) && op->tuned_k != k) {
-    // one synthesis time per step: as many columns as 2 S + 1 stage times, and half the accumulator traffic
-    S = 2 * (S + 1);
-  } else if (jump && !truncate && !(opts && opts->tile_steps > 0) && op->tuned_k != k) {
-    // the jumps' launches are short: tiles as long as 128 MB of all k vectors' snapshots (the same ones
-    // however the block is cut into groups), a window at most
-    S = (int)std::max<int64_t>(S, std::min<int64_t>(op->n_t, ((int64_t)128 << 20) / ((int64_t)k * n * 16)));
   }
   // rows of the forcing tile: steps and stage times, whole steps only, or whole steps and jumps
   auto f_rows = [&](int s_) -> int64_t { return jump ? s_ + s_ / jp + jp + 1 : sf ? s_ : 2 * (int64_t)s_ + 1; };
@@ -897,12 +906,17 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
 }
 
 // Measured choice of the tile length and vector group (rsv_autotune): candidates S in {D, D/2}
-// (D the default tile) and kg in {k, k/2, k/4, 1}, each timed on one forced and analysed tile of
-// the first vector group (run twice, the second timing kept), compared by time per vector-step.
+// (D the tile an untuned march takes; the default tile where the whole march is no longer than that)
+// and kg in {k, k/2, k/4, 1}, each timed on one forced and analysed tile of the first vector group
+// (run twice, the second timing kept), compared by time per vector-step.
 template <typename R>
 static rsv_status autotune_impl(rsv_operator op, const void* in, int k, const rsv_march_opts* opts, int32_t* tile,
                                 int32_t* group) {
-  const int d = default_tile_steps(op);
+  Schedule sc;
+  rsv_status st = make_schedule(op, opts, false, &sc);
+  if (st != RSV_OK) return st;
+  int d = default_tile_steps(op);
+  if (sc.total > d) d = untuned_tile(op, k, truncates(opts));
   std::vector<int> ss = {d};
   if (d / 2 >= 16) ss.push_back(d / 2);
   std::vector<int> gs;
@@ -915,7 +929,7 @@ static rsv_status autotune_impl(rsv_operator op, const void* in, int k, const rs
       float ms = 0.f;
       int steps = 0;
       TileTrial tr{S, kg, &ms, &steps};
-      rsv_status st = RSV_OK;
+      st = RSV_OK;
       for (int rep = 0; rep < 2 && st == RSV_OK; ++rep)
         st = march_impl<R>(op, in, k, opts, nullptr, false, SCALE_NONE, &tr);
       if (st == RSV_ERR_OOM) continue;   // does not fit next to the caller's blocks
