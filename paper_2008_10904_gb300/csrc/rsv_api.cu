@@ -54,6 +54,11 @@ rsv_status ensure(Workspace& w, size_t bytes) {
   return RSV_OK;
 }
 
+void release(Workspace& w) {
+  if (w.ptr) cudaFree(w.ptr);
+  w = Workspace();
+}
+
 rsv_status upload(rsv_operator op, const void* host, size_t bytes, void** dst) {
   void* p = nullptr;
   cudaError_t e = cudaMalloc(&p, bytes < 16 ? 16 : bytes);
@@ -598,6 +603,7 @@ struct TileTrial {
   int S, kg;
   float* ms;
   int* steps;   // steps of the timed tile
+  bool plain;   // without step form and jumps
 };
 
 template <typename R>
@@ -610,63 +616,72 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
   if (st != RSV_OK) return st;
   const int64_t n = op->n;
   const size_t se = state_elem_bytes(op);
-  const bool sf = step_form_taken(op, k);
-  const bool jump = jump_taken(op, k);
-  const int jp = jump ? jump_plan(op, adjoint).p : 1;
-  const int64_t np = sf ? step_points(op) : n;     // points per vector of the march's tiles
   // TRM truncation by the state norm: per-vector peak over the tile ends so far
   const bool truncate = truncates(opts);
+  // The form of the march: step form or jumps (neither: the caller's coefficients are read in place at the
+  // stage times), points per vector of its tiles, tile length S and vector-group size kg.
+  bool sf = false, jump = false, acc_in_out = false;
+  int jp = 1, S = 0, kg = 0;
+  int64_t np = n;
   auto scratch_bytes = [&](int kg_) { return sf ? step_scratch_bytes(op, kg_) : stage_scratch_bytes(op, kg_); };
-  const bool acc_in_out = op->prec == RSV_PREC_FP64 && trial == nullptr && np == n;
-  // Tile length S and vector-group size kg: the requested / default tile and all k vectors, shrunk
-  // (kg halved, then S down to 16) until the march workspace fits in 90% of the device memory not
-  // held by others.
-  const bool tuned = op->tuned_k == k && !(opts && opts->tile_steps > 0);
-  int S = (opts && opts->tile_steps > 0) ? opts->tile_steps : untuned_tile(op, k, truncate);
-  if (tuned) S = truncate ? std::min(S, op->tuned_tile) : op->tuned_tile;   // check points no further apart
-  int kg = tuned ? op->tuned_group : k;
-  if (opts && opts->group_vectors > 0) kg = std::min(kg, (int)opts->group_vectors);
-  if (trial) {
-    S = trial->S;
-    kg = trial->kg;
-  }
   // rows of the forcing tile: steps and stage times, whole steps only, or whole steps and jumps
   auto f_rows = [&](int s_) -> int64_t { return jump ? s_ + s_ / jp + jp + 1 : sf ? s_ : 2 * (int64_t)s_ + 1; };
-  {
-    size_t free_b = 0, total_b = 0;
-    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
-      cudaGetLastError();
-      free_b = (size_t)1 << 62;
+  auto need = [&](int s_, int kg_) {
+    const double rows_ = (double)kg_ * np;
+    double b = rows_ * se + (double)scratch_bytes(kg_) + (double)f_rows(s_) * rows_ * se + s_ * rows_ * se;
+    if (!acc_in_out) b += (double)op->n_omega * rows_ * sizeof(cpx<double>);
+    if (sf) {
+      size_t tmp = 0;
+      b += (double)step_coef_bytes(op, kg_, &tmp);
+      b += (double)tmp;
     }
-    const size_t held = op->ws_state.bytes + op->ws_ftile.bytes + op->ws_ysnap.bytes + op->ws_acc.bytes +
-                        op->ws_coef.bytes + op->ws_coef2.bytes;
-    const double budget = 0.9 * (double)(free_b + held);
-    auto need = [&](int s_, int kg_) {
-      const double rows_ = (double)kg_ * np;
-      double b = rows_ * se + (double)scratch_bytes(kg_) + (double)f_rows(s_) * rows_ * se + s_ * rows_ * se;
-      if (!acc_in_out) b += (double)op->n_omega * rows_ * sizeof(cpx<double>);
-      if (sf) {
-        size_t tmp = 0;
-        b += (double)step_coef_bytes(op, kg_, &tmp);
-        b += (double)tmp;
-      }
-      if (jump) b += 2.0 * op->n_omega * rows_ * sizeof(cpx<double>);
-      if (op->prec == RSV_PREC_FP64) b += (double)analysis64_part_bytes(op, (int64_t)rows_, np, s_);
-      if (s_in) b += (double)op->n_omega * rows_ * coef_bytes(op);
-      if (op->kind == RSV_OP_DENSE) b += 2.0 * op->n_omega * rows_ * 2 * sizeof(R);
-      if (host_in) b += 2.0 * op->n_omega * rows_ * coef_bytes(op);   // staging buffers
-      return b;
-    };
-    // per-tile traffic (coefficients, FP64 accumulators) is amortised over S, while the vector
-    // group only sets how much is resident: shrink the group first, then the tile
-    if (trial && need(S, kg) > budget) return fail(RSV_ERR_OOM, "trial configuration does not fit");
+    if (jump) b += 2.0 * op->n_omega * rows_ * sizeof(cpx<double>);
+    if (op->prec == RSV_PREC_FP64) b += (double)analysis64_part_bytes(op, (int64_t)rows_, np, s_);
+    if (s_in) b += (double)op->n_omega * rows_ * coef_bytes(op);
+    if (op->kind == RSV_OP_DENSE) b += 2.0 * op->n_omega * rows_ * 2 * sizeof(R);
+    if (host_in) b += 2.0 * op->n_omega * rows_ * coef_bytes(op);   // staging buffers
+    return b;
+  };
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    cudaGetLastError();
+    free_b = (size_t)1 << 62;
+  }
+  const size_t held = op->ws_state.bytes + op->ws_ftile.bytes + op->ws_ysnap.bytes + op->ws_acc.bytes +
+                      op->ws_coef.bytes + op->ws_coef2.bytes;
+  const double budget = 0.9 * (double)(free_b + held);
+  // The requested / default tile and all k vectors, shrunk (kg halved, then S down to 16) until the march
+  // workspace fits in 90% of the device memory not held by others; false when the smallest does not.
+  // Per-tile traffic (coefficients, FP64 accumulators) is amortised over S, while the vector group only
+  // sets how much is resident: the group shrinks first, then the tile.
+  const bool tuned = op->tuned_k == k && !(opts && opts->tile_steps > 0);
+  auto plan = [&](bool plain) -> bool {
+    sf = !plain && step_form_taken(op, k);
+    jump = !plain && jump_taken(op, k);
+    jp = jump ? jump_plan(op, adjoint).p : 1;
+    np = sf ? step_points(op) : n;
+    acc_in_out = op->prec == RSV_PREC_FP64 && trial == nullptr && np == n;
+    S = (opts && opts->tile_steps > 0) ? opts->tile_steps : plain ? default_tile_steps(op) : untuned_tile(op, k, truncate);
+    if (tuned) S = truncate || plain ? std::min(S, op->tuned_tile) : op->tuned_tile;   // check points no further apart
+    kg = tuned ? op->tuned_group : k;
+    if (opts && opts->group_vectors > 0) kg = std::min(kg, (int)opts->group_vectors);
+    if (trial) {
+      S = trial->S;
+      kg = trial->kg;
+      return need(S, kg) <= budget;
+    }
     while (need(S, kg) > budget && (S > 16 || kg > 1)) {
       if (kg > 1)
         kg = (kg + 1) / 2;
       else
         S = std::max(16, S / 2);
     }
-  }
+    return need(S, kg) <= budget;
+  };
+  const bool fits = plan(trial != nullptr && trial->plain);
+  if (trial && !fits) return fail(RSV_ERR_OOM, "trial configuration does not fit");
+  // the transformed coefficients of one vector do not fit: march at the stage times, which needs none
+  if (!fits && (sf || jump)) plan(true);
   const cudaStream_t stream = op->stream;
   cudaError_t e;
   op->last_tile = S;
@@ -675,6 +690,20 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
   const bool packed = sf && op->kind == RSV_OP_GL1D;
   if (packed && (st = step32_packs(op, kg)) != RSV_OK) return st;
   const int64_t rows_max = (int64_t)kg * np;
+  {
+    // Near the limit the plan counts on memory that workspaces of another shape hold: these go first.
+    size_t c2 = 0;
+    const size_t c1 = sf ? step_coef_bytes(op, kg, &c2)
+                         : jump || op->kind == RSV_OP_DENSE ? (c2 = (size_t)op->n_omega * rows_max * coef_bytes(op)) : 0;
+    const std::pair<Workspace*, size_t> want[] = {
+        {&op->ws_state, rows_max * se + scratch_bytes(kg)}, {&op->ws_ftile, (size_t)f_rows(S) * rows_max * se},
+        {&op->ws_ysnap, (size_t)S * rows_max * se}, {&op->ws_coef, c1}, {&op->ws_coef2, c2},
+        {&op->ws_acc, acc_in_out ? 0 : (size_t)op->n_omega * rows_max * sizeof(cpx<double>)}};
+    bool grow = false;
+    for (const auto& w : want) grow = grow || w.second > w.first->bytes;
+    if (grow && need(S, kg) > 0.9 * (double)free_b)
+      for (const auto& w : want) release(*w.first);
+  }
   if ((st = ensure(op->ws_state, rows_max * se + scratch_bytes(kg))) != RSV_OK) return st;
   if ((st = ensure(op->ws_ftile, (size_t)f_rows(S) * rows_max * se)) != RSV_OK) return st;
   if ((st = ensure(op->ws_ysnap, (size_t)S * rows_max * se)) != RSV_OK) return st;
@@ -915,32 +944,34 @@ static rsv_status autotune_impl(rsv_operator op, const void* in, int k, const rs
   Schedule sc;
   rsv_status st = make_schedule(op, opts, false, &sc);
   if (st != RSV_OK) return st;
-  int d = default_tile_steps(op);
-  if (sc.total > d) d = untuned_tile(op, k, truncates(opts));
-  std::vector<int> ss = {d};
-  if (d / 2 >= 16) ss.push_back(d / 2);
   std::vector<int> gs;
   for (int c : {k, (k + 1) / 2, (k + 3) / 4, 1})
     if (std::find(gs.begin(), gs.end(), c) == gs.end()) gs.push_back(c);
   double best = 1e300;
   int bs = 0, bg = 0;
-  for (int S : ss)
-    for (int kg : gs) {
-      float ms = 0.f;
-      int steps = 0;
-      TileTrial tr{S, kg, &ms, &steps};
-      st = RSV_OK;
-      for (int rep = 0; rep < 2 && st == RSV_OK; ++rep)
-        st = march_impl<R>(op, in, k, opts, nullptr, false, SCALE_NONE, &tr);
-      if (st == RSV_ERR_OOM) continue;   // does not fit next to the caller's blocks
-      if (st != RSV_OK) return st;
-      const double per = (double)ms / ((double)std::max(steps, 1) * std::min(kg, k));
-      if (per < best) {
-        best = per;
-        bs = S;
-        bg = kg;
+  const bool forms = step_form_taken(op, k) || jump_taken(op, k);
+  for (int plain = 0; plain <= (forms ? 1 : 0) && bs == 0; ++plain) {   // second pass: where the march falls back to
+    int d = default_tile_steps(op);
+    if (!plain && sc.total > d) d = untuned_tile(op, k, truncates(opts));
+    for (int S : {d, d / 2 >= 16 ? d / 2 : 0})
+      for (int kg : gs) {
+        if (S == 0) continue;
+        float ms = 0.f;
+        int steps = 0;
+        TileTrial tr{S, kg, &ms, &steps, plain != 0};
+        st = RSV_OK;
+        for (int rep = 0; rep < 2 && st == RSV_OK; ++rep)
+          st = march_impl<R>(op, in, k, opts, nullptr, false, SCALE_NONE, &tr);
+        if (st == RSV_ERR_OOM) continue;   // does not fit next to the caller's blocks
+        if (st != RSV_OK) return st;
+        const double per = (double)ms / ((double)std::max(steps, 1) * std::min(kg, k));
+        if (per < best) {
+          best = per;
+          bs = S;
+          bg = kg;
+        }
       }
-    }
+  }
   if (bs == 0) return fail(RSV_ERR_OOM, "no tile configuration fits in device memory");
   op->tuned_k = k;
   op->tuned_tile = bs;

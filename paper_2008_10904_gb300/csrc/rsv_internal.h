@@ -243,6 +243,7 @@ namespace rsv {
 rsv_status fail(rsv_status s, const std::string& msg);
 rsv_status cuda_fail(cudaError_t e, const char* where);
 rsv_status ensure(Workspace& w, size_t bytes);
+void release(Workspace& w);
 
 // Brackets one kernel launch with profiling events when profiling is on.
 struct ProfScope {
