@@ -647,8 +647,10 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
     cudaGetLastError();
     free_b = (size_t)1 << 62;
   }
-  const size_t held = op->ws_state.bytes + op->ws_ftile.bytes + op->ws_ysnap.bytes + op->ws_acc.bytes +
-                      op->ws_coef.bytes + op->ws_coef2.bytes;
+  size_t held = 0;   // everything that need() counts: equal calls plan equally
+  for (const Workspace* w : {&op->ws_state, &op->ws_ftile, &op->ws_ysnap, &op->ws_acc, &op->ws_coef, &op->ws_coef2,
+                             &op->ws_part, &op->ws_scaled, &op->ws_stage[0], &op->ws_stage[1]})
+    held += w->bytes;
   const double budget = 0.9 * (double)(free_b + held);
   // The requested / default tile and all k vectors, shrunk (kg halved, then S down to 16) until the march
   // workspace fits in 90% of the device memory not held by others; false when the smallest does not.
@@ -698,7 +700,11 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
     const std::pair<Workspace*, size_t> want[] = {
         {&op->ws_state, rows_max * se + scratch_bytes(kg)}, {&op->ws_ftile, (size_t)f_rows(S) * rows_max * se},
         {&op->ws_ysnap, (size_t)S * rows_max * se}, {&op->ws_coef, c1}, {&op->ws_coef2, c2},
-        {&op->ws_acc, acc_in_out ? 0 : (size_t)op->n_omega * rows_max * sizeof(cpx<double>)}};
+        {&op->ws_acc, acc_in_out ? 0 : (size_t)op->n_omega * rows_max * sizeof(cpx<double>)},
+        {&op->ws_part, op->prec == RSV_PREC_FP64 ? analysis64_part_bytes(op, rows_max, np, S) : 0},
+        {&op->ws_scaled, s_in ? (size_t)op->n_omega * kg * n * coef_bytes(op) : 0},
+        {&op->ws_stage[0], host_in ? (size_t)op->n_omega * kg * n * coef_bytes(op) : 0},
+        {&op->ws_stage[1], host_in ? (size_t)op->n_omega * kg * n * coef_bytes(op) : 0}};
     bool grow = false;
     for (const auto& w : want) grow = grow || w.second > w.first->bytes;
     if (grow && need(S, kg) > 0.9 * (double)free_b)

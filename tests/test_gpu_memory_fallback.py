@@ -53,3 +53,33 @@ def test_step_form_falls_back_to_stage_times(rsv):
         filler.clear()
         torch.cuda.empty_cache()
         rsv.rsv_destroy_operator(op)
+
+
+def test_equal_host_marches_plan_equally(rsv):
+    """Host-input march of 8 vectors of 256 x 256, 64 frequencies: 3.56 GB of workspaces, 537 MB of them staging buffers.
+    With 0.9 x 4.11 GB free the first march holds all 8 vectors; so does the second one, beside the buffers of the
+    first, and gives the same bits."""
+    import torch
+    sysm = W.ADR2D(nx=256, ny=256, lx=40.0, ly=10.0, sponge_cells=8)
+    w = W.Workload("adr_host_memory", sysm, np.linspace(0.0, 40.0, 64), 0.5 * 40.0 / 257, 8, "ssrm", n_transient_windows=0,
+                   real_state=True, seed=W.SEED_BASE + 110)
+    gen = torch.Generator().manual_seed(110)
+    x = torch.randn(w.n_omega, w.k, w.n, dtype=torch.complex64, generator=gen).pin_memory()
+    x[0].imag.zero_()
+    y = torch.empty(x.shape, dtype=x.dtype, device="cuda")
+    op = rsv.create_for_workload(w, rsv.RSV_PREC_FP32)
+    filler = []
+    try:
+        torch.cuda.empty_cache()
+        free, _ = torch.cuda.mem_get_info()
+        filler.append(torch.empty(free - 4111 * 10 ** 6, dtype=torch.uint8, device="cuda"))
+        outs = []
+        for _ in range(2):
+            rsv.rsv_march_direct_host(op, x, w.k, y, **rsv.march_opts_for(w))
+            assert "group=8 " in rsv.rsv_describe(op)
+            outs.append(y.cpu())
+        assert torch.equal(outs[0], outs[1])
+    finally:
+        filler.clear()
+        torch.cuda.empty_cache()
+        rsv.rsv_destroy_operator(op)
