@@ -466,7 +466,8 @@ rsv_status rsv_profile_read(rsv_operator op, int32_t category, int64_t* groups, 
 
 /* One-line description of the operator's execution path (kernels chosen for
  * this GPU, e.g. the dense step's tensor-core variant and resident-CTA
- * capacity) and of the latest march: "tile=" steps per time tile, "group="
+ * capacity; the march kernel is the latest march's, before the first one what
+ * one vector takes) and of the latest march: "tile=" steps per time tile, "group="
  * vectors marched together, "steps=" steps marched by its last vector group
  * (smaller than the schedule when the TRM record was truncated by tail_tol).
  * Written NUL-terminated into buf (host, buflen bytes); a longer description

@@ -214,6 +214,7 @@ rsv_status on_frequencies(rsv_operator op) {
   for (TileGraph& g : op->tile_graphs)   // the captured launches carry the step h
     if (g.exec) cudaGraphExecDestroy(g.exec);
   op->tile_graphs.clear();
+  op->last_form = -1;
   if (op->kind == RSV_OP_DENSE) return dense_on_frequencies(op);
   if (op->kind == RSV_OP_GL1D && op->scheme == RSV_SCHEME_CN) return gl1d_cn_factors(op);
   return RSV_OK;

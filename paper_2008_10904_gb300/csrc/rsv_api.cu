@@ -260,11 +260,14 @@ extern "C" rsv_status rsv_describe(rsv_operator op, char* buf, int32_t buflen) {
   if (!op || !buf || buflen < 1) return fail(RSV_ERR_INVALID_ARG, "bad describe arguments");
   static const char* kinds[] = {"gl1d", "dense", "adr2d", "adv3d"};
   const char* path = "cuda-core stages";
+  // the latest march's form; before the first one on these frequencies what a march of one vector takes
+  const bool jumped = op->last_form < 0 ? jump_taken(op, 1) : op->last_form == 2;
+  const bool stepped = op->last_form < 0 ? step_form_taken(op, 1) : op->last_form == 1;
   if (op->kind == RSV_OP_GL1D) {
-    if (jump_taken(op, 1))
+    if (jumped)
       path = op->scheme == RSV_SCHEME_CN ? "cuda-core crank-nicolson jump kernels (few pairs, else tile kernel)"
                                          : "cuda-core jump kernels (few pairs, else tile kernel)";
-    else if (step_form_taken(op, 1))
+    else if (stepped)
       path = "cuda-core packed step kernel (sampled forcing: tile kernel)";
     else
       path = op->scheme == RSV_SCHEME_CN ? "cuda-core crank-nicolson tile kernel" : "cuda-core tile kernel";
@@ -273,22 +276,22 @@ extern "C" rsv_status rsv_describe(rsv_operator op, char* buf, int32_t buflen) {
     const char* e = getenv("RSV_STENCIL3D_STAGED");
     const bool pairs = !(e != nullptr && e[0] == '1') && !op->bf16_state && op->nx % 4 == 0 &&
                        op->n < ((int64_t)1 << 31);
-    path = step_form_taken(op, 1) ? (pairs ? "cuda-core 3-D half-step kernels (sampled forcing: 3-D stage-pair kernels)"
-                                           : "cuda-core 3-D half-step kernels (sampled forcing: stages)")
-           : pairs              ? "cuda-core 3-D stage-pair kernels"
-           : op->bf16_state     ? "cuda-core stages, bf16 state"
-                                : "cuda-core stages";
+    path = stepped             ? (pairs ? "cuda-core 3-D half-step kernels (sampled forcing: 3-D stage-pair kernels)"
+                                        : "cuda-core 3-D half-step kernels (sampled forcing: stages)")
+           : pairs             ? "cuda-core 3-D stage-pair kernels"
+           : op->bf16_state    ? "cuda-core stages, bf16 state"
+                               : "cuda-core stages";
   }
   if (op->kind == RSV_OP_ADR2D) {
     const char* e = getenv("RSV_STENCIL_FUSED");
     if (e != nullptr && e[0] == '1')
       path = "cuda-core whole-step kernel";
     else if (op->prec == RSV_PREC_FP64)
-      path = step_form_taken(op, 1) ? "cuda-core step-form stages" : "cuda-core stages";
+      path = stepped ? "cuda-core step-form stages" : "cuda-core stages";
     else if (adr2d_pairs_enabled() && op->nx % 4 == 0 && op->n < ((int64_t)1 << 31))
-      path = step_form_taken(op, 1) ? "cuda-core 2-D step kernel (sampled forcing: 2-D stage-pair kernels)"
-                                    : "cuda-core 2-D stage-pair kernels";
-    else if (step_form_taken(op, 1))
+      path = stepped ? "cuda-core 2-D step kernel (sampled forcing: 2-D stage-pair kernels)"
+                     : "cuda-core 2-D stage-pair kernels";
+    else if (stepped)
       path = "cuda-core 2-D step kernel (sampled forcing: stages)";
   }
   if (op->kind == RSV_OP_DENSE) {
@@ -299,10 +302,10 @@ extern "C" rsv_status rsv_describe(rsv_operator op, char* buf, int32_t buflen) {
   }
   const char* contract = (op->prec == RSV_PREC_FP32 && !op->tc_contract_disabled) ? "tcgen05" : "cuda-core";
   char packs[96] = "";
-  if (op->kind == RSV_OP_GL1D && op->p32.kg > 0 && op->p32.q > 0)
+  if (op->kind == RSV_OP_GL1D && stepped && op->p32.kg > 0 && op->p32.q > 0)
     snprintf(packs, sizeof(packs), " packed=%d ctas of %d slots (1024x%d, %d per wave)", op->p32.packs, 1024 * op->p32.q,
              op->p32.q, op->p32.wave);
-  else if (op->kind == RSV_OP_GL1D && op->pack_kg > 0)
+  else if (op->kind == RSV_OP_GL1D && !stepped && op->pack_kg > 0)
     snprintf(packs, sizeof(packs), " packed=%d ctas of %d slots (%dx%d, %d per wave)", op->pack_count,
              op->pack_threads * op->pack_ppt, op->pack_threads, op->pack_ppt, op->pack_wave);
   else if (op->kind == RSV_OP_GL1D && op->gl_cluster > 0)
@@ -688,6 +691,7 @@ static rsv_status march_impl(rsv_operator op, const void* in, int k, const rsv_m
   cudaError_t e;
   op->last_tile = S;
   op->last_group = kg;
+  op->last_form = jump ? 2 : sf ? 1 : 0;
   // the 1-D step form's groups fill whole packs
   const bool packed = sf && op->kind == RSV_OP_GL1D;
   if (packed && (st = step32_packs(op, kg)) != RSV_OK) return st;

@@ -220,6 +220,7 @@ struct rsv_operator_s {
   };
   std::vector<ProbeMemo> probe_memo;
   int last_tile = 0, last_group = 0;   // tile length and vector-group size of the latest march
+  int last_form = -1;                  // its form: 0 stage times (or sampled forcing), 1 step form, 2 jumps; -1 none yet
   // CUDA graphs of tile launch sequences (ops.cu), the private capture stream, replays so far
   std::vector<rsv::TileGraph> tile_graphs;
   cudaStream_t cap_stream = nullptr;

@@ -500,6 +500,7 @@ rsv_status series_march_impl(rsv_operator op, bool adjoint, int k, const void* i
     for (int v = 0; v < k; ++v) stops[v] = stop_all[v];
   op->last_tile = S;
   op->last_group = kg;
+  op->last_form = 0;
   return RSV_OK;
 }
 
