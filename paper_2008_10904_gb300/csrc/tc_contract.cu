@@ -412,13 +412,13 @@ __device__ __forceinline__ void store_row_tmem(float x[kKc], uint32_t ta) {
   tc::tmem_wait_st();
 }
 
-// FP32 -> FP64 with integer instructions (exact for zero and normal values).  FP64 instructions issue once
+// FP32 -> FP64 with integer instructions, for zero and normal values (exact).  FP64 instructions issue once
 // per 19 cycles and SM, conversions among them, and the accumulation needs one FP64 addition per value
 // anyway: converting there as well held the FP64 pipe 48% busy and the epilogue at twice its loads' time.
 __device__ __forceinline__ double widen(float x) {
   const uint32_t u = __float_as_uint(x), m = u & 0x7fffffffu;
-  const uint32_t hi = m < 0x00800000u ? 0u : (m >> 3) + 0x38000000u;
-  return __hiloint2double((int)(hi | (u & 0x80000000u)), m < 0x00800000u ? 0 : (int)(u << 29));
+  const uint32_t hi = m == 0u ? 0u : (m >> 3) + 0x38000000u;
+  return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
 }
 
 // FP64 accumulators of 16 output columns from column c on (8 frequencies) of row r.
@@ -432,10 +432,14 @@ __device__ __forceinline__ void load_acc16(const ContractArgs& a, int64_t r, int
 }
 // += v, the columns' sums over the tile or a segment of it.
 __device__ __forceinline__ void add_acc16(double2 old[8], const float v[16]) {
-  uint32_t top = 0;
+  uint32_t top = 0, low = 0xffffffffu;
 #pragma unroll
-  for (int q = 0; q < 16; ++q) top = max(top, __float_as_uint(v[q]) & 0x7fffffffu);
-  const bool plain = top < 0x7f800000u;   // no infinity and no NaN
+  for (int q = 0; q < 16; ++q) {
+    const uint32_t m = __float_as_uint(v[q]) & 0x7fffffffu;
+    top = max(top, m);
+    low = min(low, m - 1u);               // zero counts as the largest
+  }
+  const bool plain = top < 0x7f800000u && low >= 0x007fffffu;   // no infinity, NaN or denormal value
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     old[q].x += plain ? widen(v[2 * q]) : (double)v[2 * q];
