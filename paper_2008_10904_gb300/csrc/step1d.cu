@@ -13,7 +13,7 @@
 // they are marched from the jumps' states, all jumps side by side over the whole GPU (fill kernels).
 //
 // The band of T_p is bounded from the coefficients on the host (products of non-negative bounds of the
-// diagonals): what lies outside sums to less than 2^-62 per row.
+// diagonals): what lies outside sums to less than 2^-61 per row.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -341,25 +341,27 @@ __global__ void __launch_bounds__(kMaxPoints) fill_kernel(Band b, int p, int n_i
 // ---------------------------------------------------------------------------
 using Laurent = std::vector<double>;            // bounds of the diagonals -w .. w, centre at size / 2
 
+// Bound of the product's diagonals up to wmax (a matrix of wmax + 1 points has no others).
 Laurent conv(const Laurent& a, const Laurent& b, int wmax) {
   const int wa = (int)a.size() / 2, wb = (int)b.size() / 2, w = std::min(wa + wb, wmax);
   Laurent o(2 * (size_t)w + 1, 0.0);
   for (int i = -wa; i <= wa; ++i) {
     if (a[i + wa] == 0.0) continue;
-    for (int j = -wb; j <= wb; ++j) {
-      const int k = std::max(-w, std::min(w, i + j));   // what leaves the range counts at its end
-      o[k + w] += a[i + wa] * b[j + wb];
-    }
+    for (int j = std::max(-wb, -w - i); j <= std::min(wb, w - i); ++j) o[i + j + w] += a[i + wa] * b[j + wb];
   }
   return o;
 }
 
-// Without the ends whose sum is far below what the band may drop.
-Laurent trimmed(const Laurent& b) {
+// The bound of p steps without its outermost ends.  What is dropped of p steps' bound b reaches kMaxP steps'
+// at most (kMaxP / p) |b|^(kMaxP / p - 1) times (|b|: the sum over the diagonals, 1 or more), which stays below 2^-70.
+Laurent trimmed(const Laurent& b, int p) {
+  double norm = 0;
+  for (double x : b) norm += x;
+  const double m = (double)kMaxP / p, tol = std::ldexp(1.0, -70) / (m * std::pow(norm, m - 1.0));
   const int w = (int)b.size() / 2;
   int c = w;
   double s = 0;
-  while (c > 0 && s + b[w - c] + b[w + c] < 1e-26) {
+  while (c > 0 && s + b[w - c] + b[w + c] < tol) {
     s += b[w - c] + b[w + c];
     --c;
   }
@@ -388,14 +390,14 @@ Laurent step_bound(rsv_operator op, bool adjoint) {
     if (!(piv > 1.0001 * (a + c))) return {};
     const double disc = std::sqrt(piv * piv - 4.0 * a * c);
     const double r = 2.0 * a / (piv + disc), q = 2.0 * c / (piv + disc), K = 1.0 / disc;
-    const int w = kMaxPoints;
+    const int w = op->gl_max_n - 1;
     Laurent o(2 * (size_t)w + 1);
     for (int d = 0; d <= w; ++d) {     // row i, column i - d: entries decay with the lower couplings
       o[w - d] = 2.0 * K * std::pow(r, d);
       o[w + d] = 2.0 * K * std::pow(q, d);
     }
     o[w] += 1.0;
-    return trimmed(o);
+    return trimmed(o, 1);
   }
   const Laurent B = {op->h * lo, op->h * di, op->h * up};
   Laurent t = {1.0};
@@ -407,7 +409,8 @@ Laurent step_bound(rsv_operator op, bool adjoint) {
   return t;
 }
 
-// Smallest (wl, wr) outside which the bounds sum to less than 2^-62.
+// Smallest (wl, wr) outside which the bounds sum to less than 2^-62 (2^-61 with what `trimmed` dropped, five times
+// 2^-70 at most).
 void band_of(const Laurent& b, int* wl, int* wr) {
   const int w = (int)b.size() / 2;
   const double tol = std::ldexp(1.0, -63);
@@ -541,7 +544,7 @@ const JumpPlan& jump_plan(rsv_operator op, bool adjoint) {
       pl.wl = wl;
       pl.wr = wr;
     }
-    if (p < kMaxP) t = trimmed(conv(t, t, 4 * kMaxPoints));
+    if (p < kMaxP) t = trimmed(conv(t, t, max_n - 1), 2 * p);
   }
   if (best < 1e300 && jump_smem(max_n, std::min(cs, 8), std::min(pl.wl1 + pl.wr1 + 1, max_n), op->tri_real) <= 200 * 1024)
     pl.state = 1;
