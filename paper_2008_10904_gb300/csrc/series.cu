@@ -98,8 +98,13 @@ __device__ void derivs(const T* src, int64_t stride, int64_t n_in, int rev, int6
 // once for these stage times, and what is left per value is the polynomial and the store
 // (a thread per value, with its 64-bit divisions and up to ten sample reads: 1.13 ms for 769 stage times of
 // 131,072 rows; 0.35 ms like this, 403 MB written).  Block (x: rows, y: pieces of the
-// intervals from q0's on).
+// intervals, from the one that holds q0 to the one that holds the last stage time).
 constexpr int kPieceTimes = 16;
+
+__host__ __device__ inline int64_t pieces_of(int64_t every) { return (2 * every + kPieceTimes - 1) / kPieceTimes; }
+__host__ __device__ inline int64_t piece_at(int64_t every, int64_t q) {   // the piece that holds half step q
+  return q / (2 * every) * pieces_of(every) + q % (2 * every) / kPieceTimes;
+}
 
 template <typename T, typename R>
 __global__ void __launch_bounds__(256) series_forcing_kernel(const T* __restrict__ src, int64_t stride, int64_t n_in,
@@ -109,12 +114,10 @@ __global__ void __launch_bounds__(256) series_forcing_kernel(const T* __restrict
   if (r >= rows) return;
   const int64_t span = 2 * (int64_t)every;
   const int64_t q_end = span * (n_in - 1);
-  const int64_t pieces = (span + kPieceTimes - 1) / kPieceTimes;
-  for (int64_t y = blockIdx.y;; y += gridDim.y) {
-    const int64_t i = q0 / span + y / pieces, p0 = i * span + y % pieces * kPieceTimes;
-    if (i * span >= q0 + n_tau) break;
+  const int64_t pieces = pieces_of(every), last = piece_at(every, q0 + n_tau - 1);
+  for (int64_t y = piece_at(every, q0) + blockIdx.y; y <= last; y += gridDim.y) {
+    const int64_t i = y / pieces, p0 = i * span + y % pieces * kPieceTimes;
     const int64_t qa = max(q0, p0), qb = min(q0 + n_tau, min(p0 + kPieceTimes, (i + 1) * span));
-    if (qa >= qb) continue;
     T* f = F + (qa - q0) * rows + r;
     if (i >= n_in - 1) {
       for (int64_t q = qa; q < qb; ++q, f += rows)
@@ -436,8 +439,7 @@ rsv_status series_march_impl(rsv_operator op, bool adjoint, int k, const void* i
       if (forced) {
         ProfScope ps(op, PROF_SYNTH);
         const int n_tau = 2 * steps + 1;
-        const int64_t span = 2 * (int64_t)every, pieces = (span + kPieceTimes - 1) / kPieceTimes;
-        const int64_t ny = ((2 * n0 + n_tau - 1) / span - 2 * n0 / span + 1) * pieces;
+        const int64_t ny = piece_at(every, 2 * n0 + n_tau - 1) - piece_at(every, 2 * n0) + 1;
         const dim3 grid((unsigned)((rows + 255) / 256), (unsigned)std::min<int64_t>(ny, 65535));
         series_forcing_kernel<T, R><<<grid, 256, 0, st>>>(
             static_cast<const T*>(forcing) + (int64_t)v0 * n, out_stride, n_in, reverse_in ? 1 : 0, every, o.interp,
