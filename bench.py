@@ -207,11 +207,20 @@ def load_peaks():
     return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0, "src": "fallback"}
 
 
-# DRAM bytes (read + write) per launch group of a category's kernels over one time tile,
-# from ncu captures of the same kernels at the same rows per launch, keyed by (workload,
-# category, tile steps, rows per launch).  An entry is dropped whenever the kernel it
+# DRAM bytes (read + write) per step of a category's kernels, from ncu captures of the same
+# kernels at the same rows per launch (profiles/march_kernels.txt), keyed by (workload,
+# category, rows per launch).  An entry is dropped or measured again whenever the kernel it
 # describes changes.
-TRAFFIC = {}
+TRAFFIC = {
+    ("dense_hermite_gl_n1024_k32_w256_trm", "march", 32768):
+        {"bytes": (86.3e6 + 22.8e6) / 256, "src": "ncu dram bytes of one 256-step launch"},
+    ("gl_batch64_k8_w64_ssrm", "march", 365184):
+        {"bytes": (754.1e6 + 698.5e6) / 256, "src": "ncu dram bytes of one 256-step launch"},
+    ("adr2d_1024x512_k16_w128_ssrm", "march", 8388608):
+        {"bytes": 74.3e6 + 19.8e6, "src": "ncu dram bytes of one step"},
+    ("adv3d_256x128x128x3_k8_w64_ssrm", "march", 25165824):
+        {"bytes": 174.6e6 + 152.4e6 + 383.1e6 + 83.5e6, "src": "ncu dram bytes of the two half steps of one step"},
+}
 
 FP32_ALU_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12     # 152 SMs x 128 FP32 lanes x FMA x 2.07 GHz
 REF_TOTAL_S = 150.0                                   # CPU seconds of the reference arm's timed steps
@@ -295,9 +304,9 @@ def kernel_model(cat, w, prec, tile, groups, ms_total, rows, path):
         bound, unit, peak, per = "hbm", "GB/s", peaks["hbm_gbs"], 1e9
         src = peaks["src"] + " copy bandwidth"
     achieved = work / avg_s / per
-    traffic = TRAFFIC.get((w.name, cat, S, rows))
+    traffic = TRAFFIC.get((w.name, cat, rows)) if prec == "fp32" else None
     return {"bound": bound, "achieved": achieved, "peak": peak, "unit": unit, "frac": achieved / peak,
-            "traffic": traffic["bytes"] if traffic else None, "traffic_src": traffic["src"] if traffic else None,
+            "traffic": traffic["bytes"] * S if traffic else None, "traffic_src": traffic["src"] if traffic else None,
             "kernel": cat, "work_per_launch": work, "avg_launch_ms": avg_s * 1e3, "peak_src": src}
 
 
