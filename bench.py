@@ -227,10 +227,18 @@ REF_TOTAL_S = 150.0                                   # CPU seconds of the refer
 FP64_ALU_TFLOPS = 1.25                                # nominal FP64 rate of the part
 
 
-def kernel_model(cat, w, prec, tile, groups, ms_total, rows, path):
+def steps_per_launch(cat, w, n_t, marches, groups, group_vectors):
+    """Mean steps of a category's launch groups: those of all marches (synthesis: forced, analysis: analysed steps)
+    over the launch groups.  A tile's nominal length would count the short last tile of every march as a whole one."""
+    trm, total = w.variant == "trm", steps_per_march(w, n_t)
+    steps = {"synthesis": n_t if trm else total, "analysis": total if trm else n_t}.get(cat, total)
+    return marches * -(-w.k // group_vectors) * steps / max(groups, 1)
+
+
+def kernel_model(cat, w, prec, S, groups, ms_total, rows, path):
     """Roofline record of one kernel category: algorithmic work per launch / average launch time.
 
-    Units of work per launch (one time tile of S steps):
+    Units of work per launch (one time tile of S steps on average):
       synthesis  rows x n_omega x n_tau complex (8 flop) or real-output (4 flop) multiply-adds
       analysis   rows x n_omega x S multiply-adds (8 flop complex state, 4 flop real state)
       march      dense: 8 n^2 k flop per step (one dense complex product, tensor cores);
@@ -252,7 +260,6 @@ def kernel_model(cat, w, prec, tile, groups, ms_total, rows, path):
     """
     peaks = load_peaks()
     avg_s = ms_total / max(groups, 1) / 1e3
-    S = tile
     dense = "kind=dense" in path
     step_form = any(t in path for t in ("jump kernels", "step kernel", "half-step", "step-form")) and "whole-step" not in path
     se = (8 if prec == "fp64" else 4) * (1 if w.real_state else 2)
@@ -590,7 +597,7 @@ def run_ours(args):
     if args.tile == 0 and not args.no_autotune:
         t_s, t_g = rsv.rsv_autotune(op, bufs[0], w.k, **opts)
         tuned = {"tile": t_s, "group": t_g, "chosen_by": "rsv_autotune: one timed tile per candidate "
-                 "(default tile and half of it x groups of k, k/2, k/4, 1 that fit), least time per vector-step"}
+                 "(the tile of an untuned march and half of it x groups of k, k/2, k/4, 1 that fit), least time per vector-step"}
     for _ in range(args.warmup):
         step()
     torch.cuda.synchronize()
@@ -657,9 +664,10 @@ def run_ours(args):
 
     dom = max(prof, key=lambda c: prof[c][2])
     desc = dict(kv.split("=", 1) for kv in path.split() if "=" in kv)
-    tile = int(desc.get("tile", args.tile or 256))
-    rows = int(desc.get("group", w.k)) * w.n
-    roof = kernel_model(dom, w, prec_name, tile, prof[dom][0], prof[dom][2], rows, path)
+    group = int(desc.get("group", w.k))
+    marches = args.steps * (marches_per_rsvd(w) if step_kind == "rsvd" else 1)
+    mean_steps = steps_per_launch(dom, w, n_t, marches, prof[dom][0], group)
+    roof = kernel_model(dom, w, prec_name, mean_steps, prof[dom][0], prof[dom][2], group * w.n, path)
     launches = sum(v[1] for v in prof.values())
     acc = None if args.skip_accuracy else accuracy_record(w, prec_name, dense, stream, rank)
     comp = None if args.no_comparator else fp64_single_vector(w, dense, stream, n_t, rank)
