@@ -2,7 +2,7 @@
 where its kernels can go wrong, against the oracle.
 
 The 2-D FP32 kernel walks strips of 120 cells in x and runs of rows in y, with rows padded to four
-cells; the 3-D FP32 kernels tile 64 x 8 columns of padded rows; the FP64 stages take any grid.  The
+cells; the 3-D FP32 kernels tile 64 x 12 columns of padded rows; the FP64 stages take any grid.  The
 grids below sit on and beside those edges.  Tolerances are those of the march parity tests (FP32
 rounding of about 6e-8 per operation through gains of up to about 30: 2e-5; FP64 1e-10).
 """
@@ -60,11 +60,25 @@ def test_2d_stages_fp64(rsv, nx, ny, sponge, adjoint):
 @pytest.mark.parametrize("nx,ny,nz,k", [(3, 3, 3, 1), (61, 7, 5, 2), (63, 8, 4, 1), (65, 9, 9, 2), (67, 17, 6, 1)])
 @pytest.mark.parametrize("adjoint", [False, True])
 def test_3d_tile_edges_fp32(rsv, nx, ny, nz, k, adjoint):
-    """Widths that are not multiples of four, tiles one cell short of, on and past the 64 x 8 tile."""
+    """Widths that are not multiples of four, one cell short of, on and past the 64-cell tile; a single tile in y, ragged
+    or (17) a second one."""
     sysm = W.ADV3D(nx=nx, ny=ny, nz=nz, lx=20.0, ly=10.0, lz=10.0, visc=0.02)
     w = W.Workload("adv_edges", sysm, np.array([0.2 * np.pi * j for j in range(5)]), min(0.3, 0.5 * 20.0 / (nx + 1)), k,
                    "trm" if nx % 4 == 1 else "ssrm", n_transient_windows=1, tail_steps=19, real_state=True,
                    seed=W.SEED_BASE + 82)
+    _check(rsv, w, operators.adv3d(w.system), 1, adjoint, tile_steps=14)
+
+
+@pytest.mark.parametrize("nx,ny,nz,k", [(63, 11, 4, 1), (64, 12, 5, 2), (65, 13, 4, 1), (33, 24, 6, 1), (5, 25, 4, 2),
+                                        (132, 26, 5, 1), (133, 27, 9, 1)])
+@pytest.mark.parametrize("adjoint", [False, True])
+def test_3d_tile_rows_and_inner_tiles_fp32(rsv, nx, ny, nz, k, adjoint):
+    """One row short of, on and past one and two tiles of 12 rows; the last two grids have a tile with no cell beside a
+    wall (x from 64, y from 12: the unmasked path) and its masked neighbours."""
+    sysm = W.ADV3D(nx=nx, ny=ny, nz=nz, lx=20.0, ly=10.0, lz=10.0, visc=0.02)
+    w = W.Workload("adv_rows", sysm, np.array([0.2 * np.pi * j for j in range(5)]), min(0.3, 0.5 * 20.0 / (nx + 1)), k,
+                   "trm" if nx % 2 else "ssrm", n_transient_windows=1, tail_steps=19, real_state=True,
+                   seed=W.SEED_BASE + 116)
     _check(rsv, w, operators.adv3d(w.system), 1, adjoint, tile_steps=14)
 
 
