@@ -16,7 +16,7 @@
 //
 // Rows of the state, forcing and snapshot tiles and of the transformed coefficients are padded to a
 // multiple of four cells (zeros), so that every grid takes the 16-byte loads and the pipelined
-// contractions; `march_finish` drops the padding.
+// contractions; `launch_finish` drops the padding.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>

@@ -832,7 +832,7 @@ EncodeTiled encode_tiled() {
 
 // Tensor map of the long operand for the pipelined kernel: FP32 values, rows fastest, boxes of one K chunk
 // by 128 rows.  False where the operand does not fit one: its base and its row stride in memory must be
-// multiples of 16 bytes and a row of it shorter than 2^32 values.
+// multiples of 16 bytes and a row of it shorter than 2^31 values.
 bool pipe_enabled(rsv_operator op) {
   static const int env = [] {
     const char* e = getenv("RSV_CONTRACT_PIPE");
