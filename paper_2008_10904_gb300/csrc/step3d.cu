@@ -19,9 +19,13 @@
 // analysed steps; half 2: w2, u and g read, u' written) against eleven for the stage pairs with
 // accumulator and forcing (stencil_kernels.cu).  Cells outside the grid hold zero (homogeneous Dirichlet).
 //
-// Rounding: stage factors come from FP64 and the last stage adds one rounded increment to u, as a stage-time march
-// does.  With factors multiplied up in FP32 and every term of every stage added to u, 97 x 61 x 43 over four windows
-// was 4.6e-6 off (the stage-time kernels 4.1e-6), 2.1e-6 like this, and the kernels take the same time.
+// Rounding.  What is systematic in it acts like a change of the operator and adds up over a march, so the stage factors
+// are formed in FP64 and rounded once, the diagonal is exactly minus the sum of the diffusion factors, advection is a
+// difference of its own (added to the diffusion, it was rounded at its own size, and rows of the operator kept a rest
+// of 1e-8 per step), and the last stage adds one rounded increment to u, as a stage-time march does.  Error against
+// FP64, contractions on the CUDA cores: 128 x 64 x 64 over four windows of 643 steps 2e-7 (3e-7 by the stage-time
+// kernels, 6e-7 with merged factors), leading gains of 256 x 128 x 128 2.5e-6 (2.5e-6, 5.4e-6).  It costs 1.6% of
+// the march, two additions per value and stage.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
@@ -45,7 +49,8 @@ constexpr size_t half_smem(bool second) {
 static_assert(half_smem(true) <= 232448 && half_smem(false) <= 232448, "3-D rings exceed the shared memory of a CTA");
 
 // Factors of one stage, formed in FP64 from f = h / m and rounded once: a relative error of them acts like one of
-// the operator itself, and adds up over a march.
+// the operator itself, and adds up over a march.  d is exactly minus twice the sum of x, y and z: what is missing
+// there acts as damping or growth, all the longer the slower the flow.
 struct Stage3D {
   float f, x, y, z, c, d;     // f; f visc / dx^2, ... / dy^2, ... / dz^2; f / (2 dx); -2 (x + y + z)
 };
@@ -94,29 +99,28 @@ template <bool ADJ, bool INC>
 __device__ __forceinline__ void stage3d(const Stage3D& S, const C3& xb, const C3& xc, const C3& xt,
                                         const float4 so[3], const float4 no[3], const float l[3], const float r[3],
                                         const Flow& w, const C3& u0, C3& o) {
-  const float f = S.f, fz = S.z, fy = S.y, fx = S.x, fc = S.c, cc = S.d;
-  float cw[4], ce[4];
+  const float f = S.f;
+  float au[4];   // advection, apart from the diffusion: added up, the two would be rounded at the size of the larger
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {
-    if (ADJ) {
-      cw[c] = fmaf(-fc, c == 0 ? w.Ul : w.U.v[c - 1], fx);
-      ce[c] = fmaf(fc, c == 3 ? w.Ur : w.U.v[c + 1], fx);
-    } else {
-      cw[c] = fmaf(fc, w.U.v[c], fx);
-      ce[c] = fmaf(-fc, w.U.v[c], fx);
-    }
-  }
+  for (int k = 0; k < 4; ++k) au[k] = S.c * w.U.v[k];
+  const float al = S.c * w.Ul, ar = S.c * w.Ur;   // transposed only
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const V4 s = v4(so[c]), n = v4(no[c]);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
+      const float we = k == 0 ? l[c] : xc.c[c].v[k - 1], ea = k == 3 ? r[c] : xc.c[c].v[k + 1];
       const float zz = xb.c[c].v[k] + xt.c[c].v[k];
-      float a = INC ? fz * zz : fmaf(fz, zz, u0.c[c].v[k]);
-      a = fmaf(fy, s.v[k] + n.v[k], a);
-      a = fmaf(cw[k], k == 0 ? l[c] : xc.c[c].v[k - 1], a);
-      a = fmaf(ce[k], k == 3 ? r[c] : xc.c[c].v[k + 1], a);
-      o.c[c].v[k] = fmaf(cc, xc.c[c].v[k], a);
+      float a = INC ? S.z * zz : fmaf(S.z, zz, u0.c[c].v[k]);
+      a = fmaf(S.y, s.v[k] + n.v[k], a);
+      a = fmaf(S.x, we + ea, a);
+      a = fmaf(S.d, xc.c[c].v[k], a);
+      if (ADJ) {
+        a = fmaf(-(k == 0 ? al : au[k - 1]), we, a);
+        o.c[c].v[k] = fmaf(k == 3 ? ar : au[k + 1], ea, a);
+      } else {
+        o.c[c].v[k] = fmaf(au[k], we - ea, a);
+      }
     }
   }
 #pragma unroll
@@ -396,8 +400,12 @@ cudaError_t step_march_3d(rsv_operator op, const MarchTile& t, void* state, cons
   P.vstride = (int64_t)3 * P.nxp * P.ny * P.nz;
   auto factors = [&](double f) {
     const double x = f * op->visc / (op->c_dx * op->c_dx), y = f * op->visc / (op->c_dy * op->c_dy),
-                 z = f * op->visc / (op->c_dz * op->c_dz);
-    return Stage3D{(float)f, (float)x, (float)y, (float)z, (float)(0.5 * f / op->c_dx), (float)(-2.0 * (x + y + z))};
+                 z = f * op->visc / (op->c_dz * op->c_dz), sum = x + y + z;
+    // the diffusion factors on the FP32 grid of their sum (at most 2e-7 off for like spacings), so that it is exact
+    const double unit = sum > 0.0 ? std::ldexp(1.0, std::ilogb(sum) - 23) : 1.0;
+    auto on_grid = [&](double v) { return (float)(unit * std::nearbyint(v / unit)); };
+    const float fx = on_grid(x), fy = on_grid(y), fz = on_grid(z);
+    return Stage3D{(float)f, fx, fy, fz, (float)(0.5 * f / op->c_dx), -2.f * (fx + fy + fz)};
   };
   const Stage3D st[4] = {factors(op->h / 4), factors(op->h / 3), factors(op->h / 2), factors(op->h)};
   P.U = (const float*)op->fldp[0];
