@@ -219,7 +219,7 @@ TRAFFIC = {
     ("adr2d_1024x512_k16_w128_ssrm", "march", 8388608):
         {"bytes": 74.3e6 + 19.8e6, "src": "ncu dram bytes of one step"},
     ("adv3d_256x128x128x3_k8_w64_ssrm", "march", 25165824):
-        {"bytes": 174.6e6 + 152.4e6 + 383.1e6 + 83.5e6, "src": "ncu dram bytes of the two half steps of one step"},
+        {"bytes": 174.7e6 + 152.8e6 + 383.3e6 + 83.7e6, "src": "ncu dram bytes of the two half steps of one step"},
 }
 
 FP32_ALU_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12     # 152 SMs x 128 FP32 lanes x FMA x 2.07 GHz
