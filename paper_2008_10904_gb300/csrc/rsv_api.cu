@@ -399,6 +399,7 @@ extern "C" rsv_status rsv_set_frequencies(rsv_operator op, const double* omega, 
     }
     tab[q] = mk<double>(re, im);
   }
+  op->have_freq = false;   // until the new tables are there: a call after a failure below gets RSV_ERR_STATE
   if (op->d_tw) cudaFree(op->d_tw);
   if (op->d_pj) cudaFree(op->d_pj);
   if (op->d_cw) cudaFree(op->d_cw);
@@ -421,7 +422,10 @@ extern "C" rsv_status rsv_set_frequencies(rsv_operator op, const double* omega, 
   if (e == cudaSuccess) e = cudaMemcpy(op->d_pj, pj.data(), n_omega * sizeof(int64_t), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc(&op->d_cw, n_omega * sizeof(float));
   if (e == cudaSuccess) e = cudaMemcpy(op->d_cw, cw.data(), n_omega * sizeof(float), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) return cuda_fail(e, "twiddle table");
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return cuda_fail(e, "twiddle table");
+  }
   op->omega.assign(omega, omega + n_omega);
   op->pj = pj;
   op->n_omega = n_omega;
